@@ -297,9 +297,9 @@ cudaError_t launch_backward_rescue_n(const SceneDev& S, const BatchDev& B, const
                                             const uint8_t* status, const float* dX, const float* dL, double* gacc,
                                             cudaStream_t stream, int n_sm, const uint32_t* rescue_list,
                                             const unsigned* rescue_count) {
-  const uint64_t rwant = (n_local / 16 + kThreads - 1) / kThreads;
-  const unsigned rgrid = (unsigned)(rwant < (uint64_t)n_sm * 4 ? (rwant ? rwant : 1) : (uint64_t)n_sm * 4);
-  backward_rescue_kernel<N><<<rgrid, kThreads, 0, stream>>>(S, B, cfg, list, T, status, dX, dL, gacc, rescue_list,
+  const unsigned rgrid = rescue_grid(n_local, n_sm);
+  if (rgrid == 0) return cudaSuccess;
+  backward_rescue_kernel<N><<<rgrid, kRescueThreads, 0, stream>>>(S, B, cfg, list, T, status, dX, dL, gacc, rescue_list,
                                                              rescue_count);
   count_launch();
   return cudaGetLastError();

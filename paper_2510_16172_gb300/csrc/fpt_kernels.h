@@ -15,6 +15,18 @@ constexpr int kThreads = 128;  // threads per CTA for all path kernels
 // at the register-resident orders.
 template <int N>
 constexpr int kLongOrderMinBlocks = N > kMaxBfgsOrder ? 1 : 0;
+// Threads per CTA of the FP64 passes over listed paths (polish64_kernel over its rescue list,
+// backward_rescue_kernel): one warp.  The GPU has few FP64 lanes per SM, so a pass is bound by the FP64 pipe of
+// the SMs it sits on, and a short list takes as long as the SM with the most listed warps: one-warp CTAs
+// deal the list's warps out over all SMs, where CTAs of kThreads put four on one SM and left most without any.
+constexpr int kRescueThreads = 32;
+constexpr int kRescueCtasPerSm = 8;  // 255 registers a thread: eight one-warp CTAs are resident per SM
+// Grid of such a pass over a slice of n_local paths: room for one path in sixteen (a longer list is strided over).
+inline unsigned rescue_grid(uint64_t n_local, int n_sm) {
+  const uint64_t want = (n_local + 16 * kRescueThreads - 1) / (16 * kRescueThreads);
+  const uint64_t cap = (uint64_t)n_sm * kRescueCtasPerSm;
+  return (unsigned)(want < cap ? want : cap);
+}
 constexpr size_t kMaxSmemBytes = 200 * 1024;  // dynamic shared memory a path kernel may request
 
 // Kernels launched by the calling thread; the API's profiler reads the

@@ -775,11 +775,12 @@ cudaError_t launch_polish_n(const SceneDev& S, const BatchDev& B, const PolishCf
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  // FP64 pass over the listed paths (its grid covers a few percent of the paths)
-  e = grid_of((const void*)polish64_kernel<N>, s64, (n_local + 15) / 16, grid);
-  if (e != cudaSuccess || grid == 0) return e;
-  polish64_kernel<N><<<grid, kThreads, s64, stream>>>(S, B, cfg, n_local, list, T, X, L, status, rho, mask, bdist,
-                                                       s64 != 0, rescue_list, rescue_count);
+  // FP64 pass over the listed paths, in CTAs of one warp (kRescueThreads) that read the records where they
+  // stand: a listed path needs a few of them, so staging the scene's tables would cost more than it saves
+  const unsigned rgrid = rescue_grid(n_local, n_sm);
+  if (rgrid == 0) return cudaSuccess;
+  polish64_kernel<N><<<rgrid, kRescueThreads, 0, stream>>>(S, B, cfg, n_local, list, T, X, L, status, rho, mask, bdist,
+                                                            0, rescue_list, rescue_count);
   count_launch();
   e = cudaGetLastError();
   if (e != cudaSuccess || !grad) return e;
