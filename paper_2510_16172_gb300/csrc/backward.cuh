@@ -315,14 +315,12 @@ cudaError_t launch_backward_n(const SceneDev& S, const BatchDev& B, const Backwa
     cfg.sel = nullptr;  // point cotangents: every path takes part
     cfg.sel_count = nullptr;
   } else {
-    cudaError_t e = cudaMemsetAsync(cfg.sel_count, 0, sizeof(unsigned), stream);
-    if (e != cudaSuccess) return e;
     const uint64_t want = (n_local + kSelChunk - 1) / kSelChunk;
     const unsigned g = (unsigned)(want < (uint64_t)n_sm * 8 ? want : (uint64_t)n_sm * 8);
     if (g == 0) return cudaSuccess;
     backward_select_kernel<N><<<g, kSelThreads, 0, stream>>>(B, cfg, n_local, list, status, dL);
     count_launch();
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   const size_t base = (size_t)S.n_obj * (kRec32 + kAux) * sizeof(float);
@@ -337,16 +335,9 @@ cudaError_t launch_backward_n(const SceneDev& S, const BatchDev& B, const Backwa
     cudaError_t e = cudaFuncSetAttribute(backward_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, backward_kernel<N>, kThreads, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
-  uint64_t want = (n_local + kThreads - 1) / kThreads;
-  uint64_t cap = (uint64_t)n_sm * (uint64_t)per_sm;
-  unsigned grid = (unsigned)(want < cap ? want : cap);
-  if (grid == 0) return cudaSuccess;
-  e = cudaMemsetAsync(rescue_count, 0, sizeof(unsigned), stream);
-  if (e != cudaSuccess) return e;
+  unsigned grid = 0;
+  cudaError_t e = strided_grid(backward_kernel<N>, kThreads, smem, n_local, n_sm, grid);
+  if (e != cudaSuccess || grid == 0) return e;
   backward_kernel<N><<<grid, kThreads, smem, stream>>>(S, B, cfg, n_local, list, T, status, dX, dL, gacc, rescue_list,
                                                         rescue_count);
   count_launch();

@@ -615,7 +615,7 @@ struct BfgsLaunch {
   uint8_t* iters;
   cudaStream_t stream;
   int n_sm;
-  unsigned long long* work;  // chunk counter of the refill kernel
+  unsigned long long* work;  // chunk counter of the refill kernel (zero at the launch)
 };
 
 template <int N, unsigned Q, int kSrc>
@@ -642,18 +642,11 @@ cudaError_t launch_bfgs_nq(const BfgsLaunch& a) {
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
-  const uint64_t want = (a.n_local + kThreads - 1) / kThreads;
-  const uint64_t cap = (uint64_t)a.n_sm * (uint64_t)per_sm;
-  const unsigned grid = (unsigned)(want < cap ? want : cap);
-  if (grid == 0) return cudaSuccess;
+  unsigned grid = 0;
+  cudaError_t e = strided_grid(fn, kThreads, smem, a.n_local, a.n_sm, grid);
+  if (e != cudaSuccess || grid == 0) return e;
   if (refill) {
     if (a.work == nullptr) return cudaErrorInvalidValue;
-    e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long), a.stream);
-    if (e != cudaSuccess) return e;
     // at least ~8 chunks per warp, in whole warps of paths
     SolveCfg cfg = a.cfg;
     BatchDev B = a.B;

@@ -10,6 +10,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <utility>
 #include <vector>
@@ -37,16 +38,21 @@ struct fpt_ctx {
   float* d_tape = nullptr;                 // per-step state of fpt_backward_unrolled
   size_t tape_cap = 0;                     // floats
   unsigned long long* d_count = nullptr;   // counters for reductions
-  unsigned long long* d_work = nullptr;    // work counters of the lane-refill solver (one per concurrent launch)
+  unsigned char* d_ctl = nullptr;          // launch counters of the orders (OrderCtl), cleared once per call
   static constexpr int kSide = FPT_SIDE_STREAMS;  // streams for the independent pattern launches of one order
   cudaStream_t side[kSide] = {};
   cudaEvent_t fork_ev = nullptr;
   cudaEvent_t join_ev[kSide] = {};
+  // orders of one call that run side by side: the first on `stream`, the others dealt over these
+  static constexpr int kOrderStreams = 4;
+  cudaStream_t ostream[kOrderStreams] = {};
+  cudaEvent_t ofork_ev = nullptr;
+  cudaEvent_t ojoin_ev[kOrderStreams] = {};
   uint32_t* d_rescue = nullptr;            // path lists: FP64 polish, FP64 adjoint, second polish pass
   float* d_step = nullptr;                 // first Newton steps of the second polish pass's paths
-  size_t rescue_cap = 0;
+  size_t rescue_cap = 0;                   // entries of each of d_rescue's three lists
   size_t step_cap = 0;                     // floats of d_step
-  unsigned* d_rescue_n = nullptr;          // counters: FP64 polish, FP64 adjoint, selected paths, dropped paths
+  unsigned* d_dropped = nullptr;           // paths the last backward left out (fpt_backward_dropped)
   fpt_mlp* init_mlp = nullptr;             // network for init_mode = 1
   int acc_flush_tiles = 64;                // backward sums: CTA tiles between flushes of the FP32 partial sums
   int acc_smem = 1;                        // backward sums: 1 = FP32 partial sums per CTA, 0 = straight to FP64
@@ -58,6 +64,16 @@ struct fpt_ctx {
   double prof_ms[FPT_K_COUNT] = {0, 0, 0, 0, 0};
   uint64_t prof_kernels[FPT_K_COUNT] = {0, 0, 0, 0, 0};
 };
+
+// Launch counters of one order, in context memory; a call clears the counters of all orders with one memset
+// before its first launch.
+struct OrderCtl {
+  unsigned long long work[40];  // path counters of the lane-refill solver: one per pattern, 32: the small buckets
+  unsigned polish64, adjoint64, stepped;  // entries of the polish's lists: FP64 polish, FP64 adjoint, second pass
+  unsigned backward64, selected;          // entries of the backward's lists: FP64 adjoint, paths with a cotangent
+  unsigned pad[3];
+};
+constexpr size_t kCtlBytes = (kMaxOrder + 1) * sizeof(OrderCtl);
 
 // Event pair around the launches of one call when timing is on; counts the kernels launched in between.
 struct ProfScope {
@@ -243,14 +259,19 @@ fpt_status fpt_create(fpt_ctx** out, int device, void* cuda_stream) {
   if (e == cudaSuccess) e = cudaMemset(ctx->d_err, 0, sizeof(int));
   static_assert(kPatternKeys <= 128, "pattern counters");
   if (e == cudaSuccess) e = cudaMalloc(&ctx->d_count, 128 * sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaMalloc(&ctx->d_work, 64 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMalloc(&ctx->d_ctl, kCtlBytes);
   for (int k = 0; k < fpt_ctx::kSide && e == cudaSuccess; ++k) {
     e = cudaStreamCreateWithFlags(&ctx->side[k], cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->join_ev[k], cudaEventDisableTiming);
   }
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaMalloc(&ctx->d_rescue_n, 4 * sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaMemset(ctx->d_rescue_n, 0, 4 * sizeof(unsigned));
+  for (int k = 0; k < fpt_ctx::kOrderStreams && e == cudaSuccess; ++k) {
+    e = cudaStreamCreateWithFlags(&ctx->ostream[k], cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ojoin_ev[k], cudaEventDisableTiming);
+  }
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ofork_ev, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaMalloc(&ctx->d_dropped, sizeof(unsigned));
+  if (e == cudaSuccess) e = cudaMemset(ctx->d_dropped, 0, sizeof(unsigned));
   // the fixed array of fpt_backward_noalloc: its address on this device, looked up again for every context
   if (e == cudaSuccess) e = noalloc_lookup(device);
   if (e != cudaSuccess) {
@@ -272,15 +293,20 @@ void fpt_destroy(fpt_ctx* ctx) {
   cudaFree(ctx->d_err);
   cudaFree(ctx->d_gacc);
   cudaFree(ctx->d_count);
-  cudaFree(ctx->d_work);
+  cudaFree(ctx->d_ctl);
   for (int k = 0; k < fpt_ctx::kSide; ++k) {
     if (ctx->side[k]) cudaStreamDestroy(ctx->side[k]);
     if (ctx->join_ev[k]) cudaEventDestroy(ctx->join_ev[k]);
   }
   if (ctx->fork_ev) cudaEventDestroy(ctx->fork_ev);
+  for (int k = 0; k < fpt_ctx::kOrderStreams; ++k) {
+    if (ctx->ostream[k]) cudaStreamDestroy(ctx->ostream[k]);
+    if (ctx->ojoin_ev[k]) cudaEventDestroy(ctx->ojoin_ev[k]);
+  }
+  if (ctx->ofork_ev) cudaEventDestroy(ctx->ofork_ev);
   cudaFree(ctx->d_rescue);
   cudaFree(ctx->d_step);
-  cudaFree(ctx->d_rescue_n);
+  cudaFree(ctx->d_dropped);
   cudaFree(ctx->d_tape);
   delete ctx;
 }
@@ -820,27 +846,6 @@ static fpt_status ensure_buckets(fpt_ctx* ctx, fpt_batch* b, const SceneDev& S) 
   return FPT_OK;
 }
 
-// Polish scratch for an order slice of n paths of order `order`: three uint32
-// lists of n entries and the first Newton steps (2 order floats per path).
-static fpt_status ensure_rescue(fpt_ctx* ctx, uint64_t n, int order) {
-  if (n > ctx->rescue_cap) {
-    cudaFree(ctx->d_rescue);
-    ctx->d_rescue = nullptr;
-    ctx->rescue_cap = 0;
-    CUDA_OR_FAIL(ctx, cudaMalloc(&ctx->d_rescue, 3 * n * sizeof(uint32_t)));
-    ctx->rescue_cap = n;
-  }
-  const size_t step = (size_t)2 * order * n;
-  if (step > ctx->step_cap) {
-    cudaFree(ctx->d_step);
-    ctx->d_step = nullptr;
-    ctx->step_cap = 0;
-    CUDA_OR_FAIL(ctx, cudaMalloc(&ctx->d_step, step * sizeof(float)));
-    ctx->step_cap = step;
-  }
-  return FPT_OK;
-}
-
 // Paths of order n in a batch: count and list (nullptr for exhaustive batches).
 static uint64_t order_slice(const fpt_batch* b, int n, const PathRec** list) {
   if (b->dev.mode == BATCH_EXHAUSTIVE) {
@@ -857,6 +862,120 @@ static uint64_t order_slice(const fpt_batch* b, int n, const PathRec** list) {
   }
   *list = b->d_lists + first;
   return c;
+}
+
+// Path scratch for `entries` paths (three uint32 lists of them) and `step` floats of first Newton steps.
+static cudaError_t ensure_rescue(fpt_ctx* ctx, uint64_t entries, size_t step) {
+  cudaError_t e = cudaSuccess;
+  if (entries > ctx->rescue_cap) {
+    cudaFree(ctx->d_rescue);
+    ctx->d_rescue = nullptr;
+    ctx->rescue_cap = 0;
+    e = cudaMalloc(&ctx->d_rescue, 3 * entries * sizeof(uint32_t));
+    if (e != cudaSuccess) return e;
+    ctx->rescue_cap = entries;
+  }
+  if (step > ctx->step_cap) {
+    cudaFree(ctx->d_step);
+    ctx->d_step = nullptr;
+    ctx->step_cap = 0;
+    e = cudaMalloc(&ctx->d_step, step * sizeof(float));
+    if (e != cudaSuccess) return e;
+    ctx->step_cap = step;
+  }
+  return cudaSuccess;
+}
+
+// One order's share of a call: its paths, the stream its kernels go to and its scratch.
+struct OrderRun {
+  int n;
+  uint64_t cnt;
+  const PathRec* list;
+  cudaStream_t stream;
+  uint32_t* lists;  // three lists of cnt entries
+  float* step;      // 2 n cnt floats (nullptr when the call asked for none)
+  OrderCtl* ctl;
+};
+
+// Largest batch whose orders run side by side.  The kernels of one order form a chain (BFGS, two polish passes,
+// FP64 polish, select, adjoint, FP64 adjoint) whose later links, and every link of a small batch, leave
+// most of the GPU idle; the orders touch different paths, so their chains can overlap.  Measured, one order
+// after the other against side by side: 200,000 tiny-scene paths of orders 1-4 353 -> 174 us, 541,000 canyon
+// paths of orders 1-3 651 -> 456 us, city batches of orders 1-5 with 8 M paths 5.70 -> 5.21 ms, 24 M 15.6 -> 14.8 ms,
+// 48 M 29.0 -> 27.9 ms.  The gain shrinks as single kernels fill the GPU, while overlapped orders need
+// their scratch side by side (12 + 8 n bytes per path of order n instead of the largest order's alone): the
+// line keeps that to a few GB.
+constexpr uint64_t kOverlapMaxPaths = 1ull << 27;
+
+// The orders of a call.  With overlap, the longest sequences come first (the longest chain) on the context's
+// stream and the others on the order streams, each with its own scratch; else all on the context's stream
+// in ascending order, sharing one scratch.  run(orders, body) forks, calls body for each order and joins.
+struct OrderPlan {
+  OrderRun runs[kMaxOrder];
+  int count = 0;
+  bool overlap = false;
+};
+
+static fpt_status plan_orders(fpt_ctx* ctx, const fpt_batch* b, bool scratch, bool steps, OrderPlan& plan) {
+  uint64_t sum = 0, most = 0;
+  size_t step_sum = 0, step_most = 0;
+  for (int n = 1; n <= kMaxOrder; ++n) {
+    const PathRec* list;
+    const uint64_t cnt = order_slice(b, n, &list);
+    if (!cnt) continue;
+    if (cnt > 0xFFFFFFFFull) return fail(ctx, FPT_EUNSUPPORTED, "more than 2^32 paths of one order");
+    OrderRun& r = plan.runs[plan.count++];
+    r = OrderRun{n, cnt, list, ctx->stream, nullptr, nullptr, reinterpret_cast<OrderCtl*>(ctx->d_ctl) + n};
+    sum += cnt;
+    most = cnt > most ? cnt : most;
+    const size_t st = steps ? (size_t)2 * n * cnt : 0;
+    step_sum += st;
+    step_most = st > step_most ? st : step_most;
+  }
+  // kernel timing brackets the launches of one class on the context's stream: one order after the other
+  plan.overlap = plan.count > 1 && sum <= kOverlapMaxPaths && !ctx->prof;
+  if (scratch && plan.count) {
+    if (plan.overlap && ensure_rescue(ctx, sum, step_sum) != cudaSuccess) {
+      cudaGetLastError();  // no room side by side: one order after the other, as for large batches
+      plan.overlap = false;
+    }
+    if (!plan.overlap) CUDA_OR_FAIL(ctx, ensure_rescue(ctx, most, step_most));
+  }
+  if (plan.overlap)
+    for (int i = 0, j = plan.count - 1; i < j; ++i, --j) std::swap(plan.runs[i], plan.runs[j]);
+  uint64_t at = 0;
+  size_t step_at = 0;
+  for (int i = 0; i < plan.count; ++i) {
+    OrderRun& r = plan.runs[i];
+    if (scratch) {
+      r.lists = ctx->d_rescue + 3 * at;
+      r.step = steps ? ctx->d_step + step_at : nullptr;
+    }
+    if (plan.overlap) {
+      if (i > 0) r.stream = ctx->ostream[(i - 1) % fpt_ctx::kOrderStreams];
+      at += r.cnt;
+      step_at += steps ? (size_t)2 * r.n * r.cnt : 0;
+    }
+  }
+  return FPT_OK;
+}
+
+static fpt_status run_orders(fpt_ctx* ctx, const OrderPlan& plan,
+                             const std::function<fpt_status(const OrderRun&)>& body) {
+  const int used = !plan.overlap ? 0 : (plan.count - 1 < fpt_ctx::kOrderStreams ? plan.count - 1 : fpt_ctx::kOrderStreams);
+  if (used) {
+    CUDA_OR_FAIL(ctx, cudaEventRecord(ctx->ofork_ev, ctx->stream));
+    for (int k = 0; k < used; ++k) CUDA_OR_FAIL(ctx, cudaStreamWaitEvent(ctx->ostream[k], ctx->ofork_ev, 0));
+  }
+  fpt_status st = FPT_OK;
+  for (int i = 0; i < plan.count && st == FPT_OK; ++i) st = body(plan.runs[i]);
+  // joined also after an error: later calls reuse the scratch, and a stream capture must end joined
+  for (int k = 0; k < used; ++k) {
+    const cudaError_t e = cudaEventRecord(ctx->ojoin_ev[k], ctx->ostream[k]);
+    const cudaError_t w = e == cudaSuccess ? cudaStreamWaitEvent(ctx->stream, ctx->ojoin_ev[k], 0) : e;
+    if (st == FPT_OK) CUDA_OR_FAIL(ctx, w);
+  }
+  return st;
 }
 
 // Paths of order n and interaction-type pattern q: count and list (nullptr for exhaustive batches).
@@ -882,10 +1001,88 @@ static fpt_status check_scene_batch(fpt_ctx* ctx, const fpt_scene* s, const fpt_
   return FPT_OK;
 }
 
-// Solve (and, with grad, the fused backward) of every order of the batch.
+// The implicit backward of one order's paths (fpt_backward, and fpt_solve_grad after its solve).
+static fpt_status backward_order(fpt_ctx* ctx, const SceneDev& S, const fpt_batch* b, const OrderRun& r,
+                                 const BackwardCfg& cfg, const float* T, const uint8_t* status, const float* dX,
+                                 const float* dL) {
+  ProfScope ps(ctx, FPT_K_BACKWARD);
+  BackwardCfg cfg_n = cfg;
+  cfg_n.sel = r.lists + 2 * r.cnt;  // the third list of the scratch (the polish's, free here)
+  cfg_n.sel_count = &r.ctl->selected;
+  CUDA_OR_FAIL(ctx, launch_backward(r.n, S, b->dev, cfg_n, r.cnt, r.list, T, status, dX, dL, ctx->d_gacc, r.stream,
+                                    ctx->n_sm, r.lists, &r.ctl->backward64));
+  return FPT_OK;
+}
+
+// BFGS of one order's paths.
+static fpt_status bfgs_order(fpt_ctx* ctx, const SceneDev& S, const fpt_batch* b, const OrderRun& r,
+                             const SolveCfg& sc, int specialize, float* T, uint8_t* status, uint8_t* iters) {
+  ProfScope ps(ctx, FPT_K_BFGS);
+  const int n = r.n;
+  // pattern kernels pay off for buckets that fill the GPU several times over.  Seeded and explicit
+  // batches keep an order's small buckets together, and the unified kernel takes them in one launch;
+  // an exhaustive order with a small pattern runs the unified kernel throughout.
+  const bool listed = b->dev.mode != BATCH_EXHAUSTIVE;
+  const bool force = specialize == 2;
+  bool by_pattern = specialize && sc.refill > 0 && n <= kMaxBfgsOrder;
+  for (unsigned q = 0; by_pattern && !listed && !force && q < (1u << n); ++q) {
+    const PathRec* qlist;
+    const uint64_t qcnt = pattern_slice(b, n, q, &qlist);
+    if (qcnt && qcnt < min_pattern_bucket(ctx)) by_pattern = false;
+  }
+  struct Launch {
+    int pattern;
+    uint64_t cnt;
+    const PathRec* list;
+    unsigned long long* work;
+  };
+  Launch todo[(1 << kMaxBfgsOrder) + 1];
+  int count = 0;
+  if (by_pattern) {
+    for (unsigned q = 0; q < (1u << n); ++q) {
+      const PathRec* qlist;
+      const uint64_t qcnt = pattern_slice(b, n, q, &qlist);
+      if (!qcnt || (listed && !force && qcnt < min_pattern_bucket(ctx))) continue;
+      todo[count++] = {(int)q, qcnt, qlist, r.ctl->work + q};
+    }
+    if (listed && !force && b->small_count[n])
+      todo[count++] = {-1, b->small_count[n], b->d_lists + b->small_start[n], r.ctl->work + 32};
+  } else {
+    todo[count++] = {-1, r.cnt, r.list, r.ctl->work + 32};
+  }
+  // the pattern launches of one order are independent: spread them over the side streams so that
+  // each launch's tail overlaps the next one; each concurrent launch has its own work counter
+  const int used = count < 2 ? 0 : (count < fpt_ctx::kSide ? count : fpt_ctx::kSide);
+  if (used) {
+    CUDA_OR_FAIL(ctx, cudaEventRecord(ctx->fork_ev, r.stream));
+    for (int k = 0; k < used; ++k) CUDA_OR_FAIL(ctx, cudaStreamWaitEvent(ctx->side[k], ctx->fork_ev, 0));
+  }
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < count && e == cudaSuccess; ++i)
+    e = launch_bfgs(n, todo[i].pattern, S, b->dev, sc, todo[i].cnt, todo[i].list, T, status, iters,
+                    used ? ctx->side[i % used] : r.stream, ctx->n_sm, todo[i].work);
+  // join every side stream that waited on the fork, also after an error (a stream capture must end joined)
+  for (int k = 0; k < used; ++k) {
+    const cudaError_t f = cudaEventRecord(ctx->join_ev[k], ctx->side[k]);
+    const cudaError_t w = f == cudaSuccess ? cudaStreamWaitEvent(r.stream, ctx->join_ev[k], 0) : f;
+    if (e == cudaSuccess) e = w;
+  }
+  CUDA_OR_FAIL(ctx, e);
+  return FPT_OK;
+}
+
+// What fpt_solve_grad asks for after each order's solve.
+struct BackwardAfter {
+  BackwardCfg cfg;
+  const float* dX;
+  const float* dL;
+};
+
+// Solve of every order of the batch; with grad, the fused backward in the polish; with after, each order's
+// adjoint kernels behind its solve on the same stream.
 static fpt_status solve_impl(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* bc, const fpt_solve_params* prm,
                              float* T, float* X, float* L, uint8_t* status, uint8_t* iters, float* rho,
-                             const GradCfg* grad) {
+                             const GradCfg* grad, const BackwardAfter* after) {
   fpt_status st = check_scene_batch(ctx, s, bc);
   if (st != FPT_OK) return st;
   if (bc->dev.n_paths > 0 && (!T || !status)) return fail(ctx, FPT_EINVAL, "T_out and status_out are required");
@@ -899,102 +1096,58 @@ static fpt_status solve_impl(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* 
     return fail(ctx, FPT_EINVAL, "bad solver parameters");
   fpt_batch* b = const_cast<fpt_batch*>(bc);
   CUDA_OR_FAIL(ctx, cudaSetDevice(ctx->device));
-  st = ensure_buckets(ctx, b, scene_dev(s));
-  if (st != FPT_OK) return st;
   const SceneDev S = scene_dev(s);
+  st = ensure_buckets(ctx, b, S);
+  if (st != FPT_OK) return st;
   const float kink = p.kink_stop > 0.f ? p.kink_stop : 0.1f * p.deg_tol;
   SolveCfg sc{p.max_iters, p.fp_iters, p.fixed_iters, p.tol_step * p.tol_step, kink * kink,
               p.refill > 32 ? 32 : p.refill, p.init_mode == 1, kMaxChunk};
   // the polish needs its Newton step only to a modest relative accuracy: 100x looser pivot test than the adjoint
   PolishCfg pc{POLISH_SOLVE, p.polish, p.solved_tol, p.deg_tol, 1e-2f * p.cond_fp64, p.polish_fp64,
                p.polish_radius};
+  OrderPlan plan;
+  st = plan_orders(ctx, b, true, true, plan);
+  if (st != FPT_OK) return st;
   if (b->dev.n_max > kMaxBfgsOrder) {
     // the kernels of orders 1-5 write the first five slots of a path; clear the rest
     CUDA_OR_FAIL(ctx, cudaMemsetAsync(T, 0, b->dev.n_paths * (uint64_t)b->dev.n_max * 2 * sizeof(float), ctx->stream));
     if (X) CUDA_OR_FAIL(ctx, cudaMemsetAsync(X, 0, b->dev.n_paths * (uint64_t)b->dev.n_max * 3 * sizeof(float), ctx->stream));
   }
-  for (int n = 1; n <= kMaxOrder; ++n) {
-    const PathRec* list;
-    uint64_t cnt = order_slice(b, n, &list);
-    if (!cnt) continue;
-    if (cnt > 0xFFFFFFFFull) return fail(ctx, FPT_EUNSUPPORTED, "more than 2^32 paths of one order");
-    if (p.init_mode == 1) {
+  fpt_mlp* m = p.init_mode == 1 ? ctx->init_mlp : nullptr;
+  if (m && plan.count && m->wt_stale) {
+    CUDA_OR_FAIL(ctx, launch_mlp_tile_weights(m->d_wb, m->d_wt, ctx->stream));
+    m->wt_stale = false;
+  }
+  CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_ctl, 0, kCtlBytes, ctx->stream));
+  return run_orders(ctx, plan, [&](const OrderRun& r) -> fpt_status {
+    if (m) {
       // learned start: fused features -> network -> T on the tensor cores
-      fpt_mlp* m = ctx->init_mlp;
-      if (m->wt_stale) {
-        CUDA_OR_FAIL(ctx, launch_mlp_tile_weights(m->d_wb, m->d_wt, ctx->stream));
-        m->wt_stale = false;
-      }
       ProfScope ps(ctx, FPT_K_MLP);
-      CUDA_OR_FAIL(ctx, launch_mlp_infer(S, b->dev, n, list, cnt, 1.f / m->scale, m->d_wt, m->d_w, T, ctx->d_err,
-                                         ctx->stream, ctx->n_sm));
+      CUDA_OR_FAIL(ctx, launch_mlp_infer(S, b->dev, r.n, r.list, r.cnt, 1.f / m->scale, m->d_wt, m->d_w, T, ctx->d_err,
+                                         r.stream, ctx->n_sm));
     }
-    {
-      ProfScope ps(ctx, FPT_K_BFGS);
-      // pattern kernels pay off for buckets that fill the GPU several times over.  Seeded and explicit
-      // batches keep an order's small buckets together, and the unified kernel takes them in one launch;
-      // an exhaustive order with a small pattern runs the unified kernel throughout.
-      const bool listed = b->dev.mode != BATCH_EXHAUSTIVE;
-      const bool force = p.specialize == 2;
-      bool by_pattern = p.specialize && sc.refill > 0 && n <= kMaxBfgsOrder;
-      for (unsigned q = 0; by_pattern && !listed && !force && q < (1u << n); ++q) {
-        const PathRec* qlist;
-        const uint64_t qcnt = pattern_slice(b, n, q, &qlist);
-        if (qcnt && qcnt < min_pattern_bucket(ctx)) by_pattern = false;
-      }
-      if (by_pattern) {
-        // the pattern launches of one order are independent: spread them over the side streams so that
-        // each launch's tail overlaps the next one; each concurrent launch has its own work counter
-        CUDA_OR_FAIL(ctx, cudaEventRecord(ctx->fork_ev, ctx->stream));
-        for (int k = 0; k < fpt_ctx::kSide; ++k) CUDA_OR_FAIL(ctx, cudaStreamWaitEvent(ctx->side[k], ctx->fork_ev, 0));
-        int used = 0;
-        for (unsigned q = 0; q < (1u << n); ++q) {
-          const PathRec* qlist;
-          const uint64_t qcnt = pattern_slice(b, n, q, &qlist);
-          if (!qcnt || (listed && !force && qcnt < min_pattern_bucket(ctx))) continue;
-          cudaStream_t sq = ctx->side[used % fpt_ctx::kSide];
-          ++used;
-          CUDA_OR_FAIL(ctx, launch_bfgs(n, (int)q, S, b->dev, sc, qcnt, qlist, T, status, iters, sq, ctx->n_sm,
-                                        ctx->d_work + q));
-        }
-        if (listed && !force && b->small_count[n]) {
-          cudaStream_t sq = ctx->side[used % fpt_ctx::kSide];
-          ++used;
-          CUDA_OR_FAIL(ctx, launch_bfgs(n, -1, S, b->dev, sc, b->small_count[n], b->d_lists + b->small_start[n], T,
-                                        status, iters, sq, ctx->n_sm, ctx->d_work + 32));
-        }
-        // join every side stream that waited on the fork, used or not (a stream capture must end joined)
-        for (int k = 0; k < fpt_ctx::kSide; ++k) {
-          CUDA_OR_FAIL(ctx, cudaEventRecord(ctx->join_ev[k], ctx->side[k]));
-          CUDA_OR_FAIL(ctx, cudaStreamWaitEvent(ctx->stream, ctx->join_ev[k], 0));
-        }
-      } else {
-        CUDA_OR_FAIL(ctx, launch_bfgs(n, -1, S, b->dev, sc, cnt, list, T, status, iters, ctx->stream, ctx->n_sm,
-                                      ctx->d_work));
-      }
-    }
-    st = ensure_rescue(ctx, cnt, n);
-    if (st != FPT_OK) return st;
+    fpt_status rs = bfgs_order(ctx, S, b, r, sc, p.specialize, T, status, iters);
+    if (rs != FPT_OK) return rs;
     {
       ProfScope ps(ctx, FPT_K_POLISH);
       GradCfg gc{};
       if (grad) {
         gc = *grad;
-        gc.rescue_list = ctx->d_rescue + cnt;
-        gc.rescue_count = ctx->d_rescue_n + 1;
+        gc.rescue_list = r.lists + r.cnt;
+        gc.rescue_count = &r.ctl->adjoint64;
       }
-      uint32_t* step_list = p.polish_all ? nullptr : ctx->d_rescue + 2 * cnt;
-      CUDA_OR_FAIL(ctx, launch_polish(n, S, b->dev, pc, cnt, list, T, X, L, status, rho, nullptr, nullptr, ctx->stream,
-                                      ctx->n_sm, ctx->d_rescue, ctx->d_rescue_n, grad ? &gc : nullptr, step_list,
-                                      ctx->d_rescue_n + 2, ctx->d_step));
+      uint32_t* step_list = p.polish_all ? nullptr : r.lists + 2 * r.cnt;
+      CUDA_OR_FAIL(ctx, launch_polish(r.n, S, b->dev, pc, r.cnt, r.list, T, X, L, status, rho, nullptr, nullptr,
+                                      r.stream, ctx->n_sm, r.lists, &r.ctl->polish64, grad ? &gc : nullptr, step_list,
+                                      &r.ctl->stepped, r.step));
     }
-  }
-  return FPT_OK;
+    return after ? backward_order(ctx, S, b, r, after->cfg, T, status, after->dX, after->dL) : FPT_OK;
+  });
 }
 
 fpt_status fpt_solve(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* bc, const fpt_solve_params* prm, float* T,
                      float* X, float* L, uint8_t* status, uint8_t* iters, float* rho) {
-  return solve_impl(ctx, s, bc, prm, T, X, L, status, iters, rho, nullptr);
+  return solve_impl(ctx, s, bc, prm, T, X, L, status, iters, rho, nullptr, nullptr);
 }
 
 // Context-owned FP64 gradient accumulators, sized for the scene and cleared.
@@ -1011,6 +1164,15 @@ static fpt_status ensure_gacc(fpt_ctx* ctx, const fpt_scene* s) {
   return FPT_OK;
 }
 
+// The settings of a backward call on this context.
+static BackwardCfg backward_cfg(fpt_ctx* ctx, uint8_t dl_mask) {
+  fpt_solve_params p;
+  fpt_default_params(&p);
+  BackwardCfg cfg{p.cond_fp64, p.deg_tol, ctx->acc_smem, ctx->acc_flush_tiles, dl_mask};
+  cfg.dropped = ctx->d_dropped;
+  return cfg;
+}
+
 fpt_status fpt_solve_grad(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* bc, const fpt_solve_params* prm,
                           const float* dX, const float* dL, uint8_t dL_status_mask, float* T, float* X, float* L,
                           uint8_t* status, uint8_t* iters, float* rho, float* g_tx, float* g_rx,
@@ -1020,29 +1182,29 @@ fpt_status fpt_solve_grad(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* bc,
   if (prm && prm->polish_fp64) return fail(ctx, FPT_EUNSUPPORTED, "fpt_solve_grad runs the double-float polish");
   if (prm && prm->polish < 1) return fail(ctx, FPT_EINVAL, "fpt_solve_grad needs polish >= 1");
   if (!status && bc->dev.n_paths > 0) return fail(ctx, FPT_EINVAL, "status_out is required");
-  if (!(prm && prm->fuse_adjoint)) {
-    // the adjoint kernels after the solve, with the cotangents given here
-    st = fpt_solve(ctx, s, bc, prm, T, X, L, status, iters, rho);
-    if (st != FPT_OK) return st;
-    return fpt_backward(ctx, s, bc, T, status, dX, dL, dL_status_mask, g_tx, g_rx, g_vertices);
-  }
   CUDA_OR_FAIL(ctx, cudaSetDevice(ctx->device));
   st = ensure_gacc(ctx, s);
   if (st != FPT_OK) return st;
-  fpt_solve_params p;
-  fpt_default_params(&p);
-  GradCfg gc{};
-  gc.dX = dX;
-  gc.dL = dL;
-  gc.dl_mask = dL ? (uint8_t)0 : dL_status_mask;
-  gc.cond_adj = p.cond_fp64;
-  gc.deg_tol = prm ? prm->deg_tol : p.deg_tol;
-  gc.gacc = ctx->d_gacc;
-  gc.flush_tiles = ctx->acc_flush_tiles;
-  gc.acc_in_smem = ctx->acc_smem;
-  gc.dropped = ctx->d_rescue_n + 3;
-  CUDA_OR_FAIL(ctx, cudaMemsetAsync(gc.dropped, 0, sizeof(unsigned), ctx->stream));
-  st = solve_impl(ctx, s, bc, prm, T, X, L, status, iters, rho, &gc);
+  CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_dropped, 0, sizeof(unsigned), ctx->stream));
+  if (!(prm && prm->fuse_adjoint)) {
+    // the adjoint kernels after each order's solve, with the cotangents given here
+    const BackwardAfter after{backward_cfg(ctx, dL ? (uint8_t)0 : dL_status_mask), dX, dL};
+    st = solve_impl(ctx, s, bc, prm, T, X, L, status, iters, rho, nullptr, &after);
+  } else {
+    fpt_solve_params p;
+    fpt_default_params(&p);
+    GradCfg gc{};
+    gc.dX = dX;
+    gc.dL = dL;
+    gc.dl_mask = dL ? (uint8_t)0 : dL_status_mask;
+    gc.cond_adj = p.cond_fp64;
+    gc.deg_tol = prm->deg_tol;
+    gc.gacc = ctx->d_gacc;
+    gc.flush_tiles = ctx->acc_flush_tiles;
+    gc.acc_in_smem = ctx->acc_smem;
+    gc.dropped = ctx->d_dropped;
+    st = solve_impl(ctx, s, bc, prm, T, X, L, status, iters, rho, &gc, nullptr);
+  }
   if (st != FPT_OK) return st;
   const SceneDev S = scene_dev(s);
   ProfScope ps(ctx, FPT_K_OTHER);
@@ -1063,18 +1225,16 @@ fpt_status fpt_validity(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* bc, c
   fpt_default_params(&p);
   const SceneDev S = scene_dev(s);
   PolishCfg pc{POLISH_VALIDITY, 0, p.solved_tol, p.deg_tol, 1e-2f * p.cond_fp64, 0};
-  for (int n = 1; n <= kMaxOrder; ++n) {
-    const PathRec* list;
-    uint64_t cnt = order_slice(b, n, &list);
-    if (!cnt) continue;
-    if (cnt > 0xFFFFFFFFull) return fail(ctx, FPT_EUNSUPPORTED, "more than 2^32 paths of one order");
-    st = ensure_rescue(ctx, cnt, n);
-    if (st != FPT_OK) return st;
+  OrderPlan plan;
+  st = plan_orders(ctx, b, true, false, plan);
+  if (st != FPT_OK) return st;
+  CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_ctl, 0, kCtlBytes, ctx->stream));
+  return run_orders(ctx, plan, [&](const OrderRun& r) -> fpt_status {
     ProfScope ps(ctx, FPT_K_POLISH);
-    CUDA_OR_FAIL(ctx, launch_polish(n, S, b->dev, pc, cnt, list, const_cast<float*>(T), nullptr, nullptr, nullptr, rho,
-                                    mask, bdist, ctx->stream, ctx->n_sm, ctx->d_rescue, ctx->d_rescue_n));
-  }
-  return FPT_OK;
+    CUDA_OR_FAIL(ctx, launch_polish(r.n, S, b->dev, pc, r.cnt, r.list, const_cast<float*>(T), nullptr, nullptr, nullptr,
+                                    rho, mask, bdist, r.stream, ctx->n_sm, r.lists, &r.ctl->polish64));
+    return FPT_OK;
+  });
 }
 
 fpt_status fpt_backward(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* bc, const float* T, const uint8_t* status,
@@ -1090,27 +1250,16 @@ fpt_status fpt_backward(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* bc, c
   st = ensure_gacc(ctx, s);
   if (st != FPT_OK) return st;
   const SceneDev S = scene_dev(s);
-  fpt_solve_params p;
-  fpt_default_params(&p);
   if (!dL && dL_status_mask && !status && bc->dev.n_paths > 0)
     return fail(ctx, FPT_EINVAL, "dL_status_mask needs status");
-  BackwardCfg bc_cfg{p.cond_fp64, p.deg_tol, ctx->acc_smem, ctx->acc_flush_tiles, dL ? (uint8_t)0 : dL_status_mask};
-  bc_cfg.dropped = ctx->d_rescue_n + 3;
-  CUDA_OR_FAIL(ctx, cudaMemsetAsync(bc_cfg.dropped, 0, sizeof(unsigned), ctx->stream));
-  for (int n = 1; n <= kMaxOrder; ++n) {
-    const PathRec* list;
-    uint64_t cnt = order_slice(b, n, &list);
-    if (!cnt) continue;
-    if (cnt > 0xFFFFFFFFull) return fail(ctx, FPT_EUNSUPPORTED, "more than 2^32 paths of one order");
-    st = ensure_rescue(ctx, cnt, n);
-    if (st != FPT_OK) return st;
-    ProfScope ps(ctx, FPT_K_BACKWARD);
-    BackwardCfg cfg_n = bc_cfg;
-    cfg_n.sel = ctx->d_rescue + 2 * cnt;  // the third list of the scratch (the polish's, free here)
-    cfg_n.sel_count = ctx->d_rescue_n + 2;
-    CUDA_OR_FAIL(ctx, launch_backward(n, S, b->dev, cfg_n, cnt, list, T, status, dX, dL, ctx->d_gacc, ctx->stream,
-                                      ctx->n_sm, ctx->d_rescue, ctx->d_rescue_n));
-  }
+  const BackwardCfg cfg = backward_cfg(ctx, dL ? (uint8_t)0 : dL_status_mask);
+  OrderPlan plan;
+  st = plan_orders(ctx, b, true, false, plan);
+  if (st != FPT_OK) return st;
+  CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_dropped, 0, sizeof(unsigned), ctx->stream));
+  CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_ctl, 0, kCtlBytes, ctx->stream));
+  st = run_orders(ctx, plan, [&](const OrderRun& r) { return backward_order(ctx, S, b, r, cfg, T, status, dX, dL); });
+  if (st != FPT_OK) return st;
   {
     ProfScope ps(ctx, FPT_K_OTHER);
     CUDA_OR_FAIL(ctx, launch_backward_finalize(S, nullptr, ctx->d_gacc, g_tx, g_rx, g_vertices, ctx->stream));
@@ -1177,18 +1326,16 @@ fpt_status fpt_occlusion(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* bc, 
   if (st != FPT_OK) return st;
   const SceneDev S = scene_dev(s);
   const float t = tol > 0.f ? tol : 1e-4f;
-  for (int n = 1; n <= kMaxOrder; ++n) {
-    const PathRec* list;
-    const uint64_t cnt = order_slice(b, n, &list);
-    if (!cnt) continue;
-    if (cnt > 0xFFFFFFFFull) return fail(ctx, FPT_EUNSUPPORTED, "more than 2^32 paths of one order");
-    st = ensure_rescue(ctx, cnt, n);
-    if (st != FPT_OK) return st;
+  OrderPlan plan;
+  st = plan_orders(ctx, b, true, false, plan);
+  if (st != FPT_OK) return st;
+  CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_ctl, 0, kCtlBytes, ctx->stream));
+  return run_orders(ctx, plan, [&](const OrderRun& r) -> fpt_status {
     ProfScope ps(ctx, FPT_K_OTHER);
-    CUDA_OR_FAIL(ctx, launch_occlusion(S, b->dev, n, list, cnt, T, status, status_mask, s->d_occ, s->n_occ, t,
-                                       blocked_out, ctx->d_rescue, ctx->d_rescue_n, ctx->stream, ctx->n_sm));
-  }
-  return FPT_OK;
+    CUDA_OR_FAIL(ctx, launch_occlusion(S, b->dev, r.n, r.list, r.cnt, T, status, status_mask, s->d_occ, s->n_occ, t,
+                                       blocked_out, r.lists, &r.ctl->selected, r.stream, ctx->n_sm));
+    return FPT_OK;
+  });
 }
 
 fpt_status fpt_backward_noalloc(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* b, const float* T,
@@ -1214,11 +1361,8 @@ fpt_status fpt_backward_noalloc(fpt_ctx* ctx, const fpt_scene* s, const fpt_batc
                   (unsigned long long)counts[n], n, kNoAllocMaxSlice);
   }
   CUDA_OR_FAIL(ctx, cudaSetDevice(ctx->device));
-  fpt_solve_params p;
-  fpt_default_params(&p);
-  BackwardCfg cfg{p.cond_fp64, p.deg_tol, ctx->acc_smem, ctx->acc_flush_tiles, dL ? (uint8_t)0 : dL_status_mask};
-  cfg.dropped = ctx->d_rescue_n + 3;  // context memory, allocated by fpt_create
-  CUDA_OR_FAIL(ctx, cudaMemsetAsync(cfg.dropped, 0, sizeof(unsigned), ctx->stream));
+  const BackwardCfg cfg = backward_cfg(ctx, dL ? (uint8_t)0 : dL_status_mask);
+  CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_dropped, 0, sizeof(unsigned), ctx->stream));
   CUDA_OR_FAIL(ctx, launch_backward_noalloc(ctx->device, scene_dev(s), b->dev, cfg, lists, counts, T, status, dX, dL,
                                             g_tx, g_rx, g_vertices, ctx->stream, ctx->n_sm));
   return FPT_OK;
@@ -1228,7 +1372,7 @@ fpt_status fpt_backward_dropped(fpt_ctx* ctx, uint64_t* count) {
   if (!ctx || !count) return fail(ctx, FPT_EINVAL, "null argument");
   CUDA_OR_FAIL(ctx, cudaSetDevice(ctx->device));
   unsigned h = 0;
-  CUDA_OR_FAIL(ctx, cudaMemcpyAsync(&h, ctx->d_rescue_n + 3, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
+  CUDA_OR_FAIL(ctx, cudaMemcpyAsync(&h, ctx->d_dropped, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
   CUDA_OR_FAIL(ctx, cudaStreamSynchronize(ctx->stream));
   *count = h;
   return FPT_OK;

@@ -27,6 +27,23 @@ inline unsigned rescue_grid(uint64_t n_local, int n_sm) {
   const uint64_t cap = (uint64_t)n_sm * kRescueCtasPerSm;
   return (unsigned)(want < cap ? want : cap);
 }
+// Grid of a kernel that strides over n items with `threads` per CTA: enough CTAs for the items, at most those
+// resident at once.  A slice that needs no more CTAs than there are SMs is below that cap whatever the
+// occupancy, and then the occupancy query (host time that small calls feel) is left out.
+template <class Kernel>
+inline cudaError_t strided_grid(Kernel fn, int threads, size_t smem, uint64_t n, int n_sm, unsigned& grid) {
+  const uint64_t want = (n + threads - 1) / threads;
+  if (want <= (uint64_t)n_sm) {
+    grid = (unsigned)want;
+    return cudaSuccess;
+  }
+  int per_sm = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
+  if (e != cudaSuccess) return e;
+  const uint64_t cap = (uint64_t)n_sm * (uint64_t)(per_sm < 1 ? 1 : per_sm);
+  grid = (unsigned)(want < cap ? want : cap);
+  return cudaSuccess;
+}
 constexpr size_t kMaxSmemBytes = 200 * 1024;  // dynamic shared memory a path kernel may request
 
 // Kernels launched by the calling thread; the API's profiler reads the
@@ -74,7 +91,8 @@ struct BackwardCfg {
   unsigned* dropped = nullptr;
 };
 
-// Per-order launches (n = 1..kMaxOrder).  `list` = nullptr for exhaustive batches.
+// Per-order launches (n = 1..kMaxOrder).  `list` = nullptr for exhaustive batches.  The counters that a launch
+// gets (work, rescue_count, step_count, sel_count) are zero when the stream reaches it: the caller clears them.
 // BFGS: pattern < 0 runs the unified kernel over every sequence of order n;
 // pattern = Q in [0, 2^n) runs the kernel of that interaction-type pattern
 // over a slice holding only sequences of pattern Q.

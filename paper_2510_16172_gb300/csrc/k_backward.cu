@@ -152,6 +152,8 @@ cudaError_t launch_backward_noalloc(int device, const SceneDev& S, const BatchDe
   if (e != cudaSuccess) return e;
   for (int n = 1; n <= kMaxOrder; ++n) {
     if (!counts[n]) continue;
+    e = cudaMemsetAsync(count, 0, sizeof(unsigned), stream);  // one counter and list, order after order
+    if (e != cudaSuccess) return e;
     e = launch_backward(n, S, B, cfg, counts[n], lists[n], T, status, dX, dL, acc, stream, n_sm, list, count);
     if (e != cudaSuccess) return e;
   }

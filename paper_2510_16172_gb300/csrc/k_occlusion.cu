@@ -111,15 +111,13 @@ cudaError_t launch_occlusion(const SceneDev& S, const BatchDev& B, int n, const 
   const bool listed = status != nullptr && mask != 0;
   if (listed) {
     if (!sel || !sel_count) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(sel_count, 0, sizeof(unsigned), stream);
-    if (e != cudaSuccess) return e;
     const uint64_t want = (n_local + kOccSelChunk - 1) / kOccSelChunk;
     const unsigned g = (unsigned)(want < (uint64_t)n_sm * 8 ? want : (uint64_t)n_sm * 8);
     if (g == 0) return cudaSuccess;
     occlusion_select_kernel<<<g, kOccSelThreads, 0, stream>>>(B, n, list, n_local, status, mask, blocked, sel,
                                                               sel_count);
     count_launch();
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   const size_t smem = (size_t)n_occ * kOcc * sizeof(float);
@@ -128,15 +126,10 @@ cudaError_t launch_occlusion(const SceneDev& S, const BatchDev& B, int n, const 
     cudaError_t e = cudaFuncSetAttribute(occlusion_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, occlusion_kernel, kThreads, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
   // a listed launch strides over the list; a full grid covers the largest list
-  const uint64_t want = (n_local + kThreads - 1) / kThreads;
-  const uint64_t cap = (uint64_t)n_sm * (uint64_t)per_sm;
-  const unsigned grid = (unsigned)(want < cap ? want : cap);
-  if (grid == 0) return cudaSuccess;
+  unsigned grid = 0;
+  const cudaError_t e = strided_grid(occlusion_kernel, kThreads, smem, n_local, n_sm, grid);
+  if (e != cudaSuccess || grid == 0) return e;
   occlusion_kernel<<<grid, kThreads, smem, stream>>>(S, B, n, list, n_local, T, listed ? sel : nullptr,
                                                      listed ? sel_count : nullptr, occ, n_occ, tol, blocked);
   count_launch();

@@ -702,14 +702,7 @@ cudaError_t launch_polish_n(const SceneDev& S, const BatchDev& B, const PolishCf
       cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
     }
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
-    uint64_t want = (n + kThreads - 1) / kThreads;
-    uint64_t cap = (uint64_t)n_sm * (uint64_t)per_sm;
-    grid = (unsigned)(want < cap ? want : cap);
-    return cudaSuccess;
+    return strided_grid(fn, kThreads, smem, n, n_sm, grid);
   };
   const size_t s64 = smem64 <= 160 * 1024 ? smem64 : 0;
   unsigned grid = 0;
@@ -737,21 +730,11 @@ cudaError_t launch_polish_n(const SceneDev& S, const BatchDev& B, const PolishCf
       }
     }
   }
-  e = cudaMemsetAsync(rescue_count, 0, sizeof(unsigned), stream);
-  if (e != cudaSuccess) return e;
   GradCfg gc{};
-  if (grad) {
-    gc = *grad;
-    e = cudaMemsetAsync(gc.rescue_count, 0, sizeof(unsigned), stream);
-    if (e != cudaSuccess) return e;
-  }
+  if (grad) gc = *grad;
   // adaptive polish: the first pass lists the paths that still need their Newton steps, the second
   // pass (a grid for a quarter of the slice; it strides over the list) takes them
   const bool two_pass = step_list != nullptr && step_delta != nullptr && cfg.mode == POLISH_SOLVE && cfg.steps > 0;
-  if (two_pass) {
-    e = cudaMemsetAsync(step_count, 0, sizeof(unsigned), stream);
-    if (e != cudaSuccess) return e;
-  }
   for (int pass = 0; pass < (two_pass ? 2 : 1); ++pass) {
     const uint32_t* in_l = pass == 1 ? step_list : nullptr;
     const unsigned* in_c = pass == 1 ? step_count : nullptr;
