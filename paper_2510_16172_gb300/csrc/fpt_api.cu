@@ -1123,7 +1123,7 @@ static fpt_status solve_impl(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* 
     if (m) {
       // learned start: fused features -> network -> T on the tensor cores
       ProfScope ps(ctx, FPT_K_MLP);
-      CUDA_OR_FAIL(ctx, launch_mlp_infer(S, b->dev, r.n, r.list, r.cnt, 1.f / m->scale, m->d_wt, m->d_w, T, ctx->d_err,
+      CUDA_OR_FAIL(ctx, launch_mlp_infer(S, b->dev, r.n, r.list, r.cnt, 1.f / m->scale, m->d_wt, m->d_w, T, 0, ctx->d_err,
                                          r.stream, ctx->n_sm));
     }
     fpt_status rs = bfgs_order(ctx, S, b, r, sc, p.specialize, T, status, iters);
@@ -1614,7 +1614,7 @@ fpt_status fpt_mlp_create(fpt_ctx* ctx, uint64_t seed, float length_scale, fpt_m
   for (float** p : {&m->d_w, &m->d_m, &m->d_v, &m->d_g})
     if (e == cudaSuccess) e = cudaMalloc(p, kMlpParams * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&m->d_wb, kMlpParams * sizeof(__nv_bfloat16));
-  if (e == cudaSuccess) e = cudaMalloc(&m->d_wt, kMlpTiledBytes);
+  if (e == cudaSuccess) e = cudaMalloc(&m->d_wt, 2 * kMlpHalfBytes);
   if (e == cudaSuccess) e = cudaMalloc(&m->d_wtT, kMlpWtElems * sizeof(__nv_bfloat16));
   if (e == cudaSuccess) e = cudaMalloc(&m->d_loss, sizeof(float));
   if (e != cudaSuccess) {
@@ -1863,19 +1863,25 @@ fpt_status fpt_mlp_infer(fpt_ctx* ctx, fpt_mlp* m, const fpt_scene* s, const fpt
   if (st != FPT_OK) return st;
   const SceneDev S = scene_dev(s);
   if (b->dev.n_paths == 0) return FPT_OK;
-  // slots past a path's order stay zero
-  CUDA_OR_FAIL(ctx, cudaMemsetAsync(T, 0, b->dev.n_paths * (uint64_t)b->dev.n_max * 2 * sizeof(float), ctx->stream));
   if (m->wt_stale) {
     CUDA_OR_FAIL(ctx, launch_mlp_tile_weights(m->d_wb, m->d_wt, ctx->stream));
     m->wt_stale = false;
   }
+  // Records carry their order, and a batch's lists follow the orders: one launch takes all orders whose records
+  // hold the ids, one the longer sequences.  The kernel also clears the slots past a path's order.
+  const PathRec* first = nullptr;
+  uint64_t run = 0;
   for (int n = 1; n <= kMaxOrder; ++n) {
     const PathRec* list;
     const uint64_t cnt = order_slice(b, n, &list);
-    if (!cnt) continue;
+    if (cnt && !run) first = list;
+    run += cnt;
+    const bool last = n == kMaxOrder || n == kMaxBfgsOrder || b->dev.mode == BATCH_EXHAUSTIVE;
+    if (!run || !last) continue;
     ProfScope ps(ctx, FPT_K_MLP);
-    CUDA_OR_FAIL(ctx, launch_mlp_infer(S, b->dev, n, list, cnt, 1.f / m->scale, m->d_wt, m->d_w, T, ctx->d_err,
-                                       ctx->stream, ctx->n_sm));
+    CUDA_OR_FAIL(ctx, launch_mlp_infer(S, b->dev, n, first, run, 1.f / m->scale, m->d_wt, m->d_w, T, b->dev.n_max,
+                                       ctx->d_err, ctx->stream, ctx->n_sm));
+    run = 0;
   }
   return FPT_OK;
 }

@@ -21,44 +21,12 @@
 
 #include "fpt_kernels.h"
 #include "mlp.h"
+#include "mlp_device.cuh"
 #include "tc.cuh"
 
 namespace fpt {
 
 constexpr int kGemmKC = 64;                  // K per chunk
-constexpr uint32_t kWaitNs = 1000000000u;   // mbarrier waits give up after 1 s
-constexpr int ERR_MMA_TIMEOUT = 3;
-
-// GELU in its tanh form (Hendrycks and Gimpel, arXiv:1606.08415):
-//   gelu(z) = z/2 (1 + tanh(u)),  u = sqrt(2/pi) (z + 0.044715 z^3),
-// with the hardware tanh approximation (PTX tanh.approx.f32, relative error
-// about 2^-11, below the BF16 rounding that follows every activation).  One
-// MUFU operation per activation: the epilogues of the inference kernel
-// evaluate 768 of them per path.
-__device__ __forceinline__ float tanh_approx(float x) {
-  float y;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-// u = z (K0 + K0 K1 z^2) and gelu = h + h tanh(u) with h = z/2: six operations.
-constexpr float kGeluK0 = 0.79788456080286536f;  // sqrt(2 / pi)
-constexpr float kGeluK1 = 0.044715f;
-constexpr float kGeluK01 = 0.0356774081363001f;  // K0 K1
-__device__ __forceinline__ float gelu(float z) {
-  const float h = 0.5f * z;
-  return fmaf(h, tanh_approx(z * fmaf(kGeluK01, z * z, kGeluK0)), h);
-}
-// gelu(z) and, in d, its derivative gelu'(z) = (1 + th) / 2 + (z / 2) (1 - th^2) K0 (1 + 3 K1 z^2), from one
-// tanh.  The training forward keeps gelu'(Z) for the backward (dZ = dH gelu'(Z)), so the backward's
-// epilogue multiplies instead of evaluating the derivative again.
-__device__ __forceinline__ float gelu_with_grad(float z, float& d) {
-  const float z2 = z * z;
-  const float th = tanh_approx(z * fmaf(kGeluK01, z2, kGeluK0));
-  const float h = 0.5f * z;
-  d = 0.5f * (1.f + th) + 0.5f * z * (1.f - th * th) * kGeluK0 * fmaf(3.f * kGeluK1, z2, 1.f);
-  return fmaf(h, th, h);
-}
-
 // Gather rows [r0, r0 + 128) x k [k0, k0 + 64) of a strided bf16 matrix into a
 // 128 x 64 K-major tile (zero outside rows < R, k < K).
 __device__ __forceinline__ void load_tile(unsigned char* tile, const __nv_bfloat16* src, long long s_r, long long s_k,
@@ -408,37 +376,6 @@ __device__ __forceinline__ void store16_bf16(__nv_bfloat16* p, const float (&x)[
     for (int i = 0; i < 16; ++i)
       if (i < nv) p[i * sn] = __float2bfloat16(x[i]);
   }
-}
-
-// Sum of x[i] over the warp's 32 lanes for each of the 16 columns i: a transposing butterfly (16 shuffles).
-// Returns the sum of column ((lane >> 1) & 8) | ((lane >> 1) & 4) | ((lane >> 1) & 2) | ((lane >> 1) & 1),
-// i.e. column lane / 2 in bit-reversed halves: lane bits 4, 3, 2, 1 select column bits 3, 2, 1, 0.
-__device__ __forceinline__ float warp_colsum16(const float (&x)[16], int lane) {
-  float a[8], b[4], c[2];
-  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4, h2 = lane & 2;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float send = h16 ? x[i] : x[i + 8];
-    const float keep = h16 ? x[i + 8] : x[i];
-    a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float send = h8 ? a[i] : a[i + 4];
-    const float keep = h8 ? a[i + 4] : a[i];
-    b[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const float send = h4 ? b[i] : b[i + 2];
-    const float keep = h4 ? b[i + 2] : b[i];
-    c[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  }
-  const float d = (h2 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h2 ? c[0] : c[1], 2);
-  return d + __shfl_xor_sync(0xffffffffu, d, 1);
-}
-__device__ __forceinline__ int warp_colsum16_column(int lane) {
-  return ((lane >> 1) & 8) | ((lane >> 1) & 4) | ((lane >> 1) & 2) | ((lane >> 1) & 1);
 }
 
 // Z[m][n0 .. n0 + 15] (zero past N or M) into registers; 16-byte loads when aligned and whole.
@@ -908,104 +845,6 @@ cudaError_t launch_gemm(const GemmArgs& g, int k_split, cudaStream_t stream) {
 // features, loss, bias gradients, Adam, learned start
 // ---------------------------------------------------------------------------
 
-// 64 features of one path (see include/fpt.h): origin o = (TX + RX)/2, scale S;
-// per interaction the orthogonal projections of TX and RX onto the object's
-// affine hull in its own parameters, their distances to it, the first basis
-// length, and the distance-weighted combination of the two projections.  Also
-// the per-slot Gram matrix A^T A / S^2 (g11, g12, g22) of the loss.
-__device__ __forceinline__ void path_features(const SceneDev& S, const PathDesc& d, float inv_scale,
-                                              __nv_bfloat16* f, float* G) {
-  float tx[3], rx[3], o[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    tx[c] = S.tx32[kEnd32 * d.tx + c] + S.tx32[kEnd32 * d.tx + 3 + c];
-    rx[c] = S.rx32[kEnd32 * d.rx + c] + S.rx32[kEnd32 * d.rx + 3 + c];
-    o[c] = 0.5f * (tx[c] + rx[c]);
-  }
-  float v[kMlpIn], gram[12];
-#pragma unroll
-  for (int k = 0; k < kMlpIn; ++k) v[k] = 0.f;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) gram[k] = 0.f;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    v[c] = (tx[c] - o[c]) * inv_scale;
-    v[3 + c] = (rx[c] - o[c]) * inv_scale;
-  }
-  const bool valid = !(d.flags & ST_INVALID);
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    if (s < d.n && valid) {
-      const float* r = S.rec32 + kRec32 * d.ids[s];
-      const bool edge = S.aux[kAux * d.ids[s] + 2] != 0.f;
-      float b[3], a1[3], a2[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        b[c] = r[c] + r[3 + c];
-        a1[c] = r[6 + c];
-        a2[c] = r[9 + c];
-      }
-      const float g11 = a1[0] * a1[0] + a1[1] * a1[1] + a1[2] * a1[2];
-      const float g12 = a1[0] * a2[0] + a1[1] * a2[1] + a1[2] * a2[2];
-      const float g22 = a2[0] * a2[0] + a2[1] * a2[1] + a2[2] * a2[2];
-      const float det = g11 * g22 - g12 * g12;
-      float tau[2][2], dist[2];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const float* pt = q == 0 ? tx : rx;
-        float rr[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) rr[c] = pt[c] - b[c];
-        const float c1 = a1[0] * rr[0] + a1[1] * rr[1] + a1[2] * rr[2];
-        const float c2 = a2[0] * rr[0] + a2[1] * rr[1] + a2[2] * rr[2];
-        if (edge) {
-          tau[q][0] = c1 / g11;
-          tau[q][1] = 0.f;
-        } else {
-          tau[q][0] = (g22 * c1 - g12 * c2) / det;
-          tau[q][1] = (g11 * c2 - g12 * c1) / det;
-        }
-        float e2 = 0.f;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const float e = rr[c] - tau[q][0] * a1[c] - tau[q][1] * a2[c];
-          e2 += e * e;
-        }
-        dist[q] = sqrtf(e2) * inv_scale;
-      }
-      const int base = 6 + 11 * s;
-      v[base] = 1.f;
-      v[base + 1] = edge ? 1.f : 0.f;
-      v[base + 2] = tau[0][0];
-      v[base + 3] = tau[0][1];
-      v[base + 4] = tau[1][0];
-      v[base + 5] = tau[1][1];
-      v[base + 6] = dist[0];
-      v[base + 7] = dist[1];
-      v[base + 8] = sqrtf(g11) * inv_scale;
-      const float dsum = dist[0] + dist[1];
-#pragma unroll
-      for (int k = 0; k < 2; ++k)
-        v[base + 9 + k] = dsum > 0.f ? (dist[1] * tau[0][k] + dist[0] * tau[1][k]) / dsum
-                                     : 0.5f * (tau[0][k] + tau[1][k]);
-      const float is2 = inv_scale * inv_scale;
-      gram[3 * s] = g11 * is2;
-      gram[3 * s + 1] = g12 * is2;
-      gram[3 * s + 2] = g22 * is2;
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < kMlpIn; k += 8) {
-    __nv_bfloat16 e[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) e[q] = __float2bfloat16(v[k + q]);
-    *reinterpret_cast<uint4*>(f + k) = *reinterpret_cast<uint4*>(e);
-  }
-  if (G)
-#pragma unroll
-    for (int k = 0; k < 12; ++k) G[k] = gram[k];
-}
-
 // all paths of a batch (global index order) or one order slice (local index order)
 __global__ void mlp_features_kernel(SceneDev S, BatchDev B, int n, const PathRec* list, uint64_t first,
                                     uint64_t count, float inv_scale, __nv_bfloat16* X, float* G) {
@@ -1182,37 +1021,14 @@ __global__ void mlp_transpose_weights_kernel(const __nv_bfloat16* __restrict__ w
   }
 }
 
+__global__ void mlp_tile_weights_kernel(const __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ wt) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < kMlpParams) tile_weight(i, wb[i], wt);
+}
+
 __global__ void to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, int n) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     dst[i] = __float2bfloat16(src[i]);
-}
-
-// Starting parameters of a path of order n from the network's outputs y (slots 1-4; an edge's
-// second parameter -- bit s of `edges` -- and the later slots start at 1/2, and so does an output
-// that is not finite or beyond 1e3, and every slot of an invalid sequence).  The slot loop runs over
-// compile-time indices so that y stays in registers.
-__device__ __forceinline__ void write_start(int n, bool use, unsigned edges, const float (&y)[8], float2* To) {
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    if (s < n) {
-      float t0 = 0.5f, t1 = 0.5f;
-      if (use) {
-        if (isfinite(y[2 * s]) && fabsf(y[2 * s]) < 1e3f) t0 = y[2 * s];
-        if (!((edges >> s) & 1u) && isfinite(y[2 * s + 1]) && fabsf(y[2 * s + 1]) < 1e3f) t1 = y[2 * s + 1];
-      }
-      To[s] = make_float2(t0, t1);
-    }
-  }
-  for (int s = 4; s < n; ++s) To[s] = make_float2(0.5f, 0.5f);
-}
-
-// bit s: slot s (s < 4) of the path is an edge
-__device__ __forceinline__ unsigned edge_mask(const SceneDev& S, const PathDesc& d) {
-  unsigned m = 0;
-#pragma unroll
-  for (int s = 0; s < 4; ++s)
-    if (s < d.n && S.aux[kAux * d.ids[s] + 2] != 0.f) m |= 1u << s;
-  return m;
 }
 
 // learned start from unfused network outputs Y [count][16] (local indices first .. first + count)
@@ -1227,313 +1043,6 @@ __global__ void mlp_start_kernel(SceneDev S, BatchDev B, int n, const PathRec* l
     write_start(d.n, !(d.flags & ST_INVALID), edge_mask(S, d), y,
                 reinterpret_cast<float2*>(T) + d.g * (uint64_t)B.n_max);
   }
-}
-
-// ---------------------------------------------------------------------------
-// Fused, persistent inference for the learned start (two CTAs per SM).
-//
-// Per tile of 128 paths: features are computed straight into the shared
-// activation tile (K-major, K = 64), then four layers run on the tensor cores
-// with the accumulator in TMEM; each epilogue adds the bias, applies GELU and
-// writes the BF16 activations back into the same tile (K = 256) for the next
-// layer; the last one writes the starting parameters into T.  The weights are
-// pre-tiled in global memory as 19 units, each K-major in core matrices: for
-// layers 1-3 all 256 outputs x 32 input columns (16 KB, two MMAs with N = 256
-// into the whole TMEM accumulator; an MMA costs about the same time whatever
-// its N, so the widest one wastes least), for the output layer all of it, 16
-// outputs x 256 columns as four 64-column chunks (8 KB, sixteen MMAs with
-// N = 16: one unit instead of four, each unit paying a copy's latency).  They
-// stream through two 16 KB shared buffers,
-// prefetched one unit ahead: lane 0 of warp 0 waits for the MMAs that last read
-// a buffer before refilling it.  A CTA's steps are serial -- features,
-// MMAs, CUDA-core epilogue -- so the kernel is sized (103 KB of shared memory,
-// 256 TMEM columns, at most 117 registers) for two CTAs per SM, whose phases
-// interleave.  All waits are bounded.
-// ---------------------------------------------------------------------------
-constexpr int kInferThreads = 256;
-constexpr int kInferCtasPerSm = 2;
-constexpr int kUnitsPerTile = 19;  // streamed units: W1 2 K-halves, W2 and W3 8 each, W4 whole
-
-// One K = 16 MMA (M = 128) occupies an SM's tensor pipe for about the same time whatever N is (measured on
-// the GB300: ~131 cycles for N = 64, 128 and 256), so the hidden layers run with N = 256: a unit of W1-W3
-// is all 256 outputs x 32 input columns (16 KB, two MMAs); the output layer (16 outputs) is one unit of
-// four 64-column chunks (2 KB each, four MMAs each).
-__host__ __device__ constexpr int unit_layer(int u) { return u < 2 ? 0 : (u < 10 ? 1 : (u < 18 ? 2 : 3)); }
-// first input column of unit u within its layer
-__host__ __device__ constexpr int unit_k0(int u) {
-  return u < 2 ? 32 * u : (u < 10 ? 32 * (u - 2) : (u < 18 ? 32 * (u - 10) : 0));
-}
-__host__ __device__ constexpr bool unit_ends_layer(int u) { return u == 1 || u == 9 || u == 17 || u == 18; }
-__host__ __device__ constexpr uint32_t unit_bytes(int u) { return u < 18 ? 256u * 32u * 2u : 4u * 16u * 64u * 2u; }
-__host__ __device__ constexpr uint32_t unit_offset(int u) { return (uint32_t)(u < 18 ? u : 18) * 16384u; }
-// the output layer's 64-column chunk c (16 x 64, 2 KB) within the tiled weights
-__host__ __device__ constexpr uint32_t w4_chunk_offset(int c) { return unit_offset(18) + (uint32_t)c * 2048u; }
-// the units of a tile cover the tiled weights once, back to back
-__host__ __device__ constexpr bool units_tile_weights() {
-  for (int u = 0; u + 1 < kUnitsPerTile; ++u)
-    if (unit_offset(u) + unit_bytes(u) != unit_offset(u + 1)) return false;
-  return unit_offset(kUnitsPerTile - 1) + unit_bytes(kUnitsPerTile - 1) == kMlpTiledBytes &&
-         kMlpTiledBytes == 2u * (kMlpHidden * kMlpIn + 2 * kMlpHidden * kMlpHidden + kMlpOut * kMlpHidden);
-}
-static_assert(units_tile_weights(), "weight units");
-
-// bf16 parameter copy ([out][in] per layer) -> the streamed units, each K-major in core matrices of 8 rows
-// x 8 columns: a W1-W3 unit (256 rows x 32 columns) has core matrix (row group, column group) at
-// (group * 4 + column group) * 128 bytes; a W4 chunk (16 x 64) at (group * 8 + column group) * 128.
-__global__ void mlp_tile_weights_kernel(const __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ wt) {
-  const int n1 = 256 * 64, n2 = 256 * 256, n4 = 16 * 256;
-  const int total = n1 + 2 * n2 + n4;
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
-    int layer, r, k, K, off;
-    if (idx < n1) {
-      layer = 0; K = 64; off = kOffW1; r = idx / K; k = idx % K;
-    } else if (idx < n1 + n2) {
-      layer = 1; K = 256; off = kOffW2; r = (idx - n1) / K; k = (idx - n1) % K;
-    } else if (idx < n1 + 2 * n2) {
-      layer = 2; K = 256; off = kOffW3; r = (idx - n1 - n2) / K; k = (idx - n1 - n2) % K;
-    } else {
-      layer = 3; K = 256; off = kOffW4; r = (idx - n1 - 2 * n2) / K; k = (idx - n1 - 2 * n2) % K;
-    }
-    uint32_t byte;
-    if (layer < 3) {
-      const int u = (layer == 0 ? 0 : (layer == 1 ? 2 : 10)) + k / 32;
-      byte = unit_offset(u) + tc::kmajor_offset(r, k % 32, 32);
-    } else {
-      byte = w4_chunk_offset(k / 64) + tc::kmajor_offset(r, k % 64, 64);
-    }
-    wt[byte / 2] = wb[off + r * K + k];
-  }
-}
-
-struct InferSmem {
-  unsigned char act[128 * 256 * 2];
-  unsigned char wbuf[2][128 * 64 * 2];
-  float bias[3 * 256 + 16];
-  uint64_t row_g[128];     // the tile's paths: global index,
-  uint32_t row_info[128];  // order | (sequence usable) << 8 | edge mask << 16 (order 0: no path)
-  uint64_t full[2], done[2], layer;
-  uint32_t tmem;
-  int fail;
-};
-
-// Path source, fixed per launch: kSrcEnum, an exhaustive batch's enumeration of order n; kSrcRec, a
-// bucket of records of order n <= kMaxBfgsOrder (the ids in the record); kSrcRecDecode, a bucket of
-// longer sequences (ids decoded from the global index).
-enum { kSrcEnum = 0, kSrcRec = 1, kSrcRecDecode = 2 };
-
-template <int kSrc>
-__device__ __forceinline__ void infer_fetch(const BatchDev& B, int n, const PathRec* list, uint64_t j, PathDesc& d) {
-  if constexpr (kSrc == kSrcEnum) {
-    decode_exhaustive_order(B, n, j, d);
-  } else {
-    load_rec(list, j, d);
-    if constexpr (kSrc == kSrcRecDecode) decode_global(B, d.g, d);
-  }
-}
-
-template <int kSrc>
-__global__ void __launch_bounds__(kInferThreads, kInferCtasPerSm) mlp_infer_kernel(SceneDev S, BatchDev B, int n,
-                                                                     const PathRec* __restrict__ list, uint64_t count,
-                                                                     float inv_scale,
-                                                                     const __nv_bfloat16* __restrict__ wt,
-                                                                     const float* __restrict__ params, float* T,
-                                                                     int* err) {
-  extern __shared__ __align__(1024) unsigned char infer_smem[];
-  InferSmem& sm = *reinterpret_cast<InferSmem*>(infer_smem);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint64_t n_tiles = (count + 127) / 128;
-  const uint64_t my_tiles = blockIdx.x < n_tiles ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  const uint64_t total_q = my_tiles * kUnitsPerTile;
-  if (tid == 0) {
-    for (int b = 0; b < 2; ++b) {
-      tc::mbar_init(&sm.full[b], 1);
-      tc::mbar_init(&sm.done[b], 1);
-    }
-    tc::mbar_init(&sm.layer, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    sm.fail = 0;
-  }
-  for (int i = tid; i < 256; i += blockDim.x) {
-    sm.bias[i] = params[kOffB1 + i];
-    sm.bias[256 + i] = params[kOffB2 + i];
-    sm.bias[512 + i] = params[kOffB3 + i];
-  }
-  if (tid < 16) sm.bias[768 + tid] = params[kOffB4 + tid];
-  if (warp == 0) {
-    tc::tmem_alloc(&sm.tmem, 256);
-    tc::tmem_relinquish();
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = sm.tmem;
-  const char* wsrc = reinterpret_cast<const char*>(wt);
-  uint32_t full_ph = 0u, done_ph = 0u, layer_ph = 0u;  // mbarrier phases, one bit per buffer
-  if (tid == 0 && total_q > 0) {
-    tc::mbar_expect_tx(&sm.full[0], unit_bytes(0));
-    tc::bulk_g2s(sm.wbuf[0], wsrc + unit_offset(0), unit_bytes(0), &sm.full[0]);
-  }
-  uint64_t q = 0;
-  for (uint64_t ti = 0; ti < my_tiles; ++ti) {
-    const uint64_t first = (blockIdx.x + ti * gridDim.x) * 128;
-    // features of the tile's 128 paths (K = 64 layout)
-    if (tid < 128) {
-      __nv_bfloat16 f[kMlpIn];
-      if (first + tid < count) {
-        PathDesc d;
-        infer_fetch<kSrc>(B, n, list, first + tid, d);
-        path_features(S, d, inv_scale, f, nullptr);
-        sm.row_g[tid] = d.g;
-        sm.row_info[tid] = (uint32_t)d.n | (d.flags & ST_INVALID ? 0u : 1u << 8) | (edge_mask(S, d) << 16);
-      } else {
-#pragma unroll
-        for (int k = 0; k < kMlpIn; ++k) f[k] = __float2bfloat16(0.f);
-        sm.row_info[tid] = 0u;
-      }
-#pragma unroll
-      for (int g8 = 0; g8 < kMlpIn / 8; ++g8)
-        *reinterpret_cast<uint4*>(sm.act + tc::kmajor_offset(tid, g8 * 8, 64)) = reinterpret_cast<uint4*>(f)[g8];
-    }
-    tc::fence_async_smem();
-    tc::fence_before_sync();
-    __syncthreads();
-    for (int lq = 0; lq < kUnitsPerTile; ++lq, ++q) {
-      const int b = (int)(q & 1);
-      const int layer = unit_layer(lq), k0 = unit_k0(lq);
-      // warp 0 issues the copies and MMAs: lane 0 works while its warp-mates wait at the warp
-      // barrier, so that their mbarrier polls below never hold up the issuing lane
-      if (warp == 0) {
-        if (lane == 0) {
-          // refill the other buffer with the next chunk once the MMAs that read it (chunk q - 1) are done
-          if (q + 1 < total_q) {
-            const int nb = b ^ 1;
-            if (q >= 1) {
-              if (!tc::mbar_wait(&sm.done[nb], (done_ph >> nb) & 1u, kWaitNs)) sm.fail = 1;
-              done_ph ^= 1u << nb;
-            }
-            const int nq = (lq + 1) % kUnitsPerTile;
-            tc::mbar_expect_tx(&sm.full[nb], unit_bytes(nq));
-            tc::bulk_g2s(sm.wbuf[nb], wsrc + unit_offset(nq), unit_bytes(nq), &sm.full[nb]);
-          }
-          if (!tc::mbar_wait(&sm.full[b], (full_ph >> b) & 1u, kWaitNs)) sm.fail = 1;
-          full_ph ^= 1u << b;
-          tc::fence_after_sync();
-          const uint32_t K_act = layer == 0 ? 64u : 256u;
-          const uint32_t a0 = tc::smem_u32(sm.act), w0 = tc::smem_u32(sm.wbuf[b]);
-          if (!sm.fail) {
-            // the unit's first descriptors; each next K = 16 step starts 256 bytes further, i.e. 16 more
-            // in the 14-bit start-address field (shared addresses stay below 2^18: the field never carries)
-            const uint64_t ad = tc::smem_desc(a0 + (uint32_t)(k0 / 8) * 128u, 128u, (K_act / 8u) * 128u);
-            if (layer < 3) {  // 256 outputs x 32 columns: two MMAs with N = 256
-              const uint64_t bd = tc::smem_desc(w0, 128u, 4u * 128u);
-              const uint32_t idesc = tc::idesc_bf16(128, 256);
-              tc::mma_bf16(tmem, ad, bd, idesc, k0 > 0 ? 1u : 0u);
-              tc::mma_bf16(tmem, ad + 16u, bd + 16u, idesc, 1u);
-            } else {  // 16 outputs x 256 columns: four 64-column chunks of four MMAs with N = 16
-              const uint32_t idesc = tc::idesc_bf16(128, 16);
-#pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                // chunk c: activation columns 64 c .. 64 c + 63 (eight 8-column groups of 128 bytes on), and its
-                // 2 KB of weights
-                const uint64_t bd = tc::smem_desc(w0 + (uint32_t)c * 2048u, 128u, 8u * 128u);
-                const uint64_t adc = ad + 64u * (uint64_t)c;
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                  tc::mma_bf16(tmem, adc + 16u * kk, bd + 16u * kk, idesc, (c > 0 || kk > 0) ? 1u : 0u);
-              }
-            }
-          }
-          tc::mma_commit(&sm.done[b]);
-          if (unit_ends_layer(lq)) tc::mma_commit(&sm.layer);
-        }
-        __syncwarp();
-      }
-      if (!unit_ends_layer(lq)) continue;
-      // end of a layer: wait for its MMAs, then the epilogue
-      if (!tc::mbar_wait(&sm.layer, layer_ph, kWaitNs)) sm.fail = 1;
-      layer_ph ^= 1u;
-      tc::fence_after_sync();
-      const int rg = warp & 3;  // TMEM lane group of this warp
-      const int row = rg * 32 + lane;
-      if (layer < 3) {
-        const int c0 = (warp >> 2) * 128;
-        const float* bias = sm.bias + layer * 256;
-        for (int cc = c0; cc < c0 + 128; cc += 32) {
-          float v[32];
-          tc::tmem_ld32(tmem + ((uint32_t)(rg * 32) << 16) + (uint32_t)cc, v);
-#pragma unroll
-          for (int g8 = 0; g8 < 4; ++g8) {
-            uint32_t w[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const int c = g8 * 8 + 2 * k;
-              const __nv_bfloat162 p = __floats2bfloat162_rn(gelu(v[c] + bias[cc + c]), gelu(v[c + 1] + bias[cc + c + 1]));
-              w[k] = *reinterpret_cast<const uint32_t*>(&p);
-            }
-            *reinterpret_cast<uint4*>(sm.act + tc::kmajor_offset(row, cc + g8 * 8, 256)) = make_uint4(w[0], w[1], w[2], w[3]);
-          }
-        }
-      } else if (warp < 4) {
-        float v[16];
-        tc::tmem_ld16(tmem + ((uint32_t)(rg * 32) << 16), v);
-        const uint32_t info = sm.row_info[row];
-        if (info & 0xFFu) {
-          float y[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) y[i] = v[i] + sm.bias[768 + i];
-          write_start((int)(info & 0xFFu), (info >> 8) & 1u, info >> 16, y,
-                      reinterpret_cast<float2*>(T) + sm.row_g[row] * (uint64_t)B.n_max);
-        }
-      }
-      tc::fence_async_smem();
-      tc::fence_before_sync();
-      __syncthreads();
-      if (sm.fail) break;
-    }
-    if (sm.fail) break;
-  }
-  if (sm.fail && tid == 0) {
-    if (err) atomicCAS(err, 0, ERR_MMA_TIMEOUT);
-    tc::mbar_wait(&sm.layer, layer_ph, kWaitNs);  // let MMAs in flight finish before TMEM is freed
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, 256);
-}
-
-// ---------------------------------------------------------------------------
-// Training data order: a seeded pseudo-random permutation of [0, n) per epoch, evaluated index by index
-// (a four-round Feistel network on 2h-bit words, 2^(2h) >= n, with cycle walking back into [0, n)), and
-// the gather of one mini-batch's rows into contiguous buffers.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint64_t mix64(uint64_t z) {
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
-  return z ^ (z >> 31);
-}
-
-__device__ __forceinline__ uint64_t feistel(uint64_t x, int h, uint64_t key) {
-  const uint64_t mask = (1ULL << h) - 1ULL;
-  uint64_t l = x >> h, r = x & mask;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const uint64_t f = mix64(r ^ (key + 0x9E3779B97F4A7C15ULL * (uint64_t)(k + 1))) & mask;
-    const uint64_t nl = r;
-    r = l ^ f;
-    l = nl;
-  }
-  return (l << h) | r;
-}
-
-// Position k of the permutation of [0, n) drawn by `key` (n >= 1).  The walk stays on k's cycle of the
-// Feistel permutation, which holds k itself, so it returns a value below n; the bound only guards the loop.
-__device__ __forceinline__ uint64_t perm_index(uint64_t k, uint64_t n, int h, uint64_t key) {
-  uint64_t x = k;
-  for (int i = 0; i < (1 << 20); ++i) {
-    x = feistel(x, h, key);
-    if (x < n) return x;
-  }
-  return k;
 }
 
 // Row i of the batch = sample perm(first + i): X (128 bytes), T (32) and G (48) copied with 16-byte loads
@@ -1602,35 +1111,6 @@ cudaError_t launch_mlp_accumulate(float* dst, const float* src, float w, cudaStr
   return cudaGetLastError();
 }
 
-cudaError_t launch_mlp_tile_weights(const __nv_bfloat16* wb, __nv_bfloat16* wt, cudaStream_t stream) {
-  mlp_tile_weights_kernel<<<128, 256, 0, stream>>>(wb, wt);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_mlp_infer(const SceneDev& S, const BatchDev& B, int n, const PathRec* list, uint64_t count,
-                             float inv_scale, const __nv_bfloat16* wt, const float* params, float* T, int* err,
-                             cudaStream_t stream, int n_sm) {
-  if (!count) return cudaSuccess;
-  static bool attr = false;
-  const int smem = (int)sizeof(InferSmem);
-  if (!attr) {
-    for (auto k : {mlp_infer_kernel<kSrcEnum>, mlp_infer_kernel<kSrcRec>, mlp_infer_kernel<kSrcRecDecode>}) {
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e != cudaSuccess) return e;
-    }
-    attr = true;
-  }
-  const uint64_t tiles = (count + 127) / 128;
-  const uint64_t cap = (uint64_t)n_sm * kInferCtasPerSm;
-  const unsigned grid = (unsigned)(tiles < cap ? tiles : cap);
-  auto kern = list == nullptr ? mlp_infer_kernel<kSrcEnum>
-                              : (n > kMaxBfgsOrder ? mlp_infer_kernel<kSrcRecDecode> : mlp_infer_kernel<kSrcRec>);
-  kern<<<grid, kInferThreads, smem, stream>>>(S, B, n, list, count, inv_scale, wt, params, T, err);
-  count_launch();
-  return cudaGetLastError();
-}
-
 static unsigned grid_1d(uint64_t n, int threads, int cap) {
   uint64_t g = (n + threads - 1) / threads;
   return (unsigned)(g < (uint64_t)cap ? (g ? g : 1) : (uint64_t)cap);
@@ -1686,6 +1166,12 @@ cudaError_t launch_bf16_transpose(const __nv_bfloat16* src, int R, int C, __nv_b
 
 cudaError_t launch_mlp_transpose_weights(const __nv_bfloat16* wb, __nv_bfloat16* wt, cudaStream_t stream) {
   mlp_transpose_weights_kernel<<<264, 512, 0, stream>>>(wb, wt);
+  count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_mlp_tile_weights(const __nv_bfloat16* wb, __nv_bfloat16* wt, cudaStream_t stream) {
+  mlp_tile_weights_kernel<<<(kMlpParams + 255) / 256, 256, 0, stream>>>(wb, wt);
   count_launch();
   return cudaGetLastError();
 }

@@ -54,11 +54,20 @@ cudaError_t launch_colsum(const float* A, uint64_t B, int N, float* out, cudaStr
 cudaError_t launch_adam(float* w, float* m, float* v, const float* g, int n, float lr, float c1, float c2,
                         __nv_bfloat16* wb, cudaStream_t stream);
 cudaError_t launch_to_bf16(const float* src, __nv_bfloat16* dst, int n, cudaStream_t stream);
-constexpr size_t kMlpTiledBytes = 9 * 32768 + 4 * 2048;  // weights pre-tiled for the fused inference
+// The weights as the fused kernels' CTA pairs read them (k_infer.cu, k_train.cu): CTA r of a pair holds outputs
+// 128 r .. 128 r + 127 of the hidden layers in chunks of 64 inputs, and the whole output layer; transposed, for the
+// back-propagation, inputs 128 r .. 128 r + 127.  Every piece is K-major in core matrices (tc.cuh).
+constexpr uint32_t kMlpChunk = 128 * 64 * 2;   // 128 rows x 64 columns
+constexpr uint32_t kMlpW4Chunk = 16 * 64 * 2;  // the output layer's 16 rows
+constexpr uint32_t kMlpTileW2 = kMlpChunk, kMlpTileW3 = 5 * kMlpChunk, kMlpTileW4 = 9 * kMlpChunk;
+constexpr uint32_t kMlpHalfBytes = 9 * kMlpChunk + 4 * kMlpW4Chunk;
 cudaError_t launch_mlp_tile_weights(const __nv_bfloat16* wb, __nv_bfloat16* wt, cudaStream_t stream);
+// The learned start of `count` paths: of order n of an exhaustive batch (list == nullptr), or of a list of
+// records, all of orders up to kMaxBfgsOrder (n any of them) or all above (n > kMaxBfgsOrder).  Slots from a
+// path's order to n_fill are set to zero.
 cudaError_t launch_mlp_infer(const SceneDev& S, const BatchDev& B, int n, const PathRec* list, uint64_t count,
-                             float inv_scale, const __nv_bfloat16* wt, const float* params, float* T, int* err,
-                             cudaStream_t stream, int n_sm);
+                             float inv_scale, const __nv_bfloat16* wt, const float* params, float* T, int n_fill,
+                             int* err, cudaStream_t stream, int n_sm);
 // Rows perm(first .. first + B - 1) of (X [n][64], T [n][8], G [n][12]) into (Xb, Tb, Gb), perm = the
 // seeded permutation of [0, n) drawn by key.
 cudaError_t launch_mlp_gather(const __nv_bfloat16* X, const float* T, const float* G, uint64_t n, uint64_t first,
