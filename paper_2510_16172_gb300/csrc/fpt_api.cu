@@ -180,30 +180,21 @@ struct fpt_mlp {
   float* d_v = nullptr;
   float* d_g = nullptr;          // gradient
   __nv_bfloat16* d_wb = nullptr;  // BF16 copy used by the tensor cores
-  __nv_bfloat16* d_wt = nullptr;  // BF16 weights pre-tiled for the fused inference kernel
+  __nv_bfloat16* d_wt = nullptr;   // the weights as the fused kernels read them (mlp.h),
+  __nv_bfloat16* d_wtT = nullptr;  // and their transposes; both brought up to date when stale
   bool wt_stale = true;
-  __nv_bfloat16* d_wtT = nullptr;  // BF16 W^T of layers 2-4 (the backward's dH = dZ W), refreshed when stale
-  bool wtT_stale = true;
-  float* d_loss = nullptr;
-  // fpt_mlp_train: one shuffled mini-batch and the per-epoch mean losses
-  __nv_bfloat16* d_Xb = nullptr;
-  float *d_Tb = nullptr, *d_Gb = nullptr, *d_hist = nullptr;
-  uint64_t train_cap = 0;
-  bool xt_ready = false;  // d_Xt already holds the transpose of d_Xb (written by the shuffle gather)
+  float* d_loss = nullptr;       // the batch's loss, behind the gradient (cleared with it)
+  float* d_hist = nullptr;       // fpt_mlp_train: per-epoch mean losses
   size_t hist_cap = 0;
-  // activations / gradients for a batch of up to cap rows
+  // forward activations and outputs for up to cap rows
   uint64_t cap = 0;
-  __nv_bfloat16 *d_H1 = nullptr, *d_H2 = nullptr, *d_H3 = nullptr, *d_dZa = nullptr, *d_dZb = nullptr,
-                *d_dYb = nullptr, *d_X = nullptr;
-  // transposed copies for the weight gradients dW = dZ^T act (K-major operands): act^T, dZ^T, dY^T
-  __nv_bfloat16 *d_Ht1 = nullptr, *d_Ht2 = nullptr, *d_Ht3 = nullptr, *d_Xt = nullptr, *d_dZta = nullptr,
-                *d_dZtb = nullptr, *d_dYt = nullptr;
-  float *d_Z1 = nullptr, *d_Z2 = nullptr, *d_Z3 = nullptr, *d_Y = nullptr, *d_dY = nullptr;
+  __nv_bfloat16 *d_H1 = nullptr, *d_H2 = nullptr;
+  // transposed operands of the weight gradients dW = dZ^T act for up to train_cap rows
+  uint64_t train_cap = 0;
+  __nv_bfloat16 *d_Ht = nullptr, *d_dZt = nullptr, *d_dYt = nullptr, *d_Xt = nullptr;
 };
 
-static fpt_status mlp_ensure_ws(fpt_ctx* ctx, fpt_mlp* m, uint64_t B, bool train);
-static fpt_status mlp_forward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16* X, uint64_t B, float* Y,
-                                   bool train);
+static fpt_status mlp_tiled_weights(fpt_ctx* ctx, fpt_mlp* m);
 
 static SceneDev scene_dev(const fpt_scene* s) {
   SceneDev d{};
@@ -1114,10 +1105,7 @@ static fpt_status solve_impl(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* 
     if (X) CUDA_OR_FAIL(ctx, cudaMemsetAsync(X, 0, b->dev.n_paths * (uint64_t)b->dev.n_max * 3 * sizeof(float), ctx->stream));
   }
   fpt_mlp* m = p.init_mode == 1 ? ctx->init_mlp : nullptr;
-  if (m && plan.count && m->wt_stale) {
-    CUDA_OR_FAIL(ctx, launch_mlp_tile_weights(m->d_wb, m->d_wt, ctx->stream));
-    m->wt_stale = false;
-  }
+  if (m && plan.count && (st = mlp_tiled_weights(ctx, m)) != FPT_OK) return st;
   CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_ctl, 0, kCtlBytes, ctx->stream));
   return run_orders(ctx, plan, [&](const OrderRun& r) -> fpt_status {
     if (m) {
@@ -1396,51 +1384,47 @@ fpt_status fpt_count_status(fpt_ctx* ctx, const uint8_t* status, uint64_t n, uin
 // learned warm start
 // ---------------------------------------------------------------------------
 static void mlp_free_ws(fpt_mlp* m) {
-  for (void* p : {(void*)m->d_H1, (void*)m->d_H2, (void*)m->d_H3, (void*)m->d_dZa, (void*)m->d_dZb, (void*)m->d_dYb,
-                  (void*)m->d_X, (void*)m->d_Z1, (void*)m->d_Z2, (void*)m->d_Z3, (void*)m->d_Y,
-                  (void*)m->d_dY, (void*)m->d_Ht1, (void*)m->d_Ht2, (void*)m->d_Ht3, (void*)m->d_Xt, (void*)m->d_dZta,
-                  (void*)m->d_dZtb, (void*)m->d_dYt})
-    cudaFree(p);
-  m->d_H1 = m->d_H2 = m->d_H3 = m->d_dZa = m->d_dZb = m->d_dYb = m->d_X = nullptr;
-  m->d_Ht1 = m->d_Ht2 = m->d_Ht3 = m->d_Xt = m->d_dZta = m->d_dZtb = m->d_dYt = nullptr;
-  m->d_Z1 = m->d_Z2 = m->d_Z3 = m->d_Y = m->d_dY = nullptr;
-  m->cap = 0;
+  for (__nv_bfloat16** p : {&m->d_H1, &m->d_H2, &m->d_Ht, &m->d_dZt, &m->d_dYt, &m->d_Xt}) {
+    cudaFree(*p);
+    *p = nullptr;
+  }
+  m->cap = m->train_cap = 0;
 }
 
+// Buffers for B rows of a forward pass, or of a training batch.
 static fpt_status mlp_ensure_ws(fpt_ctx* ctx, fpt_mlp* m, uint64_t B, bool train) {
   const uint64_t want = B < 128 ? 128 : B;
-  if (want <= m->cap && (!train || m->d_Z1)) return FPT_OK;
-  mlp_free_ws(m);
-  const size_t H = want * kMlpHidden;
+  if (want <= (train ? m->train_cap : m->cap)) return FPT_OK;
   cudaError_t e = cudaSuccess;
-  auto bf = [&](__nv_bfloat16** p, size_t n) { if (e == cudaSuccess) e = cudaMalloc(p, n * sizeof(__nv_bfloat16)); };
-  auto f32 = [&](float** p, size_t n) { if (e == cudaSuccess) e = cudaMalloc(p, n * sizeof(float)); };
-  bf(&m->d_H1, H);
-  bf(&m->d_H2, H);
-  bf(&m->d_H3, H);
-  bf(&m->d_X, want * kMlpIn);
-  f32(&m->d_Y, want * kMlpOut);
+  auto bf = [&](__nv_bfloat16** p, size_t n) {
+    cudaFree(*p);
+    *p = nullptr;
+    if (e == cudaSuccess) e = cudaMalloc(p, n * sizeof(__nv_bfloat16));
+  };
+  const size_t H = want * kMlpHidden;
   if (train) {
-    f32(&m->d_Z1, H);
-    f32(&m->d_Z2, H);
-    f32(&m->d_Z3, H);
-    bf(&m->d_dZa, H);
-    bf(&m->d_dZb, H);
-    bf(&m->d_dYb, want * kMlpOut);
-    f32(&m->d_dY, want * kMlpOut);
-    bf(&m->d_Ht1, H);
-    bf(&m->d_Ht2, H);
-    bf(&m->d_Ht3, H);
-    bf(&m->d_Xt, want * kMlpIn);
-    bf(&m->d_dZta, H);
-    bf(&m->d_dZtb, H);
+    m->train_cap = 0;
+    bf(&m->d_Ht, 3 * H);
+    bf(&m->d_dZt, 3 * H);
     bf(&m->d_dYt, want * kMlpOut);
+    bf(&m->d_Xt, want * kMlpIn);
+  } else {
+    m->cap = 0;
+    bf(&m->d_H1, H);
+    bf(&m->d_H2, H);
   }
   if (e != cudaSuccess) {
     mlp_free_ws(m);
     return fail(ctx, FPT_ENOMEM, "MLP workspace for %llu rows: %s", (unsigned long long)want, cudaGetErrorString(e));
   }
-  m->cap = want;
+  (train ? m->train_cap : m->cap) = want;
+  return FPT_OK;
+}
+
+static fpt_status mlp_tiled_weights(fpt_ctx* ctx, fpt_mlp* m) {
+  if (!m->wt_stale) return FPT_OK;
+  CUDA_OR_FAIL(ctx, launch_mlp_tile_weights(m->d_wb, m->d_wt, m->d_wtT, ctx->stream));
+  m->wt_stale = false;
   return FPT_OK;
 }
 
@@ -1461,32 +1445,21 @@ static GemmArgs gemm_args(int M, int N, int K, const __nv_bfloat16* A, long long
   return g;
 }
 
-// forward pass of B rows of X; with `train`, keeps gelu' at each hidden layer's pre-activation (Z1..Z3)
-static fpt_status mlp_forward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16* X, uint64_t B, float* Y,
-                                   bool train) {
+// forward pass of B rows of X
+static fpt_status mlp_forward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16* X, uint64_t B, float* Y) {
   const int Bi = (int)B;
   const __nv_bfloat16* W = m->d_wb;
   const float* P = m->d_w;
   const __nv_bfloat16* in = X;
-  __nv_bfloat16* H[3] = {m->d_H1, m->d_H2, m->d_H3};
-  float* Z[3] = {m->d_Z1, m->d_Z2, m->d_Z3};
+  __nv_bfloat16* H[3] = {m->d_H1, m->d_H2, m->d_H1};
   const int offW[3] = {kOffW1, kOffW2, kOffW3}, offB[3] = {kOffB1, kOffB2, kOffB3};
   for (int l = 0; l < 3; ++l) {
     const int K = l == 0 ? kMlpIn : kMlpHidden;
     GemmArgs g = gemm_args(Bi, kMlpHidden, K, in, K, 1, W + offW[l], K, 1, EPI_BIAS_GELU, ctx->d_err);
     g.bias = P + offB[l];
-    g.C = train ? Z[l] : nullptr;
-    g.scm = kMlpHidden;
-    g.scn = 1;
     g.H = H[l];
     g.shm = kMlpHidden;
     g.shn = 1;
-    if (train) {  // H^T [256][B]: the K-major operand of the next layer's weight gradient
-      __nv_bfloat16* Ht[3] = {m->d_Ht1, m->d_Ht2, m->d_Ht3};
-      g.Ht = Ht[l];
-      g.shtm = 1;
-      g.shtn = Bi;
-    }
     CUDA_OR_FAIL(ctx, launch_gemm(g, 1, ctx->stream));
     in = H[l];
   }
@@ -1499,9 +1472,6 @@ static fpt_status mlp_forward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16
   return FPT_OK;
 }
 
-// loss and gradient (into m->d_g) of a batch; loss accumulated in m->d_loss.  Every GEMM reads K-major
-// operands: the weight gradients dW = dZ^T act take the transposed copies written by the epilogues, the
-// back-propagation dH = dZ W the transposed BF16 weights.
 static int split_k(const fpt_ctx* ctx, int B, int m_tiles) {
   // one (row tile, K split) item per SM (each CTA adds one partial product into the gradient), at least
   // four 64-wide K chunks per split
@@ -1513,81 +1483,76 @@ static int split_k(const fpt_ctx* ctx, int B, int m_tiles) {
   return (B + per - 1) / per;
 }
 
+// Loss and gradient (d_loss, d_g) of a batch: one launch for the forward pass, the loss and the back-propagation, then
+// the weight gradients from its transposed operands.  These are independent and fill 64 SMs each, so they run side by
+// side on the context's order streams.  n > 0: row i is sample perm(first + i) of n (fpt_mlp_train).
 static fpt_status mlp_backward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16* X, const float* T, const float* G,
-                                    uint64_t B) {
+                                    uint64_t B, uint64_t n, uint64_t first, uint64_t key) {
   const int Bi = (int)B;
-  CUDA_OR_FAIL(ctx, cudaMemsetAsync(m->d_g, 0, kMlpParams * sizeof(float), ctx->stream));
-  CUDA_OR_FAIL(ctx, cudaMemsetAsync(m->d_loss, 0, sizeof(float), ctx->stream));
-  if (m->wtT_stale) {
-    CUDA_OR_FAIL(ctx, launch_mlp_transpose_weights(m->d_wb, m->d_wtT, ctx->stream));
-    m->wtT_stale = false;
-  }
-  const __nv_bfloat16* Wt2 = m->d_wtT;
-  const __nv_bfloat16* Wt3 = m->d_wtT + 256 * 256;
-  const __nv_bfloat16* Wt4 = m->d_wtT + 2 * 256 * 256;
-  // weight gradients: K (the batch) split into one slice per SM's item; each slice's partial product is
-  // added into m->d_g (zeroed above) by the GEMM's epilogue (TMA reduce-add, else atomics)
+  fpt_status st = mlp_ensure_ws(ctx, m, B, true);
+  if (st == FPT_OK) st = mlp_tiled_weights(ctx, m);
+  if (st != FPT_OK) return st;
+  CUDA_OR_FAIL(ctx, cudaMemsetAsync(m->d_g, 0, (kMlpParams + 1) * sizeof(float), ctx->stream));
+  TrainArgs a{};
+  a.X = X;
+  a.T = T;
+  a.G = G;
+  a.B = B;
+  a.n = n;
+  a.first = first;
+  a.key = key;
+  a.wt = m->d_wt;
+  a.wtT = m->d_wtT;
+  a.params = m->d_w;
+  a.Xt = m->d_Xt;
+  a.Ht = m->d_Ht;
+  a.dZt = m->d_dZt;
+  a.dYt = m->d_dYt;
+  a.grad = m->d_g;
+  a.loss = m->d_loss;
+  a.err = ctx->d_err;
+  CUDA_OR_FAIL(ctx, launch_mlp_train(a, ctx->stream, ctx->n_sm));
+  // dW_l [out][in] = dZ_l^T [out][b] act^T [in][b]; dW4^T [in][out] = H3^T dY.  K (the batch) is split into one slice
+  // per SM's item; each slice's partial product is added into d_g (TMA reduce-add, else atomics).
   const int ks = split_k(ctx, Bi, 2);
-  auto weight_grad = [&](int M, int N, const __nv_bfloat16* At, const __nv_bfloat16* Bt, float* dst, long long scm,
-                         long long scn) -> fpt_status {
-    GemmArgs g = gemm_args(M, N, Bi, At, Bi, 1, Bt, Bi, 1, EPI_ATOMIC, ctx->d_err);
-    g.C = dst;
-    g.scm = scm;
-    g.scn = scn;
-    CUDA_OR_FAIL(ctx, launch_gemm(g, ks, ctx->stream));
-    return FPT_OK;
+  const size_t H = (size_t)kMlpHidden * B;
+  struct Grad {
+    int N;
+    const __nv_bfloat16 *At, *Bt;
+    float* dst;
+    long long scm, scn;
   };
-  fpt_status st = mlp_forward_impl(ctx, m, X, B, m->d_Y, true);
-  if (st != FPT_OK) return st;
-  if (!(m->xt_ready && X == m->d_Xb)) CUDA_OR_FAIL(ctx, launch_bf16_transpose(X, Bi, kMlpIn, m->d_Xt, ctx->stream));
-  CUDA_OR_FAIL(ctx, launch_mlp_loss(G, m->d_Y, T, B, m->d_dY, m->d_dYb, m->d_dYt, m->d_loss, ctx->stream));
-  // last layer: dW4^T [in][out] = H3^T dY (sum over the batch); db4 = sum_b dY
-  st = weight_grad(kMlpHidden, kMlpOut, m->d_Ht3, m->d_dYt, m->d_g + kOffW4, 1, kMlpHidden);
-  if (st != FPT_OK) return st;
-  CUDA_OR_FAIL(ctx, launch_colsum(m->d_dY, B, kMlpOut, m->d_g + kOffB4, ctx->stream));
-  // dZ3 = (dY W4) * gelu'(Z3), its transpose, and db3 = sum_b dZ3 (column sums in the epilogue)
-  {
-    GemmArgs g = gemm_args(Bi, kMlpHidden, kMlpOut, m->d_dYb, kMlpOut, 1, Wt4, kMlpOut, 1, EPI_GELU_GRAD, ctx->d_err);
-    g.Zin = m->d_Z3;
-    g.szm = kMlpHidden;
-    g.szn = 1;
-    g.colsum = m->d_g + kOffB3;
-    g.H = m->d_dZa;
-    g.shm = kMlpHidden;
-    g.shn = 1;
-    g.Ht = m->d_dZta;
-    g.shtm = 1;
-    g.shtn = Bi;
-    CUDA_OR_FAIL(ctx, launch_gemm(g, 1, ctx->stream));
+  const Grad grads[4] = {{kMlpHidden, m->d_dZt + 2 * H, m->d_Ht + H, m->d_g + kOffW3, kMlpHidden, 1},
+                         {kMlpHidden, m->d_dZt + H, m->d_Ht, m->d_g + kOffW2, kMlpHidden, 1},
+                         {kMlpIn, m->d_dZt, m->d_Xt, m->d_g + kOffW1, kMlpIn, 1},
+                         {kMlpOut, m->d_Ht + 2 * H, m->d_dYt, m->d_g + kOffW4, 1, kMlpHidden}};
+  static_assert(fpt_ctx::kOrderStreams >= 3, "streams of the weight gradients");
+  CUDA_OR_FAIL(ctx, cudaEventRecord(ctx->ofork_ev, ctx->stream));
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < 4; ++k) {
+    const cudaStream_t s = k == 0 ? ctx->stream : ctx->ostream[k - 1];
+    if (k > 0 && e == cudaSuccess) e = cudaStreamWaitEvent(s, ctx->ofork_ev, 0);
+    GemmArgs g = gemm_args(kMlpHidden, grads[k].N, Bi, grads[k].At, Bi, 1, grads[k].Bt, Bi, 1, EPI_ATOMIC, ctx->d_err);
+    g.C = grads[k].dst;
+    g.scm = grads[k].scm;
+    g.scn = grads[k].scn;
+    if (e == cudaSuccess) e = launch_gemm(g, ks, s);
   }
-  const __nv_bfloat16* acts_t[3] = {m->d_Xt, m->d_Ht1, m->d_Ht2};  // inputs of layers 1..3, transposed
-  const __nv_bfloat16* wts[3] = {nullptr, Wt2, Wt3};
-  const float* Zs[2] = {m->d_Z1, m->d_Z2};
-  const int offW[3] = {kOffW1, kOffW2, kOffW3}, offB[3] = {kOffB1, kOffB2, kOffB3};
-  __nv_bfloat16 *dZ = m->d_dZa, *dZn = m->d_dZb, *dZt = m->d_dZta, *dZtn = m->d_dZtb;
-  for (int l = 2; l >= 0; --l) {
-    const int K_in = l == 0 ? kMlpIn : kMlpHidden;
-    // dW_l [out][in] = dZ^T [out][b] act^T [in][b]
-    st = weight_grad(kMlpHidden, K_in, dZt, acts_t[l], m->d_g + offW[l], K_in, 1);
-    if (st != FPT_OK) return st;
-    if (l == 0) break;
-    // dZ_{l-1} = (dZ_l W_l) * gelu'(Z_{l-1}) = dZ_l [b][out] (W_l^T)[in][out], its transpose and db_{l-1}
-    GemmArgs gd = gemm_args(Bi, kMlpHidden, kMlpHidden, dZ, kMlpHidden, 1, wts[l], kMlpHidden, 1, EPI_GELU_GRAD,
-                            ctx->d_err);
-    gd.Zin = Zs[l - 1];
-    gd.szm = kMlpHidden;
-    gd.szn = 1;
-    gd.colsum = m->d_g + offB[l - 1];
-    gd.H = dZn;
-    gd.shm = kMlpHidden;
-    gd.shn = 1;
-    gd.Ht = dZtn;
-    gd.shtm = 1;
-    gd.shtn = Bi;
-    CUDA_OR_FAIL(ctx, launch_gemm(gd, 1, ctx->stream));
-    std::swap(dZ, dZn);
-    std::swap(dZt, dZtn);
+  for (int k = 0; k < 3; ++k) {  // joined also after an error (a stream capture must end joined)
+    const cudaError_t f = cudaEventRecord(ctx->ojoin_ev[k], ctx->ostream[k]);
+    const cudaError_t w = f == cudaSuccess ? cudaStreamWaitEvent(ctx->stream, ctx->ojoin_ev[k], 0) : f;
+    if (e == cudaSuccess) e = w;
   }
+  CUDA_OR_FAIL(ctx, e);
+  return FPT_OK;
+}
+
+// Adam step on d_g; with hist, also *hist += hist_w * the batch's loss.
+static fpt_status mlp_adam(fpt_ctx* ctx, fpt_mlp* m, float lr, float* hist, float hist_w) {
+  m->step += 1;
+  const float c1 = 1.f - std::pow(0.9f, (float)m->step), c2 = 1.f - std::pow(0.999f, (float)m->step);
+  CUDA_OR_FAIL(ctx, launch_adam(m->d_w, m->d_m, m->d_v, m->d_g, lr, c1, c2, m->d_wb, m->d_wt, m->d_wtT, m->d_loss, hist,
+                                hist_w, ctx->stream));
   return FPT_OK;
 }
 
@@ -1612,11 +1577,11 @@ fpt_status fpt_mlp_create(fpt_ctx* ctx, uint64_t seed, float length_scale, fpt_m
   m->seed = seed;
   cudaError_t e = cudaSetDevice(ctx->device);
   for (float** p : {&m->d_w, &m->d_m, &m->d_v, &m->d_g})
-    if (e == cudaSuccess) e = cudaMalloc(p, kMlpParams * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(p, (kMlpParams + 1) * sizeof(float));
+  m->d_loss = m->d_g + kMlpParams;
   if (e == cudaSuccess) e = cudaMalloc(&m->d_wb, kMlpParams * sizeof(__nv_bfloat16));
   if (e == cudaSuccess) e = cudaMalloc(&m->d_wt, 2 * kMlpHalfBytes);
-  if (e == cudaSuccess) e = cudaMalloc(&m->d_wtT, kMlpWtElems * sizeof(__nv_bfloat16));
-  if (e == cudaSuccess) e = cudaMalloc(&m->d_loss, sizeof(float));
+  if (e == cudaSuccess) e = cudaMalloc(&m->d_wtT, 2 * kMlpHalfTBytes);
   if (e != cudaSuccess) {
     fpt_mlp_free(m);
     return fail(ctx, FPT_ENOMEM, "MLP parameters: %s", cudaGetErrorString(e));
@@ -1649,7 +1614,7 @@ void fpt_mlp_free(fpt_mlp* m) {
   if (m->ctx && m->ctx->init_mlp == m) m->ctx->init_mlp = nullptr;
   mlp_free_ws(m);
   for (void* p : {(void*)m->d_w, (void*)m->d_m, (void*)m->d_v, (void*)m->d_g, (void*)m->d_wb, (void*)m->d_wt,
-                  (void*)m->d_loss, (void*)m->d_Xb, (void*)m->d_Tb, (void*)m->d_Gb, (void*)m->d_hist, (void*)m->d_wtT})
+                  (void*)m->d_wtT, (void*)m->d_hist})
     cudaFree(p);
   delete m;
 }
@@ -1677,7 +1642,6 @@ fpt_status fpt_mlp_set_params(fpt_mlp* m, const float* host) {
   CUDA_OR_FAIL(ctx, cudaStreamSynchronize(ctx->stream));
   m->step = 0;
   m->wt_stale = true;
-  m->wtT_stale = true;
   return FPT_OK;
 }
 
@@ -1756,7 +1720,7 @@ fpt_status fpt_mlp_forward(fpt_ctx* ctx, fpt_mlp* m, const void* X, uint64_t B, 
   fpt_status st = mlp_ensure_ws(ctx, m, B, false);
   if (st != FPT_OK) return st;
   ProfScope ps(ctx, FPT_K_OTHER);
-  return mlp_forward_impl(ctx, m, static_cast<const __nv_bfloat16*>(X), B, Y, false);
+  return mlp_forward_impl(ctx, m, static_cast<const __nv_bfloat16*>(X), B, Y);
 }
 
 fpt_status fpt_mlp_loss_grad(fpt_ctx* ctx, fpt_mlp* m, const void* X, const float* T, const float* G, uint64_t B,
@@ -1764,9 +1728,7 @@ fpt_status fpt_mlp_loss_grad(fpt_ctx* ctx, fpt_mlp* m, const void* X, const floa
   if (!ctx || !m || !X || !T || !G) return fail(ctx, FPT_EINVAL, "null argument");
   if (B < 1 || B > (1ull << 30)) return fail(ctx, FPT_EINVAL, "bad batch size");
   CUDA_OR_FAIL(ctx, cudaSetDevice(ctx->device));
-  fpt_status st = mlp_ensure_ws(ctx, m, B, true);
-  if (st != FPT_OK) return st;
-  st = mlp_backward_impl(ctx, m, static_cast<const __nv_bfloat16*>(X), T, G, B);
+  fpt_status st = mlp_backward_impl(ctx, m, static_cast<const __nv_bfloat16*>(X), T, G, B, 0, 0, 0);
   if (st != FPT_OK) return st;
   if (grad_out)
     CUDA_OR_FAIL(ctx, cudaMemcpyAsync(grad_out, m->d_g, kMlpParams * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
@@ -1781,12 +1743,8 @@ fpt_status fpt_mlp_train_step(fpt_ctx* ctx, fpt_mlp* m, const void* X, const flo
                               float lr, float* loss) {
   if (!(lr > 0.f)) return fail(ctx, FPT_EINVAL, "learning rate must be positive");
   fpt_status st = fpt_mlp_loss_grad(ctx, m, X, T, G, B, nullptr, nullptr);
+  if (st == FPT_OK) st = mlp_adam(ctx, m, lr, nullptr, 0.f);
   if (st != FPT_OK) return st;
-  m->step += 1;
-  const float c1 = 1.f - std::pow(0.9f, (float)m->step), c2 = 1.f - std::pow(0.999f, (float)m->step);
-  CUDA_OR_FAIL(ctx, launch_adam(m->d_w, m->d_m, m->d_v, m->d_g, kMlpParams, lr, c1, c2, m->d_wb, ctx->stream));
-  m->wt_stale = true;
-  m->wtT_stale = true;
   if (loss) {
     CUDA_OR_FAIL(ctx, cudaMemcpyAsync(loss, m->d_loss, sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
     CUDA_OR_FAIL(ctx, cudaStreamSynchronize(ctx->stream));
@@ -1806,22 +1764,12 @@ fpt_status fpt_mlp_train(fpt_ctx* ctx, fpt_mlp* m, const void* X, const float* T
   if (!X || !T || !G) return fail(ctx, FPT_EINVAL, "fpt_mlp_train: X, T and G are required");
   CUDA_OR_FAIL(ctx, cudaSetDevice(ctx->device));
   const uint64_t B = (uint64_t)p.batch;
-  fpt_status st = mlp_ensure_ws(ctx, m, B, true);
-  if (st != FPT_OK) return st;
-  if (B > m->train_cap || (size_t)p.epochs > m->hist_cap) {
-    cudaFree(m->d_Xb);
-    cudaFree(m->d_Tb);
-    cudaFree(m->d_Gb);
+  if ((size_t)p.epochs > m->hist_cap) {
     cudaFree(m->d_hist);
-    m->d_Xb = nullptr;
-    m->d_Tb = m->d_Gb = m->d_hist = nullptr;
-    m->train_cap = m->hist_cap = 0;
-    cudaError_t e = cudaMalloc(&m->d_Xb, B * kMlpIn * sizeof(__nv_bfloat16));
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_Tb, B * 8 * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_Gb, B * 12 * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_hist, (size_t)p.epochs * sizeof(float));
-    if (e != cudaSuccess) return fail(ctx, FPT_ENOMEM, "fpt_mlp_train: batch buffers: %s", cudaGetErrorString(e));
-    m->train_cap = B;
+    m->d_hist = nullptr;
+    m->hist_cap = 0;
+    const cudaError_t e = cudaMalloc(&m->d_hist, (size_t)p.epochs * sizeof(float));
+    if (e != cudaSuccess) return fail(ctx, FPT_ENOMEM, "fpt_mlp_train: losses: %s", cudaGetErrorString(e));
     m->hist_cap = (size_t)p.epochs;
   }
   CUDA_OR_FAIL(ctx, cudaMemsetAsync(m->d_hist, 0, (size_t)p.epochs * sizeof(float), ctx->stream));
@@ -1833,13 +1781,9 @@ fpt_status fpt_mlp_train(fpt_ctx* ctx, fpt_mlp* m, const void* X, const float* T
     uint64_t s0 = p.seed + 0x9E3779B97F4A7C15ULL * (uint64_t)(ep + 1);
     const uint64_t key = sm64_next(s0);
     for (uint64_t k = 0; k < steps; ++k) {
-      CUDA_OR_FAIL(ctx, launch_mlp_gather(Xs, T, G, n, k * B, B, key, m->d_Xb, m->d_Tb, m->d_Gb, m->d_Xt,
-                                          ctx->stream));
-      m->xt_ready = true;
-      st = fpt_mlp_train_step(ctx, m, m->d_Xb, m->d_Tb, m->d_Gb, B, lr, nullptr);
-      m->xt_ready = false;
+      fpt_status st = mlp_backward_impl(ctx, m, Xs, T, G, B, n, k * B, key);
+      if (st == FPT_OK) st = mlp_adam(ctx, m, lr, m->d_hist + ep, 1.f / (float)steps);
       if (st != FPT_OK) return st;
-      CUDA_OR_FAIL(ctx, launch_mlp_accumulate(m->d_hist + ep, m->d_loss, 1.f / (float)steps, ctx->stream));
     }
     lr *= p.lr_decay;
   }
@@ -1863,10 +1807,8 @@ fpt_status fpt_mlp_infer(fpt_ctx* ctx, fpt_mlp* m, const fpt_scene* s, const fpt
   if (st != FPT_OK) return st;
   const SceneDev S = scene_dev(s);
   if (b->dev.n_paths == 0) return FPT_OK;
-  if (m->wt_stale) {
-    CUDA_OR_FAIL(ctx, launch_mlp_tile_weights(m->d_wb, m->d_wt, ctx->stream));
-    m->wt_stale = false;
-  }
+  st = mlp_tiled_weights(ctx, m);
+  if (st != FPT_OK) return st;
   // Records carry their order, and a batch's lists follow the orders: one launch takes all orders whose records
   // hold the ids, one the longer sequences.  The kernel also clears the slots past a path's order.
   const PathRec* first = nullptr;

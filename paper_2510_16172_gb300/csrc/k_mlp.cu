@@ -27,6 +27,7 @@
 namespace fpt {
 
 constexpr int kGemmKC = 64;                  // K per chunk
+
 // Gather rows [r0, r0 + 128) x k [k0, k0 + 64) of a strided bf16 matrix into a
 // 128 x 64 K-major tile (zero outside rows < R, k < K).
 __device__ __forceinline__ void load_tile(unsigned char* tile, const __nv_bfloat16* src, long long s_r, long long s_k,
@@ -858,172 +859,31 @@ __global__ void mlp_features_kernel(SceneDev S, BatchDev B, int n, const PathRec
   }
 }
 
-// loss (1/B) sum_b sum_s dy_s^T G_s dy_s (G_s = A_s^T A_s / S^2 per slot, zero for unused slots) and dY
-// Per sample: d = Y[:8] - T, the Gram-weighted loss sum_s d_s^T G_s d_s and its gradient dY = (2 / B) G d
-// (the padded outputs 8..15 get zero), in FP32, BF16 and transposed BF16.  vec: the rows of G, Y, T and the
-// outputs start on 16-byte boundaries (16-byte loads and stores).
-__global__ void mlp_loss_kernel(const float* __restrict__ G, const float* __restrict__ Y,
-                                const float* __restrict__ T, uint64_t B, float* __restrict__ dY,
-                                __nv_bfloat16* __restrict__ dYb, __nv_bfloat16* __restrict__ dYt, float* loss,
-                                int vec) {
-  float acc = 0.f;
-  const float w = 2.f / (float)B;
-  for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < B; b += (uint64_t)gridDim.x * blockDim.x) {
-    float gm[12], y[8], t[8];
-    if (vec) {
-      const float4* gp = reinterpret_cast<const float4*>(G + b * 12);
-      const float4* yp = reinterpret_cast<const float4*>(Y + b * kMlpOut);
-      const float4* tp = reinterpret_cast<const float4*>(T + b * 8);
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const float4 v = __ldg(gp + q);
-        gm[4 * q] = v.x;
-        gm[4 * q + 1] = v.y;
-        gm[4 * q + 2] = v.z;
-        gm[4 * q + 3] = v.w;
-      }
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const float4 v = yp[q], u = __ldg(tp + q);
-        y[4 * q] = v.x;
-        y[4 * q + 1] = v.y;
-        y[4 * q + 2] = v.z;
-        y[4 * q + 3] = v.w;
-        t[4 * q] = u.x;
-        t[4 * q + 1] = u.y;
-        t[4 * q + 2] = u.z;
-        t[4 * q + 3] = u.w;
-      }
-    } else {
-#pragma unroll
-      for (int q = 0; q < 12; ++q) gm[q] = G[b * 12 + q];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        y[q] = Y[b * kMlpOut + q];
-        t[q] = T[b * 8 + q];
-      }
-    }
-    float g[kMlpOut];
-#pragma unroll
-    for (int k = 0; k < kMlpOut; ++k) g[k] = 0.f;
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      const float g11 = gm[3 * s], g12 = gm[3 * s + 1], g22 = gm[3 * s + 2];
-      const float d0 = y[2 * s] - t[2 * s];
-      const float d1 = y[2 * s + 1] - t[2 * s + 1];
-      const float m0 = g11 * d0 + g12 * d1, m1 = g12 * d0 + g22 * d1;
-      acc += d0 * m0 + d1 * m1;
-      g[2 * s] = w * m0;
-      g[2 * s + 1] = w * m1;
-    }
-    if (vec) {
-      float4* dp = reinterpret_cast<float4*>(dY + b * kMlpOut);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) dp[q] = make_float4(g[4 * q], g[4 * q + 1], g[4 * q + 2], g[4 * q + 3]);
-      uint32_t wv[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const __nv_bfloat162 b2 = __floats2bfloat162_rn(g[2 * q], g[2 * q + 1]);
-        wv[q] = *reinterpret_cast<const uint32_t*>(&b2);
-      }
-      uint4* bp = reinterpret_cast<uint4*>(dYb + b * kMlpOut);
-      bp[0] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-      bp[1] = make_uint4(wv[4], wv[5], wv[6], wv[7]);
-    } else {
-#pragma unroll
-      for (int k = 0; k < kMlpOut; ++k) {
-        dY[b * kMlpOut + k] = g[k];
-        dYb[b * kMlpOut + k] = __float2bfloat16(g[k]);
-      }
-    }
-    if (dYt) {
-#pragma unroll
-      for (int k = 0; k < kMlpOut; ++k) dYt[(uint64_t)k * B + b] = __float2bfloat16(g[k]);
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc / (float)B);
-}
-
-// out[n] += sum_b A[b][n]  (bias gradients), A: [B][N] row-major
-// out[n] += sum_b A[b][n]: each thread one column and a strided set of rows (four sums in flight), then
-// the block's row lanes combined in shared memory and one atomic per column and block.
-__global__ void colsum_kernel(const float* __restrict__ A, uint64_t B, int N, float* out) {
-  __shared__ float part[256];
-  const int n = threadIdx.x % N;
-  const int lanes = blockDim.x / N;
-  const int rl = threadIdx.x / N;
-  const uint64_t step = (uint64_t)gridDim.x * lanes;
-  float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-  uint64_t b = (uint64_t)blockIdx.x * lanes + rl;
-  if (rl < lanes) {
-    for (; b + 3 * step < B; b += 4 * step) {
-      a0 += A[b * N + n];
-      a1 += A[(b + step) * N + n];
-      a2 += A[(b + 2 * step) * N + n];
-      a3 += A[(b + 3 * step) * N + n];
-    }
-    for (; b < B; b += step) a0 += A[b * N + n];
-  }
-  part[threadIdx.x] = rl < lanes ? (a0 + a1) + (a2 + a3) : 0.f;
-  __syncthreads();
-  if (threadIdx.x < N) {
-    float acc = 0.f;
-    for (int r = 0; r < lanes; ++r) acc += part[r * N + threadIdx.x];
-    atomicAdd(out + threadIdx.x, acc);
-  }
-}
-
+// One Adam step; the updated weights' BF16 copies go straight into every layout that reads them, and one thread
+// adds the batch's loss to its epoch's mean.
 __global__ void adam_kernel(float* __restrict__ w, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ g, int n, float lr, float c1, float c2,
-                            __nv_bfloat16* __restrict__ wb) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = 0.9f * m[i] + 0.1f * gi;
-    const float vi = 0.999f * v[i] + 0.001f * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
-    w[i] = wi;
-    wb[i] = __float2bfloat16(wi);
-  }
-}
-
-// dst [C][R] = src [R][C]^T through a 32 x 32 shared-memory tile (both sides coalesced)
-__global__ void bf16_transpose_kernel(const __nv_bfloat16* __restrict__ src, int R, int C,
-                                      __nv_bfloat16* __restrict__ dst) {
-  __shared__ __nv_bfloat16 tile[32][33];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int r = r0 + i, c = c0 + threadIdx.x;
-    if (r < R && c < C) tile[i][threadIdx.x] = src[(long long)r * C + c];
-  }
-  __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int c = c0 + i, r = r0 + threadIdx.x;
-    if (r < R && c < C) dst[(long long)c * R + r] = tile[threadIdx.x][i];
-  }
-}
-
-// W^T of layers 2, 3 (256 x 256) and 4 (16 x 256 -> 256 x 16), back to back in wt
-__global__ void mlp_transpose_weights_kernel(const __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ wt) {
-  const int n2 = 256 * 256, n4 = 16 * 256;
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < 2 * n2 + n4; idx += gridDim.x * blockDim.x) {
-    if (idx < 2 * n2) {
-      const int l = idx / n2, e = idx % n2;  // wt element (in = e / 256, out = e % 256)
-      const int in = e / 256, out = e % 256;
-      wt[idx] = wb[(l == 0 ? kOffW2 : kOffW3) + out * 256 + in];
-    } else {
-      const int e = idx - 2 * n2;  // (in = e / 16, out = e % 16)
-      const int in = e / 16, out = e % 16;
-      wt[idx] = wb[kOffW4 + out * 256 + in];
-    }
-  }
-}
-
-__global__ void mlp_tile_weights_kernel(const __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ wt) {
+                            const float* __restrict__ g, float lr, float c1, float c2, __nv_bfloat16* __restrict__ wb,
+                            __nv_bfloat16* __restrict__ wt, __nv_bfloat16* __restrict__ wtT,
+                            const float* __restrict__ loss, float* hist, float hist_w) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < kMlpParams) tile_weight(i, wb[i], wt);
+  if (i == 0 && hist) *hist += hist_w * *loss;
+  if (i >= kMlpParams) return;
+  const float gi = g[i];
+  const float mi = 0.9f * m[i] + 0.1f * gi;
+  const float vi = 0.999f * v[i] + 0.001f * gi * gi;
+  m[i] = mi;
+  v[i] = vi;
+  const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+  w[i] = wi;
+  const __nv_bfloat16 b = __float2bfloat16(wi);
+  wb[i] = b;
+  tile_weight(i, b, wt, wtT);
+}
+
+__global__ void mlp_tile_weights_kernel(const __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ wt,
+                                        __nv_bfloat16* __restrict__ wtT) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < kMlpParams) tile_weight(i, wb[i], wt, wtT);
 }
 
 __global__ void to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, int n) {
@@ -1045,72 +905,7 @@ __global__ void mlp_start_kernel(SceneDev S, BatchDev B, int n, const PathRec* l
   }
 }
 
-// Row i of the batch = sample perm(first + i): X (128 bytes), T (32) and G (48) copied with 16-byte loads
-// and stores; with Xt, also the transposed features Xt[k][i] (consecutive threads, consecutive i).
-__global__ void mlp_gather_kernel(const __nv_bfloat16* __restrict__ X, const float* __restrict__ T,
-                                  const float* __restrict__ G, uint64_t n, uint64_t first, uint64_t B, int h,
-                                  uint64_t key, __nv_bfloat16* __restrict__ Xb, float* __restrict__ Tb,
-                                  float* __restrict__ Gb, __nv_bfloat16* __restrict__ Xt, int vec_tg) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < B; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t src = perm_index(first + i, n, h, key);
-    const uint4* xs = reinterpret_cast<const uint4*>(X + src * kMlpIn);
-    uint4* xd = reinterpret_cast<uint4*>(Xb + i * kMlpIn);
-    uint4 xv[kMlpIn / 8];
-#pragma unroll
-    for (int q = 0; q < kMlpIn / 8; ++q) xv[q] = __ldg(xs + q);
-    if (vec_tg) {
-      const float4* ts = reinterpret_cast<const float4*>(T + src * 8);
-      const float4* gs = reinterpret_cast<const float4*>(G + src * 12);
-      float4* td = reinterpret_cast<float4*>(Tb + i * 8);
-      float4* gd = reinterpret_cast<float4*>(Gb + i * 12);
-      const float4 t0 = __ldg(ts), t1 = __ldg(ts + 1);
-      const float4 g0 = __ldg(gs), g1 = __ldg(gs + 1), g2 = __ldg(gs + 2);
-      td[0] = t0;
-      td[1] = t1;
-      gd[0] = g0;
-      gd[1] = g1;
-      gd[2] = g2;
-    } else {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) Tb[i * 8 + q] = T[src * 8 + q];
-#pragma unroll
-      for (int q = 0; q < 12; ++q) Gb[i * 12 + q] = G[src * 12 + q];
-    }
-#pragma unroll
-    for (int q = 0; q < kMlpIn / 8; ++q) xd[q] = xv[q];
-    if (Xt) {
-      const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(xv);
-#pragma unroll
-      for (int k = 0; k < kMlpIn; ++k) Xt[(uint64_t)k * B + i] = e[k];
-    }
-  }
-}
-
-// dst += w * src (one value: a batch's loss into its epoch's mean)
-__global__ void mlp_accumulate_kernel(float* dst, const float* src, float w) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) *dst += w * *src;
-}
-
-cudaError_t launch_mlp_gather(const __nv_bfloat16* X, const float* T, const float* G, uint64_t n, uint64_t first,
-                              uint64_t B, uint64_t key, __nv_bfloat16* Xb, float* Tb, float* Gb, __nv_bfloat16* Xt,
-                              cudaStream_t stream) {
-  int h = 1;
-  while ((1ULL << (2 * h)) < n) ++h;
-  const uint64_t want = (B + 255) / 256;
-  auto a16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  const int vec_tg = a16(T) && a16(G) && a16(Tb) && a16(Gb);
-  mlp_gather_kernel<<<(unsigned)(want < 4096 ? (want ? want : 1) : 4096), 256, 0, stream>>>(X, T, G, n, first, B, h,
-                                                                                           key, Xb, Tb, Gb, Xt, vec_tg);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_mlp_accumulate(float* dst, const float* src, float w, cudaStream_t stream) {
-  mlp_accumulate_kernel<<<1, 32, 0, stream>>>(dst, src, w);
-  count_launch();
-  return cudaGetLastError();
-}
-
+// ---------------------------------------------------------------------------
 static unsigned grid_1d(uint64_t n, int threads, int cap) {
   uint64_t g = (n + threads - 1) / threads;
   return (unsigned)(g < (uint64_t)cap ? (g ? g : 1) : (uint64_t)cap);
@@ -1124,54 +919,17 @@ cudaError_t launch_mlp_features(const SceneDev& S, const BatchDev& B, int n, con
   return cudaGetLastError();
 }
 
-cudaError_t launch_mlp_loss(const float* G, const float* Y, const float* T, uint64_t B, float* dY,
-                            __nv_bfloat16* dYb, __nv_bfloat16* dYt, float* loss, cudaStream_t stream) {
-  auto a16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  const int vec = a16(G) && a16(Y) && a16(T) && a16(dY) && a16(dYb);
-  mlp_loss_kernel<<<grid_1d(B, 256, 1024), 256, 0, stream>>>(G, Y, T, B, dY, dYb, dYt, loss, vec);
+cudaError_t launch_adam(float* w, float* m, float* v, const float* g, float lr, float c1, float c2, __nv_bfloat16* wb,
+                        __nv_bfloat16* wt, __nv_bfloat16* wtT, const float* loss, float* hist, float hist_w,
+                        cudaStream_t stream) {
+  adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, stream>>>(w, m, v, g, lr, c1, c2, wb, wt, wtT, loss, hist, hist_w);
   count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_colsum(const float* A, uint64_t B, int N, float* out, cudaStream_t stream) {
-  if (N < 1 || N > 256) return cudaErrorInvalidValue;
-  const int threads = (256 / N) * N;
-  int dev = 0, n_sm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  const uint64_t rows_per_block = (uint64_t)(threads / N) * 16;  // at least 16 rows per thread
-  uint64_t blocks = (B + rows_per_block - 1) / rows_per_block;
-  if (blocks > (uint64_t)(4 * n_sm)) blocks = 4 * n_sm;
-  if (blocks < 1) blocks = 1;
-  colsum_kernel<<<(unsigned)blocks, 256, 0, stream>>>(A, B, N, out);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_adam(float* w, float* m, float* v, const float* g, int n, float lr, float c1, float c2,
-                        __nv_bfloat16* wb, cudaStream_t stream) {
-  adam_kernel<<<grid_1d(n, 256, 1024), 256, 0, stream>>>(w, m, v, g, n, lr, c1, c2, wb);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_bf16_transpose(const __nv_bfloat16* src, int R, int C, __nv_bfloat16* dst, cudaStream_t stream) {
-  if (R < 1 || C < 1) return cudaSuccess;
-  dim3 grid((C + 31) / 32, (R + 31) / 32);
-  bf16_transpose_kernel<<<grid, dim3(32, 8), 0, stream>>>(src, R, C, dst);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_mlp_transpose_weights(const __nv_bfloat16* wb, __nv_bfloat16* wt, cudaStream_t stream) {
-  mlp_transpose_weights_kernel<<<264, 512, 0, stream>>>(wb, wt);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_mlp_tile_weights(const __nv_bfloat16* wb, __nv_bfloat16* wt, cudaStream_t stream) {
-  mlp_tile_weights_kernel<<<(kMlpParams + 255) / 256, 256, 0, stream>>>(wb, wt);
+cudaError_t launch_mlp_tile_weights(const __nv_bfloat16* wb, __nv_bfloat16* wt, __nv_bfloat16* wtT,
+                                    cudaStream_t stream) {
+  mlp_tile_weights_kernel<<<(kMlpParams + 255) / 256, 256, 0, stream>>>(wb, wt, wtT);
   count_launch();
   return cudaGetLastError();
 }

@@ -41,18 +41,13 @@ struct GemmArgs {
 };
 
 cudaError_t launch_gemm(const GemmArgs& g, int k_split, cudaStream_t stream);
-// dst [C][R] = src [R][C]^T (bf16)
-cudaError_t launch_bf16_transpose(const __nv_bfloat16* src, int R, int C, __nv_bfloat16* dst, cudaStream_t stream);
-// The transposed BF16 weights of layers 2-4 (W^T [in][out]) from the BF16 parameter copy.
-constexpr int kMlpWtElems = 256 * 256 + 256 * 256 + 256 * 16;
-cudaError_t launch_mlp_transpose_weights(const __nv_bfloat16* wb, __nv_bfloat16* wt, cudaStream_t stream);
 cudaError_t launch_mlp_features(const SceneDev& S, const BatchDev& B, int n, const PathRec* list, uint64_t first,
                                 uint64_t count, float inv_scale, __nv_bfloat16* X, float* G, cudaStream_t stream);
-cudaError_t launch_mlp_loss(const float* G, const float* Y, const float* T, uint64_t B, float* dY,
-                            __nv_bfloat16* dYb, __nv_bfloat16* dYt, float* loss, cudaStream_t stream);
-cudaError_t launch_colsum(const float* A, uint64_t B, int N, float* out, cudaStream_t stream);
-cudaError_t launch_adam(float* w, float* m, float* v, const float* g, int n, float lr, float c1, float c2,
-                        __nv_bfloat16* wb, cudaStream_t stream);
+// One Adam step, with the BF16 copies of the parameters (plain and as launch_mlp_tile_weights lays them out); with
+// hist, also *hist += hist_w * *loss.
+cudaError_t launch_adam(float* w, float* m, float* v, const float* g, float lr, float c1, float c2, __nv_bfloat16* wb,
+                        __nv_bfloat16* wt, __nv_bfloat16* wtT, const float* loss, float* hist, float hist_w,
+                        cudaStream_t stream);
 cudaError_t launch_to_bf16(const float* src, __nv_bfloat16* dst, int n, cudaStream_t stream);
 // The weights as the fused kernels' CTA pairs read them (k_infer.cu, k_train.cu): CTA r of a pair holds outputs
 // 128 r .. 128 r + 127 of the hidden layers in chunks of 64 inputs, and the whole output layer; transposed, for the
@@ -61,19 +56,34 @@ constexpr uint32_t kMlpChunk = 128 * 64 * 2;   // 128 rows x 64 columns
 constexpr uint32_t kMlpW4Chunk = 16 * 64 * 2;  // the output layer's 16 rows
 constexpr uint32_t kMlpTileW2 = kMlpChunk, kMlpTileW3 = 5 * kMlpChunk, kMlpTileW4 = 9 * kMlpChunk;
 constexpr uint32_t kMlpHalfBytes = 9 * kMlpChunk + 4 * kMlpW4Chunk;
-cudaError_t launch_mlp_tile_weights(const __nv_bfloat16* wb, __nv_bfloat16* wt, cudaStream_t stream);
+constexpr uint32_t kMlpTileW3t = 0, kMlpTileW2t = 4 * kMlpChunk, kMlpTileW4t = 8 * kMlpChunk;
+constexpr uint32_t kMlpHalfTBytes = 8 * kMlpChunk + 128 * 16 * 2;
+// both from the BF16 parameter copy
+cudaError_t launch_mlp_tile_weights(const __nv_bfloat16* wb, __nv_bfloat16* wt, __nv_bfloat16* wtT,
+                                    cudaStream_t stream);
+// Forward pass, loss and back-propagation of B rows.  Row i is sample perm(first + i) of n when n > 0 (perm = the
+// seeded permutation of [0, n) drawn by key), else sample i.  Written: the transposed features [64][B], hidden
+// activations [3][256][B] and gradients at the layers' outputs dZ [3][256][B], dY [16][B]; added: the bias
+// gradients (at their places in grad) and the mean loss.
+struct TrainArgs {
+  const __nv_bfloat16* X;
+  const float* T;
+  const float* G;
+  uint64_t B, n, first, key;
+  const __nv_bfloat16 *wt, *wtT;
+  const float* params;
+  __nv_bfloat16 *Xt, *Ht, *dZt, *dYt;
+  float *grad, *loss;
+  int* err;
+  int h, vec_x, vec_tg;  // set by the launch: half the permutation's bits, 16-byte alignment of X, of T and G
+};
+cudaError_t launch_mlp_train(const TrainArgs& a, cudaStream_t stream, int n_sm);
 // The learned start of `count` paths: of order n of an exhaustive batch (list == nullptr), or of a list of
 // records, all of orders up to kMaxBfgsOrder (n any of them) or all above (n > kMaxBfgsOrder).  Slots from a
 // path's order to n_fill are set to zero.
 cudaError_t launch_mlp_infer(const SceneDev& S, const BatchDev& B, int n, const PathRec* list, uint64_t count,
                              float inv_scale, const __nv_bfloat16* wt, const float* params, float* T, int n_fill,
                              int* err, cudaStream_t stream, int n_sm);
-// Rows perm(first .. first + B - 1) of (X [n][64], T [n][8], G [n][12]) into (Xb, Tb, Gb), perm = the
-// seeded permutation of [0, n) drawn by key.
-cudaError_t launch_mlp_gather(const __nv_bfloat16* X, const float* T, const float* G, uint64_t n, uint64_t first,
-                              uint64_t B, uint64_t key, __nv_bfloat16* Xb, float* Tb, float* Gb, __nv_bfloat16* Xt,
-                              cudaStream_t stream);
-cudaError_t launch_mlp_accumulate(float* dst, const float* src, float w, cudaStream_t stream);
 // One CTA waits, for at most `limit_ns` (1 ns .. 1 s), on an mbarrier that receives an arrival only
 // when `arrive` != 0; a wait that runs out sets *err (if 0) to the MMA-timeout code.  `elapsed`
 // (device, optional) receives the wait's duration in nanoseconds of the global timer.

@@ -235,22 +235,24 @@ __device__ __forceinline__ uint64_t perm_index(uint64_t k, uint64_t n, int h, ui
   return k;
 }
 
-// Place of flat parameter i in the fused inference's weight layout (mlp.h) and its BF16 value there; biases have
-// none.  Outputs by rows, split by output; the output layer in both halves.
-__device__ __forceinline__ void tile_weight(int i, __nv_bfloat16 v, __nv_bfloat16* fwd) {
-  uint32_t first;
+// Places of flat parameter i in the fused kernels' weight layouts (mlp.h) and its BF16 value there; biases have
+// none.  fwd: outputs by rows, split by output; the output layer in both halves.  back: the transposes of
+// layers 2-4, split by input.
+__device__ __forceinline__ void tile_weight(int i, __nv_bfloat16 v, __nv_bfloat16* fwd, __nv_bfloat16* back) {
+  uint32_t first, back_first = 0;
   int off, K;
   if (i < kOffB1) {
     off = kOffW1; K = kMlpIn; first = 0;
   } else if (i >= kOffW2 && i < kOffB2) {
-    off = kOffW2; K = kMlpHidden; first = kMlpTileW2;
+    off = kOffW2; K = kMlpHidden; first = kMlpTileW2; back_first = kMlpTileW2t;
   } else if (i >= kOffW3 && i < kOffB3) {
-    off = kOffW3; K = kMlpHidden; first = kMlpTileW3;
+    off = kOffW3; K = kMlpHidden; first = kMlpTileW3; back_first = kMlpTileW3t;
   } else if (i >= kOffW4 && i < kOffB4) {
     const int r = (i - kOffW4) >> 8, k = (i - kOffW4) & 255;
     const uint32_t byte = kMlpTileW4 + (uint32_t)(k >> 6) * kMlpW4Chunk + tc::sw128_offset(r, k & 63);
     fwd[byte / 2] = v;
     fwd[(kMlpHalfBytes + byte) / 2] = v;
+    back[((uint32_t)(k >> 7) * kMlpHalfTBytes + kMlpTileW4t + tc::kmajor_offset(k & 127, r, kMlpOut)) / 2] = v;
     return;
   } else {
     return;
@@ -258,6 +260,9 @@ __device__ __forceinline__ void tile_weight(int i, __nv_bfloat16 v, __nv_bfloat1
   const int r = (i - off) / K, k = (i - off) % K;
   fwd[((uint32_t)(r >> 7) * kMlpHalfBytes + first + (uint32_t)(k >> 6) * kMlpChunk +
        tc::sw128_offset(r & 127, k & 63)) / 2] = v;
+  if (K == kMlpHidden)
+    back[((uint32_t)(k >> 7) * kMlpHalfTBytes + back_first + (uint32_t)(r >> 6) * kMlpChunk +
+          tc::sw128_offset(k & 127, r & 63)) / 2] = v;
 }
 
 }  // namespace fpt
