@@ -905,6 +905,10 @@ struct OrderPlan {
   OrderRun runs[kMaxOrder];
   int count = 0;
   bool overlap = false;
+  void run_in_turn(cudaStream_t stream) {
+    overlap = false;
+    for (int i = 0; i < count; ++i) runs[i].stream = stream;
+  }
 };
 
 static fpt_status plan_orders(fpt_ctx* ctx, const fpt_batch* b, bool scratch, bool steps, OrderPlan& plan) {
@@ -914,7 +918,8 @@ static fpt_status plan_orders(fpt_ctx* ctx, const fpt_batch* b, bool scratch, bo
     const PathRec* list;
     const uint64_t cnt = order_slice(b, n, &list);
     if (!cnt) continue;
-    if (cnt > 0xFFFFFFFFull) return fail(ctx, FPT_EUNSUPPORTED, "more than 2^32 paths of one order");
+    if (scratch && cnt > 0xFFFFFFFFull)  // the lists hold 32-bit path numbers
+      return fail(ctx, FPT_EUNSUPPORTED, "more than 2^32 paths of one order");
     OrderRun& r = plan.runs[plan.count++];
     r = OrderRun{n, cnt, list, ctx->stream, nullptr, nullptr, reinterpret_cast<OrderCtl*>(ctx->d_ctl) + n};
     sum += cnt;
@@ -1271,27 +1276,51 @@ fpt_status fpt_backward_unrolled(fpt_ctx* ctx, const fpt_scene* s, const fpt_bat
   st = ensure_gacc(ctx, s);
   if (st != FPT_OK) return st;
   const SceneDev S = scene_dev(s);
-  for (int n = 1; n <= kMaxOrder; ++n) {
-    const PathRec* list;
-    const uint64_t cnt = order_slice(b, n, &list);
-    if (!cnt) continue;
-    // tape for every resident thread (at most 8 CTAs of kThreads per SM), within kUnrolledMaxTape bytes
-    uint64_t threads = ((cnt + kThreads - 1) / kThreads) * kThreads;
+  // tape for every resident thread of an order (at most 8 CTAs of kThreads per SM), within kUnrolledMaxTape bytes
+  auto tape_floats = [&](const OrderRun& r) {
+    uint64_t threads = ((r.cnt + kThreads - 1) / kThreads) * kThreads;
     const uint64_t resident = (uint64_t)ctx->n_sm * 8 * kThreads;
     if (threads > resident) threads = resident;
-    size_t need = unrolled_tape_floats(n, steps, threads);
-    if (need * sizeof(float) > kUnrolledMaxTape) need = kUnrolledMaxTape / sizeof(float);
-    if (need > ctx->tape_cap) {
-      cudaFree(ctx->d_tape);
-      ctx->d_tape = nullptr;
-      ctx->tape_cap = 0;
-      CUDA_OR_FAIL(ctx, cudaMalloc(&ctx->d_tape, need * sizeof(float)));
-      ctx->tape_cap = need;
-    }
-    ProfScope ps(ctx, FPT_K_BACKWARD);
-    CUDA_OR_FAIL(ctx, launch_unrolled(n, S, b->dev, steps, fp_iters, cnt, list, dX, dL, ctx->d_gacc, ctx->d_tape,
-                                      ctx->tape_cap, T_out, status_out, ctx->stream, ctx->n_sm));
+    const size_t need = unrolled_tape_floats(r.n, steps, threads), most = kUnrolledMaxTape / sizeof(float);
+    return need > most ? most : need;
+  };
+  // Orders side by side where their tapes fit kUnrolledMaxTape together: the shorter orders run on the SMs that the
+  // longest one's last, partly filled round of CTAs leaves idle.
+  OrderPlan plan;
+  st = plan_orders(ctx, b, false, false, plan);
+  if (st != FPT_OK) return st;
+  size_t sum = 0, most = 0;
+  for (int i = 0; i < plan.count; ++i) {
+    const size_t need = tape_floats(plan.runs[i]);
+    sum += need;
+    most = need > most ? need : most;
   }
+  if (sum * sizeof(float) > kUnrolledMaxTape) plan.run_in_turn(ctx->stream);
+  for (size_t cap = plan.overlap ? sum : most; cap > ctx->tape_cap;) {
+    cudaFree(ctx->d_tape);
+    ctx->d_tape = nullptr;
+    ctx->tape_cap = 0;
+    const cudaError_t e = cudaMalloc(&ctx->d_tape, cap * sizeof(float));
+    if (e == cudaSuccess) {
+      ctx->tape_cap = cap;
+    } else if (plan.overlap) {  // no room side by side
+      cudaGetLastError();
+      plan.run_in_turn(ctx->stream);
+      cap = most;
+    } else {
+      CUDA_OR_FAIL(ctx, e);
+    }
+  }
+  size_t at = 0;
+  st = run_orders(ctx, plan, [&](const OrderRun& r) -> fpt_status {
+    ProfScope ps(ctx, FPT_K_BACKWARD);
+    const size_t need = tape_floats(r);
+    CUDA_OR_FAIL(ctx, launch_unrolled(r.n, S, b->dev, steps, fp_iters, r.cnt, r.list, dX, dL, ctx->d_gacc,
+                                      ctx->d_tape + at, need, T_out, status_out, r.stream, ctx->n_sm));
+    if (plan.overlap) at += need;
+    return FPT_OK;
+  });
+  if (st != FPT_OK) return st;
   {
     ProfScope ps(ctx, FPT_K_OTHER);
     CUDA_OR_FAIL(ctx, launch_backward_finalize(S, nullptr, ctx->d_gacc, g_tx, g_rx, g_vertices, ctx->stream));

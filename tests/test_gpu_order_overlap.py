@@ -83,3 +83,28 @@ def test_overlapped_orders_match_sequential_orders(ctx, kind):
         assert torch.equal(torch.nan_to_num(a.float(), nan=7e30), torch.nan_to_num(b.float(), nan=7e30))
     for a, b in zip(side_sums, seq_sums):
         assert float((a - b).abs().max()) <= 1e-5 * max(1e-30, float(b.abs().max()))
+
+
+def test_overlapped_unrolled_orders_match_sequential_orders(ctx):
+    """Reverse mode through the steps: orders side by side (each with its own tape) against one after the other."""
+    import torch
+
+    scene, batch = _batch(ctx, "orders-1-10")
+
+    def run():
+        out = fpt.backward_unrolled(ctx, scene, batch, 5, 1, dL=torch.ones(batch.n_paths, device="cuda"), want_T=True)
+        ctx.sync()
+        return [t.clone() for t in out]
+
+    side = run()
+    fpt.profile_enable(ctx, True)
+    try:
+        seq = run()
+    finally:
+        fpt.profile_enable(ctx, False)
+        fpt.profile_read(ctx)
+    for k, (a, b) in enumerate(zip(side, seq)):
+        if k < 3:
+            assert float((a - b).abs().max()) <= 1e-5 * max(1e-30, float(b.abs().max()))
+        else:
+            assert torch.equal(torch.nan_to_num(a.float(), nan=7e30), torch.nan_to_num(b.float(), nan=7e30))
