@@ -189,9 +189,9 @@ struct fpt_mlp {
   // forward activations and outputs for up to cap rows
   uint64_t cap = 0;
   __nv_bfloat16 *d_H1 = nullptr, *d_H2 = nullptr;
-  // transposed operands of the weight gradients dW = dZ^T act for up to train_cap rows
+  // operands of the weight gradients dW = dZ^T act for up to train_cap rows
   uint64_t train_cap = 0;
-  __nv_bfloat16 *d_Ht = nullptr, *d_dZt = nullptr, *d_dYt = nullptr, *d_Xt = nullptr;
+  __nv_bfloat16 *d_H = nullptr, *d_dZ = nullptr, *d_dYt = nullptr, *d_X = nullptr;
 };
 
 static fpt_status mlp_tiled_weights(fpt_ctx* ctx, fpt_mlp* m);
@@ -1413,7 +1413,7 @@ fpt_status fpt_count_status(fpt_ctx* ctx, const uint8_t* status, uint64_t n, uin
 // learned warm start
 // ---------------------------------------------------------------------------
 static void mlp_free_ws(fpt_mlp* m) {
-  for (__nv_bfloat16** p : {&m->d_H1, &m->d_H2, &m->d_Ht, &m->d_dZt, &m->d_dYt, &m->d_Xt}) {
+  for (__nv_bfloat16** p : {&m->d_H1, &m->d_H2, &m->d_H, &m->d_dZ, &m->d_dYt, &m->d_X}) {
     cudaFree(*p);
     *p = nullptr;
   }
@@ -1433,10 +1433,10 @@ static fpt_status mlp_ensure_ws(fpt_ctx* ctx, fpt_mlp* m, uint64_t B, bool train
   const size_t H = want * kMlpHidden;
   if (train) {
     m->train_cap = 0;
-    bf(&m->d_Ht, 3 * H);
-    bf(&m->d_dZt, 3 * H);
-    bf(&m->d_dYt, want * kMlpOut);
-    bf(&m->d_Xt, want * kMlpIn);
+    bf(&m->d_H, 3 * H);
+    bf(&m->d_dZ, 3 * H);
+    bf(&m->d_dYt, (want + 7) / 8 * 8 * kMlpOut);
+    bf(&m->d_X, want * kMlpIn);
   } else {
     m->cap = 0;
     bf(&m->d_H1, H);
@@ -1489,7 +1489,7 @@ static fpt_status mlp_forward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16
     g.H = H[l];
     g.shm = kMlpHidden;
     g.shn = 1;
-    CUDA_OR_FAIL(ctx, launch_gemm(g, 1, ctx->stream));
+    CUDA_OR_FAIL(ctx, launch_gemm(g, ctx->stream));
     in = H[l];
   }
   GemmArgs g = gemm_args(Bi, kMlpOut, kMlpHidden, in, kMlpHidden, 1, W + kOffW4, kMlpHidden, 1, EPI_STORE, ctx->d_err);
@@ -1497,27 +1497,13 @@ static fpt_status mlp_forward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16
   g.C = Y;
   g.scm = kMlpOut;
   g.scn = 1;
-  CUDA_OR_FAIL(ctx, launch_gemm(g, 1, ctx->stream));
+  CUDA_OR_FAIL(ctx, launch_gemm(g, ctx->stream));
   return FPT_OK;
 }
 
-static int split_k(const fpt_ctx* ctx, int B, int m_tiles) {
-  // one (row tile, K split) item per SM (each CTA adds one partial product into the gradient), at least
-  // four 64-wide K chunks per split
-  int ks = ctx->n_sm / m_tiles;
-  const int max_ks = B / 256 > 1 ? B / 256 : 1;
-  ks = ks < 1 ? 1 : (ks > max_ks ? max_ks : ks);
-  // the GEMM gives each split ceil(B / (ks 64)) chunks of 64: count only the splits that get some
-  const int per = (B + ks * 64 - 1) / (ks * 64) * 64;
-  return (B + per - 1) / per;
-}
-
-// Loss and gradient (d_loss, d_g) of a batch: one launch for the forward pass, the loss and the back-propagation, then
-// the weight gradients from its transposed operands.  These are independent and fill 64 SMs each, so they run side by
-// side on the context's order streams.  n > 0: row i is sample perm(first + i) of n (fpt_mlp_train).
+// Loss and gradient (d_loss, d_g) of a batch.  n > 0: row i is sample perm(first + i) of n (fpt_mlp_train).
 static fpt_status mlp_backward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16* X, const float* T, const float* G,
                                     uint64_t B, uint64_t n, uint64_t first, uint64_t key) {
-  const int Bi = (int)B;
   fpt_status st = mlp_ensure_ws(ctx, m, B, true);
   if (st == FPT_OK) st = mlp_tiled_weights(ctx, m);
   if (st != FPT_OK) return st;
@@ -1533,46 +1519,15 @@ static fpt_status mlp_backward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat1
   a.wt = m->d_wt;
   a.wtT = m->d_wtT;
   a.params = m->d_w;
-  a.Xt = m->d_Xt;
-  a.Ht = m->d_Ht;
-  a.dZt = m->d_dZt;
+  a.Xb = m->d_X;
+  a.H = m->d_H;
+  a.dZ = m->d_dZ;
   a.dYt = m->d_dYt;
+  a.ldY = (B + 7) / 8 * 8;
   a.grad = m->d_g;
   a.loss = m->d_loss;
   a.err = ctx->d_err;
   CUDA_OR_FAIL(ctx, launch_mlp_train(a, ctx->stream, ctx->n_sm));
-  // dW_l [out][in] = dZ_l^T [out][b] act^T [in][b]; dW4^T [in][out] = H3^T dY.  K (the batch) is split into one slice
-  // per SM's item; each slice's partial product is added into d_g (TMA reduce-add, else atomics).
-  const int ks = split_k(ctx, Bi, 2);
-  const size_t H = (size_t)kMlpHidden * B;
-  struct Grad {
-    int N;
-    const __nv_bfloat16 *At, *Bt;
-    float* dst;
-    long long scm, scn;
-  };
-  const Grad grads[4] = {{kMlpHidden, m->d_dZt + 2 * H, m->d_Ht + H, m->d_g + kOffW3, kMlpHidden, 1},
-                         {kMlpHidden, m->d_dZt + H, m->d_Ht, m->d_g + kOffW2, kMlpHidden, 1},
-                         {kMlpIn, m->d_dZt, m->d_Xt, m->d_g + kOffW1, kMlpIn, 1},
-                         {kMlpOut, m->d_Ht + 2 * H, m->d_dYt, m->d_g + kOffW4, 1, kMlpHidden}};
-  static_assert(fpt_ctx::kOrderStreams >= 3, "streams of the weight gradients");
-  CUDA_OR_FAIL(ctx, cudaEventRecord(ctx->ofork_ev, ctx->stream));
-  cudaError_t e = cudaSuccess;
-  for (int k = 0; k < 4; ++k) {
-    const cudaStream_t s = k == 0 ? ctx->stream : ctx->ostream[k - 1];
-    if (k > 0 && e == cudaSuccess) e = cudaStreamWaitEvent(s, ctx->ofork_ev, 0);
-    GemmArgs g = gemm_args(kMlpHidden, grads[k].N, Bi, grads[k].At, Bi, 1, grads[k].Bt, Bi, 1, EPI_ATOMIC, ctx->d_err);
-    g.C = grads[k].dst;
-    g.scm = grads[k].scm;
-    g.scn = grads[k].scn;
-    if (e == cudaSuccess) e = launch_gemm(g, ks, s);
-  }
-  for (int k = 0; k < 3; ++k) {  // joined also after an error (a stream capture must end joined)
-    const cudaError_t f = cudaEventRecord(ctx->ojoin_ev[k], ctx->ostream[k]);
-    const cudaError_t w = f == cudaSuccess ? cudaStreamWaitEvent(ctx->stream, ctx->ojoin_ev[k], 0) : f;
-    if (e == cudaSuccess) e = w;
-  }
-  CUDA_OR_FAIL(ctx, e);
   return FPT_OK;
 }
 
@@ -1886,7 +1841,7 @@ fpt_status fpt_tc_gemm_bf16(fpt_ctx* ctx, int32_t M, int32_t N, int32_t K, const
   g.err = ctx->d_err;
   CUDA_OR_FAIL(ctx, cudaSetDevice(ctx->device));
   ProfScope ps(ctx, FPT_K_OTHER);
-  CUDA_OR_FAIL(ctx, launch_gemm(g, 1, ctx->stream));
+  CUDA_OR_FAIL(ctx, launch_gemm(g, ctx->stream));
   return FPT_OK;
 }
 

@@ -5,17 +5,12 @@
 // the solver.  Weights are BF16, accumulation FP32 in tensor memory,
 // activations are rounded to BF16 between layers.
 //
-// GEMMs D[M x N] = sum_k A(m, k) B(n, k), N <= 256, K in chunks of 64.  Operands whose rows are
-// contiguous and 16-byte aligned go to gemm_ws_kernel: persistent, one CTA per SM over (128-row tile,
-// K split) items, the chunks loaded by TMA into a two-stage ring (128-byte swizzled K-major tiles), one
-// thread issuing the MMAs into two TMEM accumulators, twelve epilogue warps staging the outputs in shared
-// memory for TMA tensor stores.
-// Other strides take gemm_kernel, one tile per CTA with the operands gathered element by element.  The
-// training pass keeps every operand K-major: its epilogues also write the transposes that the weight
-// gradients read.  Epilogues: plain store; addition into the output (the weight gradients' split-K
-// partial products, by TMA reduce-adds); bias + GELU with a BF16 activation (and its transpose) and, for
-// training, the GELU derivative at the pre-activation; or the backward's product with that derivative
-// (and its transpose).
+// GEMMs D[M x N] = sum_k A(m, k) B(n, k), N <= 256, K in chunks of 64, for the unfused forward pass.  Operands whose
+// rows are contiguous and 16-byte aligned go to gemm_ws_kernel: persistent, one CTA per SM over 128-row tiles, the
+// chunks loaded by TMA into a three- or two-stage ring (128-byte swizzled K-major tiles), one thread issuing the MMAs
+// into two TMEM accumulators, twelve epilogue warps staging the outputs in shared memory for TMA tensor stores.
+// Other strides take gemm_kernel, one tile per CTA with the operands gathered element by element.  Epilogues: plain
+// store (+ bias); bias + GELU with a BF16 activation.  Inference is fused in k_infer.cu, training in k_train.cu.
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
@@ -104,9 +99,7 @@ static_assert(4 * 32 * kEpiStride * 4 <= kGemmSmem, "epilogue slabs");
 
 // Epilogue of one warp's 32 accumulator rows (TMEM lanes 32 w .. 32 w + 31, matrix rows mrow0 ..).  Per
 // 64-column slab: (a) the accumulator (+ bias) goes from TMEM to the warp's staging slab, lane = row;
-// (b) row by row, consecutive lanes on consecutive columns, the row-major outputs are formed and stored
-// (coalesced; Zin read the same way), and the final value is kept in the slab; (c) column by column,
-// consecutive lanes on consecutive rows, the transposed copy Ht is stored (coalesced too).
+// (b) row by row, consecutive lanes on consecutive columns, the output is formed and stored (coalesced).
 __device__ __forceinline__ void gemm_epilogue_staged(const GemmArgs& g, uint32_t tmem_warp, int mrow0, int lane,
                                                      int n_pad, float* slab) {
   for (int c0 = 0; c0 < n_pad; c0 += kEpiCols) {
@@ -118,7 +111,7 @@ __device__ __forceinline__ void gemm_epilogue_staged(const GemmArgs& g, uint32_t
       for (int q = 0; q < 16; ++q) {
         const int n = c0 + cc + q;
         float x = v[q];
-        if ((g.op == EPI_STORE || g.op == EPI_BIAS_GELU) && g.bias && n < g.N) x += g.bias[n];
+        if (g.bias && n < g.N) x += g.bias[n];
         slab[lane * kEpiStride + cc + q] = x;
       }
     }
@@ -130,46 +123,10 @@ __device__ __forceinline__ void gemm_epilogue_staged(const GemmArgs& g, uint32_t
         const int n = c0 + cc;
         if (n >= g.N) continue;
         const float x = slab[r * kEpiStride + cc];
-        float y = x;
-        switch (g.op) {
-          case EPI_STORE:
-            g.C[(long long)m * g.scm + (long long)n * g.scn] = x;
-            break;
-          case EPI_ATOMIC:
-            atomicAdd(g.C + (long long)m * g.scm + (long long)n * g.scn, x);
-            break;
-          case EPI_BIAS_GELU: {
-            float d;
-            y = __bfloat162float(__float2bfloat16(gelu_with_grad(x, d)));
-            if (g.C) g.C[(long long)m * g.scm + (long long)n * g.scn] = d;
-            g.H[(long long)m * g.shm + (long long)n * g.shn] = __float2bfloat16(y);
-            break;
-          }
-          case EPI_GELU_GRAD:
-            y = x * g.Zin[(long long)m * g.szm + (long long)n * g.szn];
-            if (g.C) g.C[(long long)m * g.scm + (long long)n * g.scn] = y;
-            g.H[(long long)m * g.shm + (long long)n * g.shn] = __float2bfloat16(y);
-            break;
-        }
-        slab[r * kEpiStride + cc] = y;
-      }
-    }
-    __syncwarp();
-    if (g.op == EPI_GELU_GRAD && g.colsum) {  // this warp's rows of each column (rows past M hold no value)
-      const int rows = min(32, g.M - mrow0);
-      for (int cc = lane; cc < cols; cc += 32) {
-        if (c0 + cc >= g.N) continue;
-        float acc = 0.f;
-        for (int r = 0; r < rows; ++r) acc += slab[r * kEpiStride + cc];
-        atomicAdd(g.colsum + c0 + cc, acc);
-      }
-    }
-    if (g.Ht) {
-      const int m = mrow0 + lane;
-      for (int cc = 0; cc < cols; ++cc) {
-        const int n = c0 + cc;
-        if (n < g.N && m < g.M)
-          g.Ht[(long long)m * g.shtm + (long long)n * g.shtn] = __float2bfloat16(slab[lane * kEpiStride + cc]);
+        if (g.op == EPI_STORE)
+          g.C[(long long)m * g.scm + (long long)n * g.scn] = x;
+        else
+          g.H[(long long)m * g.shm + (long long)n * g.shn] = __float2bfloat16(gelu(x));
       }
     }
     __syncwarp();
@@ -185,10 +142,7 @@ __global__ void __launch_bounds__(128) gemm_kernel(GemmArgs g) {
   const int m0 = blockIdx.x * 128;
   const int n_pad = (g.N + 15) & ~15;
   const uint32_t ncols = n_pad <= 32 ? 32 : (n_pad <= 64 ? 64 : (n_pad <= 128 ? 128 : 256));
-  // K range of this split
-  const int k_per = ((g.K + gridDim.y * kGemmKC - 1) / (gridDim.y * kGemmKC)) * kGemmKC;
-  const int kb = blockIdx.y * k_per, ke = min(g.K, kb + k_per);
-  const int n_chunks = ke > kb ? (ke - kb + kGemmKC - 1) / kGemmKC : 0;
+  const int n_chunks = (g.K + kGemmKC - 1) / kGemmKC;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kGemmStages; ++s) tc::mbar_init(&bar[s], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -228,8 +182,8 @@ __global__ void __launch_bounds__(128) gemm_kernel(GemmArgs g) {
     // pipelined: chunks load (cp.async, one commit group per chunk) kGemmStages - 1 ahead of the MMAs
     for (int c = 0; c < kGemmStages - 1; ++c) {
       if (c < n_chunks) {
-        load_tile_async(stage_a(c), g.A, g.sam, g.M, g.K, m0, kb + c * kGemmKC, 128);
-        load_tile_async(stage_b(c), g.B, g.sbn, g.N, g.K, 0, kb + c * kGemmKC, n_pad);
+        load_tile_async(stage_a(c), g.A, g.sam, g.M, g.K, m0, c * kGemmKC, 128);
+        load_tile_async(stage_b(c), g.B, g.sbn, g.N, g.K, 0, c * kGemmKC, n_pad);
       }
       cp_async_commit();
     }
@@ -244,8 +198,8 @@ __global__ void __launch_bounds__(128) gemm_kernel(GemmArgs g) {
       const int cn = c + kGemmStages - 1;
       if (cn < n_chunks && (c == 0 || wait_chunk(c - 1))) {
         const int sn = cn % kGemmStages;
-        load_tile_async(stage_a(sn), g.A, g.sam, g.M, g.K, m0, kb + cn * kGemmKC, 128);
-        load_tile_async(stage_b(sn), g.B, g.sbn, g.N, g.K, 0, kb + cn * kGemmKC, n_pad);
+        load_tile_async(stage_a(sn), g.A, g.sam, g.M, g.K, m0, cn * kGemmKC, 128);
+        load_tile_async(stage_b(sn), g.B, g.sbn, g.N, g.K, 0, cn * kGemmKC, n_pad);
       }
       cp_async_commit();
     }
@@ -253,8 +207,8 @@ __global__ void __launch_bounds__(128) gemm_kernel(GemmArgs g) {
   } else {
     // element gathers from arbitrary strides: one stage, each chunk waited for before the next
     for (int c = 0; c < n_chunks; ++c) {
-      load_tile(stage_a(0), g.A, g.sam, g.sak, g.M, g.K, m0, kb + c * kGemmKC, 128);
-      load_tile(stage_b(0), g.B, g.sbn, g.sbk, g.N, g.K, 0, kb + c * kGemmKC, n_pad);
+      load_tile(stage_a(0), g.A, g.sam, g.sak, g.M, g.K, m0, c * kGemmKC, 128);
+      load_tile(stage_b(0), g.B, g.sbn, g.sbk, g.N, g.K, 0, c * kGemmKC, n_pad);
       tc::fence_async_smem();
       __syncthreads();
       if (threadIdx.x == 0) {
@@ -295,7 +249,7 @@ __global__ void __launch_bounds__(128) gemm_kernel(GemmArgs g) {
 }
 
 // ---- persistent warp-specialised GEMM (TMA operands) -------------------------------------------------
-// One CTA per SM walks the (128-row tile, K split) items.  Warp 0 (one thread) loads each 64-wide K chunk
+// One CTA per SM walks the 128-row tiles.  Warp 0 (one thread) loads each 64-wide K chunk
 // of A (128 rows) and B (n_pad rows) with one TMA tile load per operand into a ring of kWsStages stages,
 // in the 128-byte swizzled K-major layout; rows past M or N and k past K arrive as zeros.  Warp 1 (one
 // thread) issues four 128 x n_pad x 16 MMAs per chunk into one of two TMEM accumulators (columns 0-255,
@@ -307,28 +261,14 @@ __global__ void __launch_bounds__(128) gemm_kernel(GemmArgs g) {
 // The warps hand the accumulator back through `acc_empty`, so the MMAs of the tile after next may start
 // while this tile's epilogue runs.  Every wait is bounded; a timeout sets the CTA's fail flag, which every
 // role polls and leaves on.
-constexpr int kWsStages = 2;     // operand ring stages when the epilogue stages BF16 outputs
-constexpr int kWsStagesMax = 3;  // ... and when it stages only the FP32 box (plain stores, reduce-adds)
+constexpr int kWsStages = 3;  // operand ring
 constexpr int kWsEpiWarps = 12;
 constexpr int kWsGroupStride = kWsEpiWarps / 4;  // epilogue warps per 32-lane quarter of TMEM
 constexpr int kWsThreads = 32 * (2 + kWsEpiWarps);
 constexpr int kWsTileA = 128 * 128;                       // 128 rows x 128 bytes
 constexpr int kWsStageBytes = kWsTileA + 256 * 128;       // + B, up to 256 rows: 48 KB
-// the ring, two 4 KB output staging buffers per epilogue warp, slack to align the ring to 1024 bytes
-constexpr int kWsSmem = kWsStages * kWsStageBytes + kWsEpiWarps * 2 * 4096 + 1024;
-static_assert(kWsStagesMax * kWsStageBytes + kWsEpiWarps * 2 * 2048 + 1024 <= kWsSmem, "ring and staging");
-
-struct WsItem {
-  int m0, kb, ke, split;
-};
-__device__ __forceinline__ WsItem ws_item(const GemmArgs& g, int item, int m_tiles, int k_per) {
-  WsItem w;
-  w.m0 = (item % m_tiles) * 128;
-  w.split = item / m_tiles;
-  w.kb = w.split * k_per;
-  w.ke = min(g.K, w.kb + k_per);
-  return w;
-}
+// the ring, two 2 KB output staging buffers per epilogue warp, slack to align the ring to 1024 bytes
+constexpr int kWsSmem = kWsStages * kWsStageBytes + kWsEpiWarps * 2 * 2048 + 1024;
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
@@ -336,16 +276,15 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
-// Which outputs may use 16-byte vector accesses (unit stride along n, row strides and bases aligned).
+// Which accesses may take 16 bytes (unit stride along n, row strides and bases aligned).
 struct EpiVec {
-  bool c, h, z, bias;
+  bool c, h, bias;
 };
 __device__ __forceinline__ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 __device__ __forceinline__ EpiVec epi_vec(const GemmArgs& g) {
   EpiVec v;
   v.c = g.scn == 1 && g.scm % 4 == 0 && aligned16(g.C);
   v.h = g.shn == 1 && g.shm % 8 == 0 && aligned16(g.H);
-  v.z = g.szn == 1 && g.szm % 4 == 0 && aligned16(g.Zin);
   v.bias = aligned16(g.bias);
   return v;
 }
@@ -379,60 +318,22 @@ __device__ __forceinline__ void store16_bf16(__nv_bfloat16* p, const float (&x)[
   }
 }
 
-// Z[m][n0 .. n0 + 15] (zero past N or M) into registers; 16-byte loads when aligned and whole.
-__device__ __forceinline__ void load_z16(const GemmArgs& g, const EpiVec& ev, int m, bool row, int n0, float (&z)[16]) {
-  const float* zp = g.Zin + (long long)m * g.szm + (long long)n0 * g.szn;
-  const int nv = min(16, g.N - n0);
-  if (row && nv == 16 && ev.z) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float4 t = __ldg(reinterpret_cast<const float4*>(zp) + i);
-      z[4 * i] = t.x;
-      z[4 * i + 1] = t.y;
-      z[4 * i + 2] = t.z;
-      z[4 * i + 3] = t.w;
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 16; ++i) z[i] = row && i < nv ? zp[i * g.szn] : 0.f;
-  }
-}
-
 // Staging of one warp's 32 x 16 output group for the TMA tensor stores (two buffers per warp, used in
 // turn): the FP32 box in the 64-byte swizzled layout (row r, 16-byte chunk c at r 64 + 16 (c ^ (r / 2 mod 4))),
-// the BF16 box in the 32-byte swizzled layout (r 32 + 16 (c ^ (r / 4 mod 2))), the transposed BF16 box
-// plainly (column n of the group at n 64, row r at 2 r).  Consecutive lanes (rows) hit different banks
-// in all three.
-constexpr int kStgC = 0, kStgH = 2048, kStgHt = 3072, kStgBytes = 4096;
-constexpr int kOutC = 1, kOutH = 2, kOutHt = 4;  // outputs that go through TMA stores
-constexpr int kOutCt = 8;  // EPI_ATOMIC into a column-major destination: the FP32 box staged transposed
-
-struct OutMaps {
-  const CUtensorMap* c;
-  const CUtensorMap* h;
-  const CUtensorMap* ht;
-  int flags;
-};
+// the BF16 box in the 32-byte swizzled layout (r 32 + 16 (c ^ (r / 4 mod 2))).  Consecutive lanes (rows) hit
+// different banks in both.
+constexpr int kStgBytes = 2048;
 
 // One warp's share of a finished 128 x n_pad accumulator: its lane quarter, column groups j0, j0 + kWsGroupStride, ...
-// m = this lane's output row, mrow0 = the warp's first row.  Each output goes out through a TMA store of the
-// staged group when its tensor map exists (flags), else with this lane's own stores.  gi counts the warp's
-// groups (it picks the staging buffer).  For EPI_GELU_GRAD the pre-activations of the next group are
-// loaded while the current one is worked on, and the column sums of dZ are added to s_col.
+// m = this lane's output row, mrow0 = the warp's first row.  The output goes out through a TMA store of the
+// staged group when its tensor map exists (`tma`), else with this lane's own stores.  gi counts the warp's
+// groups (it picks the staging buffer).
 template <int OP>
 __device__ __forceinline__ void ws_epilogue(const GemmArgs& g, const EpiVec& ev, uint32_t tacc, int m, int mrow0,
-                                            int j0, int n_groups, float* s_col, const OutMaps& om,
-                                            unsigned char* stg, int stg_bytes, int& gi) {
+                                            int j0, int n_groups, const CUtensorMap* out, bool tma, unsigned char* stg,
+                                            int& gi) {
   const int lane = lane_id();
   const bool row = m < g.M;
-  const bool has_c = OP == EPI_STORE || OP == EPI_ATOMIC || g.C != nullptr;
-  const bool has_h = OP == EPI_BIAS_GELU || OP == EPI_GELU_GRAD;
-  const bool has_ht = has_h && g.Ht != nullptr;
-  const bool tma_c = has_c && (om.flags & (kOutC | kOutCt)), tma_h = has_h && (om.flags & kOutH),
-             tma_ht = has_ht && (om.flags & kOutHt);
-  const bool any_tma = tma_c || tma_h || tma_ht;
-  float zq[16];  // the pre-activations of the next column group (EPI_GELU_GRAD)
-  if (OP == EPI_GELU_GRAD && j0 < n_groups) load_z16(g, ev, m, row, 16 * j0, zq);
   for (int j = j0; j < n_groups; j += kWsGroupStride) {
     const int n0 = 16 * j;
     const int nv = min(16, g.N - n0);
@@ -440,7 +341,7 @@ __device__ __forceinline__ void ws_epilogue(const GemmArgs& g, const EpiVec& ev,
     float x[16];
     __syncwarp();
     tc::tmem_ld16(tacc + (uint32_t)n0, x);
-    if ((OP == EPI_STORE || OP == EPI_BIAS_GELU) && g.bias) {
+    if (g.bias) {
       if (full && ev.bias) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -456,106 +357,46 @@ __device__ __forceinline__ void ws_epilogue(const GemmArgs& g, const EpiVec& ev,
           if (i < nv) x[i] += g.bias[n0 + i];
       }
     }
-    float h[16];  // the BF16 output (rounded when stored): the activation, or dZ
-    if (OP == EPI_GELU_GRAD) {
-      float z[16];
+    if (OP == EPI_BIAS_GELU) {
 #pragma unroll
-      for (int i = 0; i < 16; ++i) z[i] = zq[i];
-      if (j + kWsGroupStride < n_groups) load_z16(g, ev, m, row, 16 * (j + kWsGroupStride), zq);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) x[i] = row ? x[i] * z[i] : 0.f;
-      if (s_col) {
-        const float cs = warp_colsum16(x, lane);
-        if ((lane & 1) == 0) {
-          const int c = warp_colsum16_column(lane);
-          if (c < nv) atomicAdd(s_col + n0 + c, cs);
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 16; ++i) h[i] = x[i];
-    } else if (OP == EPI_BIAS_GELU) {
-      if (has_c) {  // training: the FP32 output is gelu'(Z) for the backward
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          float d;
-          h[i] = gelu_with_grad(x[i], d);
-          x[i] = d;
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) h[i] = gelu(x[i]);
-      }
+      for (int i = 0; i < 16; ++i) x[i] = gelu(x[i]);
     }
-    // this lane's own stores for the outputs without a tensor map
-    if (row) {
-      if (has_c && !tma_c) {
-        if (OP == EPI_ATOMIC) {
-#pragma unroll
-          for (int i = 0; i < 16; ++i)
-            if (i < nv) atomicAdd(g.C + (long long)m * g.scm + (long long)(n0 + i) * g.scn, x[i]);
-        } else {
-          store16_f32(g.C + (long long)m * g.scm + (long long)n0 * g.scn, x, full && ev.c, nv, g.scn);
-        }
-      }
-      if (has_h && !tma_h) store16_bf16(g.H + (long long)m * g.shm + (long long)n0 * g.shn, h, full && ev.h, nv, g.shn);
-      if (has_ht && !tma_ht) {
-        __nv_bfloat16* tp = g.Ht + (long long)m * g.shtm + (long long)n0 * g.shtn;
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-          if (i < nv) tp[i * g.shtn] = __float2bfloat16(h[i]);
-      }
+    if (!tma) {  // this lane's own stores
+      if (row && OP == EPI_STORE)
+        store16_f32(g.C + (long long)m * g.scm + (long long)n0 * g.scn, x, full && ev.c, nv, g.scn);
+      if (row && OP == EPI_BIAS_GELU)
+        store16_bf16(g.H + (long long)m * g.shm + (long long)n0 * g.shn, x, full && ev.h, nv, g.shn);
+      continue;
     }
-    if (!any_tma) continue;
     // the staged group: wait until the engine has read this buffer's previous group, fill it, store it
-    unsigned char* buf = stg + (gi & 1) * stg_bytes;
+    unsigned char* buf = stg + (gi & 1) * kStgBytes;
     ++gi;
     if (lane == 0) tc::bulk_wait_read<1>();
     __syncwarp();
-    if (tma_c && (om.flags & kOutCt)) {  // column n of the group at n 128 bytes, row r at 4 r
-      float* tb = reinterpret_cast<float*>(buf + kStgC) + lane;
-#pragma unroll
-      for (int i = 0; i < 16; ++i) tb[32 * i] = x[i];
-    } else if (tma_c) {
-      unsigned char* cb = buf + kStgC + lane * 64;
+    if (OP == EPI_STORE) {
+      unsigned char* cb = buf + lane * 64;
       const int sw = (lane >> 1) & 3;
 #pragma unroll
       for (int c = 0; c < 4; ++c)
         *reinterpret_cast<float4*>(cb + 16 * (c ^ sw)) = make_float4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
-    }
-    if (tma_h) {
-      unsigned char* hb = buf + kStgH + lane * 32;
+    } else {
+      unsigned char* hb = buf + lane * 32;
       const int sw = (lane >> 2) & 1;
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         uint32_t w[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const __nv_bfloat162 b2 = __floats2bfloat162_rn(h[8 * c + 2 * i], h[8 * c + 2 * i + 1]);
+          const __nv_bfloat162 b2 = __floats2bfloat162_rn(x[8 * c + 2 * i], x[8 * c + 2 * i + 1]);
           w[i] = *reinterpret_cast<const uint32_t*>(&b2);
         }
         *reinterpret_cast<uint4*>(hb + 16 * (c ^ sw)) = make_uint4(w[0], w[1], w[2], w[3]);
       }
     }
-    if (tma_ht) {
-      __nv_bfloat16* tb = reinterpret_cast<__nv_bfloat16*>(buf + kStgHt) + lane;
-#pragma unroll
-      for (int i = 0; i < 16; ++i) tb[32 * i] = __float2bfloat16(h[i]);
-    }
     tc::fence_async_smem();
     __syncwarp();
     if (lane == 0 && mrow0 < g.M) {
-      if (tma_c) {
-        if (OP == EPI_ATOMIC) {
-          if (om.flags & kOutCt)
-            tc::tma_reduce_add_2d(om.c, buf + kStgC, mrow0, n0);
-          else
-            tc::tma_reduce_add_2d(om.c, buf + kStgC, n0, mrow0);
-        } else {
-          tc::tma_store_2d(om.c, buf + kStgC, n0, mrow0);
-        }
-      }
-      if (tma_h) tc::tma_store_2d(om.h, buf + kStgH, n0, mrow0);
-      if (tma_ht) tc::tma_store_2d(om.ht, buf + kStgHt, mrow0, n0);
+      tc::tma_store_2d(out, buf, n0, mrow0);
       tc::bulk_commit();
     }
   }
@@ -563,27 +404,19 @@ __device__ __forceinline__ void ws_epilogue(const GemmArgs& g, const EpiVec& ev,
 
 __global__ void __launch_bounds__(kWsThreads, 1)
     gemm_ws_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmH,
-                   const __grid_constant__ CUtensorMap tmHt, int out_flags, GemmArgs g, int m_tiles, int n_items,
-                   int k_per) {
+                   const __grid_constant__ CUtensorMap tmOut, int tma_out, GemmArgs g, int m_tiles) {
   extern __shared__ unsigned char ws_raw[];
-  __shared__ __align__(8) uint64_t full[kWsStagesMax], empty[kWsStagesMax], acc_full[2], acc_empty[2];
+  __shared__ __align__(8) uint64_t full[kWsStages], empty[kWsStages], acc_full[2], acc_empty[2];
   __shared__ uint32_t s_tmem;
   __shared__ int s_fail;
   __shared__ int s_last_q;             // the MMA thread's last committed chunk (-1: none)
-  __shared__ int s_armed[kWsStagesMax];  // each stage's last phase handed to the TMA engine (-1: none)
-  __shared__ float s_col[256];         // this CTA's column sums (EPI_GELU_GRAD with colsum)
+  __shared__ int s_armed[kWsStages];  // each stage's last phase handed to the TMA engine (-1: none)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned all = 0xffffffffu;
   const int n_pad = (g.N + 15) & ~15;
-  // outputs staged only in the FP32 slot leave room for a deeper operand ring (long K of the weight
-  // gradients); the BF16 outputs need the whole 4 KB staging buffers
-  const bool fp32_only = g.op == EPI_STORE || g.op == EPI_ATOMIC;
-  const int stages = fp32_only ? kWsStagesMax : kWsStages;
-  const int stg_bytes = fp32_only ? 2048 : kStgBytes;
   unsigned char* ring = ws_raw + ((1024u - (tc::smem_u32(ws_raw) & 1023u)) & 1023u);
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kWsStagesMax; ++s) {
+    for (int s = 0; s < kWsStages; ++s) {
       tc::mbar_init(&full[s], 1);
       tc::mbar_init(&empty[s], 1);
       s_armed[s] = -1;
@@ -596,9 +429,6 @@ __global__ void __launch_bounds__(kWsThreads, 1)
     s_fail = 0;
     s_last_q = -1;
   }
-  const bool want_col = g.op == EPI_GELU_GRAD && g.colsum != nullptr;
-  if (want_col)
-    for (int k = threadIdx.x; k < 256; k += blockDim.x) s_col[k] = 0.f;
   if (warp == 0) {
     tc::tmem_alloc(&s_tmem, 512);
     tc::tmem_relinquish();
@@ -617,17 +447,16 @@ __global__ void __launch_bounds__(kWsThreads, 1)
       const uint32_t tx_bytes = (uint32_t)(128 + n_pad) * 128u;
       int q = 0;
       bool ok = true;
-      for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
-        const WsItem w = ws_item(g, item, m_tiles, k_per);
-        for (int k0 = w.kb; k0 < w.ke; k0 += kGemmKC, ++q) {
-          const int s = q % stages, u = q / stages;
+      for (int item = blockIdx.x; ok && item < m_tiles; item += gridDim.x) {
+        for (int k0 = 0; k0 < g.K; k0 += kGemmKC, ++q) {
+          const int s = q % kWsStages, u = q / kWsStages;
           if (u > 0) {  // the stage's previous chunk has been read by its MMAs
             ok = !failed() && tc::mbar_wait(&empty[s], (uint32_t)((u - 1) & 1), kWaitNs);
             if (!ok) break;
           }
           tc::mbar_expect_tx(&full[s], tx_bytes);
           s_armed[s] = u;
-          tc::tma_load_2d(stage_a(s), &tmA, k0, w.m0, &full[s]);
+          tc::tma_load_2d(stage_a(s), &tmA, k0, item * 128, &full[s]);
           tc::tma_load_2d(stage_b(s), &tmB, k0, 0, &full[s]);
         }
       }
@@ -640,15 +469,14 @@ __global__ void __launch_bounds__(kWsThreads, 1)
       int q = 0, i = 0;
       bool ok = true;
       const uint32_t idesc = tc::idesc_bf16(128, (uint32_t)n_pad);
-      for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x, ++i) {
-        const WsItem w = ws_item(g, item, m_tiles, k_per);
+      for (int item = blockIdx.x; ok && item < m_tiles; item += gridDim.x, ++i) {
         const int b = i & 1, v = i >> 1;
         if (v > 0) ok = !failed() && tc::mbar_wait(&acc_empty[b], (uint32_t)((v - 1) & 1), kWaitNs);
         if (!ok) break;
         tc::fence_after_sync();
         const uint32_t d = tmem + (uint32_t)(b * 256);
-        for (int k0 = w.kb, c = 0; k0 < w.ke; k0 += kGemmKC, ++q, ++c) {
-          const int s = q % stages, u = q / stages;
+        for (int k0 = 0, c = 0; k0 < g.K; k0 += kGemmKC, ++q, ++c) {
+          const int s = q % kWsStages, u = q / kWsStages;
           ok = !failed() && tc::mbar_wait(&full[s], (uint32_t)(u & 1), kWaitNs);
           if (!ok) break;
           tc::fence_after_sync();
@@ -672,12 +500,10 @@ __global__ void __launch_bounds__(kWsThreads, 1)
     const int j0 = (warp - 2) >> 2;          // its column groups: j0, j0 + kWsGroupStride, ...
     const int n_groups = n_pad / 16;
     const EpiVec ev = epi_vec(g);
-    const OutMaps om{&tmC, &tmH, &tmHt, out_flags};
-    unsigned char* stg = ring + stages * kWsStageBytes + (warp - 2) * 2 * stg_bytes;
+    unsigned char* stg = ring + kWsStages * kWsStageBytes + (warp - 2) * 2 * kStgBytes;
     int gi = 0;
     int i = 0;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++i) {
-      const WsItem w = ws_item(g, item, m_tiles, k_per);
+    for (int item = blockIdx.x; item < m_tiles; item += gridDim.x, ++i) {
       const int b = i & 1, v = i >> 1;
       const bool ok = __all_sync(all, !failed() && tc::mbar_wait(&acc_full[b], (uint32_t)(v & 1), kWaitNs));
       if (!ok) {
@@ -686,23 +512,12 @@ __global__ void __launch_bounds__(kWsThreads, 1)
       }
       tc::fence_after_sync();
       const uint32_t tacc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * 256);
-      const int mrow0 = w.m0 + quarter * 32;
+      const int mrow0 = item * 128 + quarter * 32;
       const int m = mrow0 + lane;
-      switch (g.op) {
-        case EPI_STORE:
-          ws_epilogue<EPI_STORE>(g, ev, tacc, m, mrow0, j0, n_groups, nullptr, om, stg, stg_bytes, gi);
-          break;
-        case EPI_ATOMIC:
-          ws_epilogue<EPI_ATOMIC>(g, ev, tacc, m, mrow0, j0, n_groups, nullptr, om, stg, stg_bytes, gi);
-          break;
-        case EPI_BIAS_GELU:
-          ws_epilogue<EPI_BIAS_GELU>(g, ev, tacc, m, mrow0, j0, n_groups, nullptr, om, stg, stg_bytes, gi);
-          break;
-        default:
-          ws_epilogue<EPI_GELU_GRAD>(g, ev, tacc, m, mrow0, j0, n_groups, want_col ? s_col : nullptr, om,
-                                     stg, stg_bytes, gi);
-          break;
-      }
+      if (g.op == EPI_STORE)
+        ws_epilogue<EPI_STORE>(g, ev, tacc, m, mrow0, j0, n_groups, &tmOut, tma_out != 0, stg, gi);
+      else
+        ws_epilogue<EPI_BIAS_GELU>(g, ev, tacc, m, mrow0, j0, n_groups, &tmOut, tma_out != 0, stg, gi);
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[b]);
@@ -716,14 +531,12 @@ __global__ void __launch_bounds__(kWsThreads, 1)
   if (s_fail && threadIdx.x == 0) {
     if (g.err) atomicCAS(g.err, 0, ERR_MMA_TIMEOUT);
     // let the copies and MMAs already issued finish (bounded) before shared and tensor memory go away
-    for (int s = 0; s < stages; ++s)
+    for (int s = 0; s < kWsStages; ++s)
       if (s_armed[s] >= 0) tc::mbar_wait(&full[s], (uint32_t)(s_armed[s] & 1), kWaitNs);
     const int q = s_last_q;
-    if (q >= 0) tc::mbar_wait(&empty[q % stages], (uint32_t)((q / stages) & 1), kWaitNs);
+    if (q >= 0) tc::mbar_wait(&empty[q % kWsStages], (uint32_t)((q / kWsStages) & 1), kWaitNs);
   }
   __syncthreads();
-  if (want_col && !s_fail)
-    for (int k = threadIdx.x; k < g.N; k += blockDim.x) atomicAdd(g.colsum + k, s_col[k]);
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
@@ -742,8 +555,8 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 
 // A tiled tensor map of `rank` dimensions (dims innermost first, strides in bytes for dimensions 1..),
 // elements outside the tensor read as zero and are not written.
-static bool encode_map(CUtensorMap* map, CUtensorMapDataType type, int rank, const void* base, const cuuint64_t* dims,
-                       const cuuint64_t* strides, const cuuint32_t* box, CUtensorMapSwizzle swizzle) {
+bool encode_map(CUtensorMap* map, CUtensorMapDataType type, int rank, const void* base, const cuuint64_t* dims,
+                const cuuint64_t* strides, const cuuint32_t* box, CUtensorMapSwizzle swizzle) {
   const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc || (reinterpret_cast<uintptr_t>(base) & 15) != 0) return false;
   for (int d = 0; d + 1 < rank; ++d)
@@ -763,50 +576,19 @@ static bool encode_operand(CUtensorMap* map, const __nv_bfloat16* base, int rows
   return encode_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-// Tensor maps of the epilogue's outputs (32-row x 16-column boxes, laid out as the staging buffers are);
-// returns the kOut* flags of the outputs that have one.
-static int encode_outputs(const GemmArgs& g, CUtensorMap* tmC, CUtensorMap* tmH, CUtensorMap* tmHt) {
-  int flags = 0;
-  if (g.op == EPI_ATOMIC) {
-    if (g.scn == 1) {  // row-major destination: boxes as the FP32 stores
-      const cuuint64_t dims[2] = {(cuuint64_t)g.N, (cuuint64_t)g.M};
-      const cuuint64_t strides[1] = {(cuuint64_t)g.scm * 4u};
-      const cuuint32_t box[2] = {16, 32};
-      if (encode_map(tmC, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, g.C, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B))
-        flags |= kOutC;
-    } else if (g.scm == 1) {  // column-major destination: the transposed box
-      const cuuint64_t dims[2] = {(cuuint64_t)g.M, (cuuint64_t)g.N};
-      const cuuint64_t strides[1] = {(cuuint64_t)g.scn * 4u};
-      const cuuint32_t box[2] = {32, 16};
-      if (encode_map(tmC, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, g.C, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE))
-        flags |= kOutCt;
-    }
-  } else if (g.C && g.scn == 1) {
-    const cuuint64_t dims[2] = {(cuuint64_t)g.N, (cuuint64_t)g.M};
-    const cuuint64_t strides[1] = {(cuuint64_t)g.scm * 4u};
-    const cuuint32_t box[2] = {16, 32};
-    if (encode_map(tmC, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, g.C, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B))
-      flags |= kOutC;
-  }
-  if ((g.op == EPI_BIAS_GELU || g.op == EPI_GELU_GRAD) && g.H && g.shn == 1) {
-    const cuuint64_t dims[2] = {(cuuint64_t)g.N, (cuuint64_t)g.M};
-    const cuuint64_t strides[1] = {(cuuint64_t)g.shm * 2u};
-    const cuuint32_t box[2] = {16, 32};
-    if (encode_map(tmH, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, g.H, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_32B))
-      flags |= kOutH;
-  }
-  if ((g.op == EPI_BIAS_GELU || g.op == EPI_GELU_GRAD) && g.Ht && g.shtm == 1) {
-    const cuuint64_t dims[2] = {(cuuint64_t)g.M, (cuuint64_t)g.N};
-    const cuuint64_t strides[1] = {(cuuint64_t)g.shtn * 2u};
-    const cuuint32_t box[2] = {32, 16};
-    if (encode_map(tmHt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, g.Ht, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE))
-      flags |= kOutHt;
-  }
-  return flags;
+// Tensor map of the epilogue's output (32-row x 16-column boxes, laid out as the staging buffers are), if it has one.
+static bool encode_output(const GemmArgs& g, CUtensorMap* map) {
+  const bool f32 = g.op == EPI_STORE;
+  if ((f32 ? g.scn : g.shn) != 1) return false;
+  const cuuint64_t dims[2] = {(cuuint64_t)g.N, (cuuint64_t)g.M};
+  const cuuint64_t strides[1] = {f32 ? (cuuint64_t)g.scm * 4u : (cuuint64_t)g.shm * 2u};
+  const cuuint32_t box[2] = {16, 32};
+  return f32 ? encode_map(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, g.C, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B)
+             : encode_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, g.H, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_32B);
 }
 
-cudaError_t launch_gemm(const GemmArgs& g, int k_split, cudaStream_t stream) {
-  if (g.N < 1 || g.N > 256 || g.M < 1 || g.K < 1 || k_split < 1) return cudaErrorInvalidValue;
+cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t stream) {
+  if (g.N < 1 || g.N > 256 || g.M < 1 || g.K < 1) return cudaErrorInvalidValue;
   static bool attr = false;
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
@@ -818,32 +600,26 @@ cudaError_t launch_gemm(const GemmArgs& g, int k_split, cudaStream_t stream) {
     const int n_pad = (g.N + 15) & ~15;
     CUtensorMap tmA, tmB;
     if (encode_operand(&tmA, g.A, g.M, g.K, g.sam, 128) && encode_operand(&tmB, g.B, g.N, g.K, g.sbn, n_pad)) {
-      // persistent: one CTA per SM over the (tile, split) items
+      // persistent: one CTA per SM over the row tiles
       const int m_tiles = (g.M + 127) / 128;
-      const int k_per = ((g.K + k_split * kGemmKC - 1) / (k_split * kGemmKC)) * kGemmKC;
-      const int splits = (g.K + k_per - 1) / k_per;
-      const int n_items = m_tiles * splits;
       int dev = 0, n_sm = 0;
       cudaError_t e = cudaGetDevice(&dev);
       if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
       if (e != cudaSuccess) return e;
-      const int grid = n_items < n_sm ? n_items : n_sm;
-      CUtensorMap tmC{}, tmH{}, tmHt{};
-      const int out_flags = encode_outputs(g, &tmC, &tmH, &tmHt);
-      gemm_ws_kernel<<<grid, kWsThreads, kWsSmem, stream>>>(tmA, tmB, tmC, tmH, tmHt, out_flags, g, m_tiles, n_items,
-                                                            k_per);
+      CUtensorMap out{};
+      const int tma_out = encode_output(g, &out);
+      gemm_ws_kernel<<<m_tiles < n_sm ? m_tiles : n_sm, kWsThreads, kWsSmem, stream>>>(tmA, tmB, out, tma_out, g, m_tiles);
       count_launch();
       return cudaGetLastError();
     }
   }
-  dim3 grid((g.M + 127) / 128, k_split);
-  gemm_kernel<<<grid, 128, kGemmSmem, stream>>>(g);
+  gemm_kernel<<<(g.M + 127) / 128, 128, kGemmSmem, stream>>>(g);
   count_launch();
   return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
-// features, loss, bias gradients, Adam, learned start
+// features, Adam, learned start
 // ---------------------------------------------------------------------------
 
 // all paths of a batch (global index order) or one order slice (local index order)
@@ -891,21 +667,6 @@ __global__ void to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __r
     dst[i] = __float2bfloat16(src[i]);
 }
 
-// learned start from unfused network outputs Y [count][16] (local indices first .. first + count)
-__global__ void mlp_start_kernel(SceneDev S, BatchDev B, int n, const PathRec* list, uint64_t first, uint64_t count,
-                                 const float* __restrict__ Y, float* __restrict__ T) {
-  for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count; k += (uint64_t)gridDim.x * blockDim.x) {
-    PathDesc d;
-    fetch_path(B, n, list, first + k, d);
-    float y[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) y[i] = Y[k * kMlpOut + i];
-    write_start(d.n, !(d.flags & ST_INVALID), edge_mask(S, d), y,
-                reinterpret_cast<float2*>(T) + d.g * (uint64_t)B.n_max);
-  }
-}
-
-// ---------------------------------------------------------------------------
 static unsigned grid_1d(uint64_t n, int threads, int cap) {
   uint64_t g = (n + threads - 1) / threads;
   return (unsigned)(g < (uint64_t)cap ? (g ? g : 1) : (uint64_t)cap);
@@ -962,14 +723,6 @@ cudaError_t launch_bounded_wait_check(uint32_t limit_ns, int arrive, int* err, u
                                       cudaStream_t stream) {
   if (limit_ns < 1 || limit_ns > kWaitNs) return cudaErrorInvalidValue;
   bounded_wait_check_kernel<<<1, 32, 0, stream>>>(limit_ns, arrive, err, elapsed);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_mlp_start(const SceneDev& S, const BatchDev& B, int n, const PathRec* list, uint64_t first,
-                             uint64_t count, const float* Y, float* T, cudaStream_t stream) {
-  if (!count) return cudaSuccess;
-  mlp_start_kernel<<<grid_1d(count, 128, 4096), 128, 0, stream>>>(S, B, n, list, first, count, Y, T);
   count_launch();
   return cudaGetLastError();
 }

@@ -1,22 +1,31 @@
-// k_train.cu -- forward pass, loss and back-propagation of a training batch in one launch (tcgen05, CTA pairs).
+// k_train.cu -- a training step's batch in two launches (tcgen05): forward pass, loss and back-propagation on CTA
+// pairs, then the weight gradients.
 //
-// Run layer by layer, a batch of 8192 rows took 19 dependent launches a step, 64 CTAs each on 152 SMs, and
-// every hidden layer wrote its activations, their transpose and the FP32 GELU derivative to HBM and read
-// them back (15 KB per sample): 165 us a step for 7 GFLOP.  Here a cluster of two CTAs takes a tile of 128
-// rows through all layers and back.  Each CTA computes half of every hidden layer's outputs (M = 128, N = 128
-// MMAs), so the epilogues, which cost more than the MMAs, are spread over twice the SMs; it stores its
-// half of the BF16 activations into both CTAs' shared memory, where the next layer reads all of them.  The
-// derivatives stay in TMEM, in FP32, in place of the accumulators they came from: three 128-column regions
-// for the hidden layers, one for the output layer and the first back-propagated accumulator; each further
-// one takes the region whose derivative was used last.  What leaves the chip is what the weight gradients
-// read: the transposed activations and layer gradients (3 KB per sample), and the bias gradients' column
-// sums, kept per CTA until its last tile.
+// Run layer by layer, a batch of 8192 rows took 19 dependent launches a step, 64 CTAs each on 152 SMs, and every
+// hidden layer wrote its activations, their transpose and the FP32 GELU derivative to HBM and read them back (15 KB
+// per sample): 165 us a step for 7 GFLOP.
 //
-// Shared memory (220 KB, one CTA per SM): the CTA's halves of W1, W4 and W4^T for the whole launch; two 64 KB
-// buffers for W2 then W3^T, and W3 then W2^T, refilled while other layers run; 64 KB of activations.
-// The chain per tile is serial: seven MMA groups, each followed by its epilogue.  Waits are bounded as in
-// k_infer.cu.
+// mlp_train_kernel: a cluster of two CTAs takes a tile of 128 rows through all layers and back.  Each CTA computes half
+// of every hidden layer's outputs (M = 128, N = 128 MMAs), so the epilogues, which cost more than the MMAs, are spread
+// over twice the SMs.  An epilogue writes its half of the BF16 activations into its own shared memory; from there the
+// TMA engine copies it into the peer's, where the next layer reads all of it, and stores it to HBM for the weight
+// gradients, while the next layer's MMAs already run on the halves that are there.  (Threads storing to the peer and, two
+// bytes at a time, to transposed arrays in HBM took 39 us a batch of 8192; this takes 27.5.)  The derivatives stay in TMEM, in FP32, in place of
+// the accumulators they came from: three 128-column regions for the hidden layers, one for the output layer and the
+// first back-propagated accumulator; each further one takes the region whose derivative was used last.  Bias gradients
+// are column sums kept per CTA until its last tile.
+// Shared memory (220 KB, one CTA per SM): the CTA's halves of W1, W4 and W4^T for the whole launch; two 64 KB buffers
+// for W2 then W3^T, and W3 then W2^T, refilled while other layers run; 64 KB of activations.  The chain per tile is
+// serial: seven MMA groups, each followed by its epilogue; that latency bounds it (one tile per pair at 8192 rows).
+//
+// mlp_wgrad_kernel: all four weight gradients dW = dZ^T act at once, one CTA per item (128 rows of a dW, a slice of the
+// batch).  Both operands are read as they were stored, [row][column], as MN-major operands of the MMAs, so nothing is
+// transposed; partial products are added by TMA reductions.  10.8 us at 8192 rows (four GEMMs side by side 20): about
+// half of it is the start of a CTA and the reductions, the rest 48 KB of loads per 64 rows.
+//
+// Waits are bounded as in k_infer.cu.
 #include <cuda_bf16.h>
+#include <cudaTypedefs.h>
 
 #include "fpt_kernels.h"
 #include "mlp.h"
@@ -27,7 +36,7 @@ namespace fpt {
 
 constexpr int kTrainEpiWarps = 16;   // four per 32-lane quarter of TMEM, 32 of the CTA's 128 columns each
 constexpr int kTrainLoadWarps = 4;   // one thread per row
-constexpr int kTrainThreads = 32 * (kTrainEpiWarps + kTrainLoadWarps + 1);
+constexpr int kTrainThreads = 32 * (kTrainEpiWarps + kTrainLoadWarps + 2);  // + MMAs, + activation copies
 constexpr uint32_t kW4tBytes = 128 * kMlpOut * 2;
 
 struct TrainSmem {
@@ -41,11 +50,13 @@ struct TrainSmem {
   uint64_t src[128];                    // the rows' samples
   uint64_t fixed, full[2];              // weight copies
   uint64_t rows;                        // the tile's features are in act
-  uint64_t act_full;                    // both CTAs' halves of the activations are written
+  uint64_t half[2];                     // the CTA's own chunks of the activations are written,
+  uint64_t peer;                        // the peer's have arrived,
+  uint64_t stored;                      // and its own have been read by their copies to HBM
   uint64_t dy;                          // dY is written
   uint64_t tile;                        // the epilogues have read the tile's last accumulator
   uint64_t layer;                       // an MMA group of both CTAs is done
-  uint64_t act_free;                    // the tile's last MMA group of this CTA has read act
+  uint64_t act_free;                    // the tile's last layer gradient has been read
   uint64_t drain;
   uint32_t tmem;
   int fail;
@@ -116,6 +127,24 @@ __device__ __forceinline__ float row_loss(const float* t, const float* gm, const
   return acc;
 }
 
+// BF16 GELU of two accumulator values plus bias (returned) and its derivative gelu'(z) = (1 + th) / 2 + (z / 2)
+// (1 - th^2) K0 (1 + 3 K1 z^2) in FP32 (d0, d1), from one tanh each, in packed FP32 instructions.
+__device__ __forceinline__ uint32_t gelu_grad_pair(float v0, float v1, uint64_t bias, float& d0, float& d1) {
+  const uint64_t half = tc::splat2(0.5f), k0 = tc::splat2(kGeluK0);
+  const uint64_t z = tc::add2(tc::pack2(__float_as_uint(v0), __float_as_uint(v1)), bias);
+  const uint64_t z2 = tc::mul2(z, z), h = tc::mul2(half, z);
+  float u0, u1;
+  tc::unpack2(tc::mul2(z, tc::fma2(tc::splat2(kGeluK01), z2, k0)), u0, u1);
+  const uint64_t th = tc::pack2(__float_as_uint(tanh_approx(u0)), __float_as_uint(tanh_approx(u1)));
+  const uint64_t s = tc::fma2(tc::mul2(th, tc::splat2(-1.f)), th, tc::splat2(1.f));  // 1 - th^2
+  const uint64_t q = tc::fma2(tc::splat2(3.f * kGeluK1), z2, tc::splat2(1.f));
+  tc::unpack2(tc::fma2(tc::mul2(tc::mul2(h, s), k0), q, tc::fma2(half, th, half)), d0, d1);
+  float y0, y1;
+  tc::unpack2(tc::fma2(h, th, h), y0, y1);
+  const __nv_bfloat162 p = __floats2bfloat162_rn(y0, y1);
+  return *reinterpret_cast<const uint32_t*>(&p);
+}
+
 __device__ __forceinline__ void pack_bf16(const float (&x)[16], uint32_t (&w)[8]) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -128,7 +157,8 @@ __device__ __forceinline__ bool train_warp_wait(uint64_t* bar, uint32_t parity) 
   return __all_sync(0xffffffffu, tc::mbar_wait_cluster(bar, parity, kWaitNs));
 }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1) mlp_train_kernel(TrainArgs a) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
+    mlp_train_kernel(TrainArgs a, const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmZ) {
   extern __shared__ __align__(1024) unsigned char train_smem[];
   TrainSmem& sm = *reinterpret_cast<TrainSmem*>(train_smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -149,7 +179,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1) ml
     tc::mbar_init(&sm.full[0], 1);
     tc::mbar_init(&sm.full[1], 1);
     tc::mbar_init(&sm.rows, kTrainLoadWarps);
-    tc::mbar_init(&sm.act_full, 2 * kTrainEpiWarps);
+    tc::mbar_init(&sm.half[0], kTrainEpiWarps / 2);
+    tc::mbar_init(&sm.half[1], kTrainEpiWarps / 2);
+    tc::mbar_init(&sm.peer, 1);
+    tc::mbar_init(&sm.stored, 1);
     tc::mbar_init(&sm.dy, kTrainEpiWarps);
     tc::mbar_init(&sm.tile, kTrainEpiWarps);
     tc::mbar_init(&sm.layer, 2);
@@ -186,11 +219,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1) ml
     const int q = warp & 3, jc = warp >> 2;  // TMEM lane quarter; which 32 of the CTA's 128 columns
     const int row = q * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-    // this warp's 32 columns of the activations: chunk and the column within it
-    const uint32_t act_off = (2u * rank + (uint32_t)(jc >> 1)) * kMlpChunk;
-    unsigned char* act_own = sm.act + act_off;
-    const uint32_t act_peer = tc::map_rank(sm.act, rank ^ 1u) + act_off;
-    uint32_t ph_layer = 0u;
+    // this warp's 32 columns of the activations: its chunk (of the CTA's two) and the column within it
+    unsigned char* const act_own = sm.act + (2u * rank + (uint32_t)(jc >> 1)) * kMlpChunk;
+    uint32_t ph_layer = 0u, ph_stored = 0u;
+    bool first_store = true;
     float loss = 0.f;
     bool ok = true;
     auto layer_wait = [&]() {
@@ -199,46 +231,47 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1) ml
       tc::fence_after_sync();
       return ok;
     };
-    // 16 columns (step s) of the half-layer into both CTAs' activations
+    // the copies of the last activations have read them
+    auto stored_wait = [&]() {
+      if (!first_store) {
+        ok = train_warp_wait(&sm.stored, ph_stored);
+        ph_stored ^= 1u;
+      }
+      first_store = false;
+      return ok;
+    };
+    // 16 columns (step s) of the half-layer into the CTA's activations
     auto put_act = [&](int s, const uint32_t (&w)[8]) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const uint4 v = make_uint4(w[4 * h], w[4 * h + 1], w[4 * h + 2], w[4 * h + 3]);
-        const uint32_t o = tc::sw128_offset(row, (jc & 1) * 32 + 16 * s + 8 * h);
-        *reinterpret_cast<uint4*>(act_own + o) = v;
-        tc::st_cluster(act_peer + o, v);
-      }
+      for (int h = 0; h < 2; ++h)
+        *reinterpret_cast<uint4*>(act_own + tc::sw128_offset(row, (jc & 1) * 32 + 16 * s + 8 * h)) =
+            make_uint4(w[4 * h], w[4 * h + 1], w[4 * h + 2], w[4 * h + 3]);
     };
     auto act_done = [&]() {
-      tc::fence_async_all();
+      tc::fence_async_smem();
       tc::fence_before_sync();
       __syncwarp();
-      if (lane == 0) {
-        tc::mbar_arrive(&sm.act_full);
-        tc::mbar_arrive_rank(&sm.act_full, rank ^ 1u);
-      }
+      if (lane == 0) tc::mbar_arrive(&sm.half[jc >> 1]);
     };
     for (uint64_t ti = 0; ti < my_tiles && ok; ++ti) {
       const uint64_t b = (cluster + ti * n_clusters) * 128 + row;
       const bool live = b < a.B;
-      const int c0 = (int)rank * 128 + jc * 32;  // this warp's first output
 #pragma unroll 1
-      for (int l = 0; l < 3 && ok; ++l) {  // hidden layers: activation, its transpose, the derivative
-        if (!layer_wait()) break;
+      for (int l = 0; l < 3 && ok; ++l) {  // hidden layers: activation and derivative
+        if (!layer_wait() || !stored_wait()) break;
         const uint32_t acc = lane_addr + (uint32_t)(l * 128 + jc * 32);
-        __nv_bfloat16* ht = a.Ht + ((uint64_t)l * kMlpHidden + c0) * a.B + b;
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
           float z[16], d[16];
           tc::tmem_ld16(acc + 16u * s, z);
           const float* bias = sm.bias + l * 128 + jc * 32 + s * 16;
-#pragma unroll
-          for (int i = 0; i < 16; ++i) z[i] = gelu_with_grad(z[i] + bias[i], d[i]);
-          tc::tmem_st16(acc + 16u * s, d);
           uint32_t w[8];
-          pack_bf16(z, w);
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            w[i] = gelu_grad_pair(z[2 * i], z[2 * i + 1], *reinterpret_cast<const uint64_t*>(bias + 2 * i), d[2 * i],
+                                  d[2 * i + 1]);
+          tc::tmem_st16(acc + 16u * s, d);
           put_act(s, w);
-          if (live) store_transposed(ht + (uint64_t)(16 * s) * a.B, a.B, w);
         }
         act_done();
       }
@@ -249,8 +282,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1) ml
         ok = train_warp_wait(&sm.rows, (uint32_t)(ti & 1));
         if (live && ok) load_targets(a, sm.src[row], tg);
       }
-      ok = __all_sync(0xffffffffu, ok) && layer_wait();
-      if (!ok) break;
+      // (dY goes where the last activations were)
+      if (!__all_sync(0xffffffffu, ok) || !layer_wait() || !stored_wait()) {
+        ok = false;
+        break;
+      }
       if (jc == 0) {
         float y[16], g[16];
         tc::tmem_ld16(lane_addr + 384u, y);
@@ -266,7 +302,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1) ml
         *reinterpret_cast<uint4*>(sm.act + tc::kmajor_offset(row, 0, 16)) = make_uint4(w[0], w[1], w[2], w[3]);
         *reinterpret_cast<uint4*>(sm.act + tc::kmajor_offset(row, 8, 16)) = make_uint4(w[4], w[5], w[6], w[7]);
         if (rank == 0) {
-          if (live) store_transposed(a.dYt + b, a.B, w);
+          if (live) store_transposed(a.dYt + b, a.ldY, w);
           const float v = warp_colsum16(g, lane);
           if (!(lane & 1)) atomicAdd(&sm.col[384 + warp_colsum16_column(lane)], v);
         }
@@ -277,9 +313,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1) ml
       if (lane == 0) tc::mbar_arrive(&sm.dy);
 #pragma unroll 1
       for (int l = 2; l >= 0 && ok; --l) {  // layer gradients: the accumulator times the derivative in TMEM
-        if (!layer_wait()) break;
+        if (!layer_wait() || (l < 2 && !stored_wait())) break;
         const uint32_t acc = lane_addr + (uint32_t)((l + 1) * 128 + jc * 32);
-        __nv_bfloat16* zt = a.dZt + ((uint64_t)l * kMlpHidden + c0) * a.B + b;
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
           float x[16], d[16];
@@ -289,25 +324,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1) ml
           for (int i = 0; i < 16; ++i) x[i] *= d[i];
           uint32_t w[8];
           pack_bf16(x, w);
-          if (l > 0) put_act(s, w);
-          if (live) store_transposed(zt + (uint64_t)(16 * s) * a.B, a.B, w);
+          put_act(s, w);
           const float v = warp_colsum16(x, lane);
           if (!(lane & 1)) atomicAdd(&sm.col[l * 128 + jc * 32 + s * 16 + warp_colsum16_column(lane)], v);
         }
-        if (l > 0) {
-          act_done();
-        } else {
-          tc::fence_before_sync();
-          __syncwarp();
-          if (lane == 0) tc::mbar_arrive(&sm.tile);
-        }
+        act_done();
+        if (l == 0 && lane == 0) tc::mbar_arrive(&sm.tile);
       }
     }
     for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
     if (jc == 0 && rank == 0 && lane == 0) atomicAdd(a.loss, loss / (float)a.B);
     if (!ok) sm.fail = 1;
   } else if (warp < kTrainEpiWarps + kTrainLoadWarps) {
-    // ---- the tile's rows: sample numbers, features, their transpose ----
+    // ---- the tile's rows: sample numbers, features ----
     const int row = tid - 32 * kTrainEpiWarps;
     bool ok = true;
     for (uint64_t ti = 0; ti < my_tiles; ++ti) {
@@ -331,48 +360,74 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1) ml
       tc::fence_async_smem();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&sm.rows);
-      if (b < a.B) {  // each CTA writes half of the features' transpose
-        const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(f);
-        if (rank == 0) {
+      if (b < a.B) {  // each CTA writes half of the row for the weight gradient
+        uint4* xb = reinterpret_cast<uint4*>(a.Xb + b * kMlpIn);
 #pragma unroll
-          for (int k = 0; k < kMlpIn / 2; ++k) a.Xt[(uint64_t)k * a.B + b] = e[k];
-        } else {
-#pragma unroll
-          for (int k = kMlpIn / 2; k < kMlpIn; ++k) a.Xt[(uint64_t)k * a.B + b] = e[k];
-        }
+        for (int k = 0; k < kMlpIn / 16; ++k) xb[rank * (kMlpIn / 16) + k] = rank == 0 ? f[k] : f[kMlpIn / 16 + k];
       }
     }
     // the last tile's arrival too, so that none is on its way to a CTA that has left
     if (ok && my_tiles > 0) ok = train_warp_wait(&sm.act_free, (uint32_t)(my_tiles - 1) & 1u);
     if (!ok) sm.fail = 1;
+  } else if (warp == kTrainEpiWarps + kTrainLoadWarps + 1) {
+    if (lane == 0) {
+      // ---- copies of the CTA's half of the activations: to the peer for the next layer, to HBM ----
+      const uint32_t peer_act = tc::map_rank(sm.act, rank ^ 1u), peer_bar = tc::map_rank(&sm.peer, rank ^ 1u);
+      uint32_t ph = 0u;
+      bool ok = true;
+      for (uint64_t ti = 0; ti < my_tiles && ok; ++ti) {
+        const int row0 = (int)((cluster + ti * n_clusters) * 128);
+        for (int e = 0; e < 6 && ok; ++e) {  // activations of layers 1-3, layer gradients 3-1 (1 stays)
+          for (uint32_t c = 0; c < 2; ++c) {
+            if (!(ok = tc::mbar_wait(&sm.half[c], ph, kWaitNs))) break;
+            const uint32_t at = 2u * rank + c;
+            if (e < 5) tc::bulk_s2s(peer_act + at * kMlpChunk, sm.act + at * kMlpChunk, kMlpChunk, peer_bar);
+            tc::tma_store_3d(e < 3 ? &tmH : &tmZ, sm.act + at * kMlpChunk, (int)at * 64, row0, e < 3 ? e : 5 - e);
+          }
+          ph ^= 1u;
+          tc::bulk_commit();
+          tc::bulk_wait_read<0>();
+          if (!ok) break;
+          tc::mbar_arrive(&sm.stored);
+          if (e == 5) tc::mbar_arrive(&sm.act_free);
+        }
+      }
+      tc::bulk_wait_all();
+      if (!ok) sm.fail = 1;
+    }
+    __syncwarp();
   } else {
     if (lane == 0) {
-      // ---- copies and MMAs ----
+      // ---- weight copies and MMAs ----
       bool ok = tc::mbar_wait(&sm.fixed, 0u, kWaitNs);
       const uint32_t act = tc::smem_u32(sm.act);
       constexpr uint32_t id128 = tc::idesc_bf16(128, 128), id16 = tc::idesc_bf16(128, kMlpOut);
-      uint32_t ph_act = 0u, n_fill[2] = {1u, 1u}, n_full[2] = {0u, 0u};
+      uint32_t ph_half = 0u, ph_peer = 0u, n_fill[2] = {1u, 1u}, n_full[2] = {0u, 0u};
       // one 64-column chunk: four K = 16 steps
       auto chunk = [&](uint32_t d, uint32_t x, uint32_t w, uint32_t idesc, bool fresh) {
         const uint64_t ad = tc::smem_desc_sw128(x), bd = tc::smem_desc_sw128(w);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) tc::mma_bf16(d, ad + 2u * kk, bd + 2u * kk, idesc, fresh && kk == 0 ? 0u : 1u);
       };
-      auto act_wait = [&]() {
-        ok = ok && tc::mbar_wait_cluster(&sm.act_full, ph_act, kWaitNs);
-        ph_act ^= 1u;
-        tc::fence_async_all();
-        tc::fence_after_sync();
-        return ok;
+      // a layer from the activations and weights of 64-column chunks of w_stride bytes.  Columns in ascending order in
+      // both CTAs: the first CTA starts with its own half, the second waits for the first one's.
+      auto layer = [&](uint32_t d, uint32_t w, uint32_t w_stride, uint32_t idesc) {
+        tc::mbar_expect_tx(&sm.peer, 2 * kMlpChunk);
+        for (uint32_t c = 0; c < 4 && ok; ++c) {
+          ok = c / 2 == rank ? tc::mbar_wait(&sm.half[c & 1], ph_half, kWaitNs)
+                             : ((c & 1) || tc::mbar_wait_cluster(&sm.peer, ph_peer, kWaitNs));
+          if (!ok) return;
+          tc::fence_after_sync();
+          chunk(d, act + c * kMlpChunk, w + c * w_stride, idesc, c == 0);
+        }
+        ph_half ^= 1u;
+        ph_peer ^= 1u;
+        tc::mma_commit_both(&sm.layer);
       };
-      // a layer from the activations and weight buffer b
       auto buffered = [&](int b, uint32_t d) {
         ok = ok && tc::mbar_wait(&sm.full[b], n_full[b] & 1u, kWaitNs);
         ++n_full[b];
-        if (!ok) return;
-        const uint32_t w = tc::smem_u32(sm.buf[b]);
-        for (int c = 0; c < 4; ++c) chunk(d, act + c * kMlpChunk, w + c * kMlpChunk, id128, c == 0);
-        tc::mma_commit_both(&sm.layer);
+        if (ok) layer(d, tc::smem_u32(sm.buf[b]), kMlpChunk, id128);
       };
       auto refill = [&](int b, bool back) {
         fill(b, back);
@@ -388,27 +443,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1) ml
         tc::fence_after_sync();
         chunk(tmem, act, tc::smem_u32(sm.w1), id128, true);
         tc::mma_commit_both(&sm.layer);
-        if (!act_wait()) break;
         buffered(0, tmem + 128u);
-        if (!act_wait()) break;
-        refill(0, true);  // the epilogue behind this wait waited for layer 2's MMAs: W2 has been read
+        if (!ok) break;
         buffered(1, tmem + 256u);
-        if (!act_wait()) break;
+        if (!ok) break;
+        refill(0, true);  // layer 3 waited for layer 2's epilogue, and so for its MMAs: W2 has been read
+        layer(tmem + 384u, tc::smem_u32(sm.w4), kMlpW4Chunk, id16);
+        if (!ok) break;
         refill(1, true);
-        for (int c = 0; c < 4; ++c)
-          chunk(tmem + 384u, act + c * kMlpChunk, tc::smem_u32(sm.w4) + c * kMlpW4Chunk, id16, c == 0);
-        tc::mma_commit_both(&sm.layer);
         if (!(ok = tc::mbar_wait(&sm.dy, (uint32_t)(ti & 1), kWaitNs))) break;
         tc::fence_after_sync();
         tc::mma_bf16(tmem + 384u, tc::smem_desc(act, 128u, 256u), tc::smem_desc(tc::smem_u32(sm.w4t), 128u, 256u), id128,
                      0u);
         tc::mma_commit_both(&sm.layer);
-        if (!act_wait()) break;
         buffered(0, tmem + 256u);
-        if (!act_wait()) break;
-        if (more) refill(0, false);
+        if (!ok) break;
         buffered(1, tmem + 128u);
-        if (ok) tc::mma_commit(&sm.act_free);
+        if (!ok) break;
+        if (more) refill(0, false);
+        ph_half ^= 1u;  // the last layer gradient is only stored; the wait for `tile` covers it
       }
       if (!ok) {  // let the copies and MMAs in flight finish before the memory goes
         tc::mma_commit(&sm.drain);
@@ -434,6 +487,184 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1) ml
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
+// ---- weight gradients --------------------------------------------------------------------------------------
+constexpr int kWgStages = 4, kWgEpiWarps = 8, kWgThreads = 32 * (2 + kWgEpiWarps);
+constexpr uint32_t kWgBox = 64 * 128;           // 64 rows of the batch x 64 columns (128-byte swizzled)
+constexpr uint32_t kWgStage = 6 * kWgBox;       // A: 128 columns; B: up to 256
+constexpr uint32_t kWgSmem = kWgStages * kWgStage + 1024;
+
+struct WgradArgs {
+  uint64_t B;
+  int k_hidden, k_first, k_last;  // batch slices of dW2 and dW3, of dW1, of dW4
+  float* grad;
+  int* err;
+};
+
+// Descriptor of an MN-major operand: boxes of 64 columns (the M or N dimension) x 64 rows (K), 128-byte swizzled;
+// the next 64 columns one box further, the next 8 rows 1024 bytes.
+__device__ __forceinline__ uint64_t wg_desc_mn(uint32_t saddr) {
+  uint64_t d = tc::smem_desc_sw128(saddr);
+  d &= ~((uint64_t)0x3FFFu << 16);
+  return d | (uint64_t)(kWgBox >> 4) << 16;
+}
+
+__global__ void __launch_bounds__(kWgThreads, 1)
+    mlp_wgrad_kernel(WgradArgs a, const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmZ,
+                     const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmY,
+                     const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2,
+                     const __grid_constant__ CUtensorMap tmW3) {
+  extern __shared__ unsigned char wg_raw[];
+  __shared__ __align__(8) uint64_t full[kWgStages], empty[kWgStages], acc_full;
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_fail;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned char* ring = wg_raw + ((1024u - (tc::smem_u32(wg_raw) & 1023u)) & 1023u);
+  // this CTA's item: layer gradient `job` (3, 2, 1: dW3, dW2, dW1; 4: dW4), rows m0 .. m0 + 127, slice of the batch
+  int job, m0, slice, slices;
+  {
+    int i = blockIdx.x;
+    if (i < 4 * a.k_hidden) {
+      slices = a.k_hidden;
+      job = i < 2 * slices ? 3 : 2;
+      i -= job == 3 ? 0 : 2 * slices;
+    } else if (i < 4 * a.k_hidden + 2 * a.k_first) {
+      slices = a.k_first;
+      job = 1;
+      i -= 4 * a.k_hidden;
+    } else {
+      slices = a.k_last;
+      job = 4;
+      i -= 4 * a.k_hidden + 2 * a.k_first;
+    }
+    m0 = i < slices ? 0 : 128;
+    slice = i < slices ? i : i - slices;
+  }
+  const int total = (int)((a.B + 63) / 64), per = (total + slices - 1) / slices;
+  const int first = slice * per, last = first + per < total ? first + per : total;
+  if (first >= last) return;  // (the whole CTA)
+  const int count = last - first;
+  const int n_cols = job == 4 ? kMlpOut : (job == 1 ? kMlpIn : kMlpHidden);
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kWgStages; ++s) {
+      tc::mbar_init(&full[s], 1);
+      tc::mbar_init(&empty[s], 1);
+    }
+    tc::mbar_init(&acc_full, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_fail = 0;
+  }
+  __syncwarp();
+  if (warp == 0) {
+    tc::tmem_alloc(&s_tmem, 256);
+    tc::tmem_relinquish();
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = s_tmem;
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---- loads ----
+      const uint32_t bytes = 2 * kWgBox + (job == 4 ? kMlpOut * 128u : (uint32_t)n_cols * 128u);
+      bool ok = true;
+      int q = 0;
+      for (; q < count; ++q) {
+        const int s = q % kWgStages, u = q / kWgStages;
+        if (u > 0 && !(ok = tc::mbar_wait(&empty[s], (uint32_t)(u - 1) & 1u, kWaitNs))) break;
+        unsigned char* st = ring + s * kWgStage;
+        const int b0 = (first + q) * 64;
+        tc::mbar_expect_tx(&full[s], bytes);
+        for (int k = 0; k < 2; ++k)
+          tc::tma_load_3d(st + k * kWgBox, job == 4 ? &tmH : &tmZ, m0 + 64 * k, b0, job == 4 ? 2 : job - 1, &full[s]);
+        if (job == 4) {
+          tc::tma_load_2d(st + 2 * kWgBox, &tmY, b0, 0, &full[s]);
+        } else if (job == 1) {
+          tc::tma_load_2d(st + 2 * kWgBox, &tmX, 0, b0, &full[s]);
+        } else {
+          for (int k = 0; k < 4; ++k) tc::tma_load_3d(st + (2 + k) * kWgBox, &tmH, 64 * k, b0, job - 2, &full[s]);
+        }
+      }
+      if (!ok) {  // the loads in flight finish before the memory goes
+        s_fail = 1;
+        for (int p = q > kWgStages ? q - kWgStages : 0; p < q; ++p)
+          tc::mbar_wait(&full[p % kWgStages], (uint32_t)(p / kWgStages) & 1u, kWaitNs);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // ---- MMAs: A MN-major; B MN-major, but dY, which is stored transposed, K-major ----
+      const uint32_t idesc = tc::idesc_bf16(128, (uint32_t)n_cols) | 1u << 15 | (job == 4 ? 0u : 1u << 16);
+      bool ok = true;
+      for (int q = 0; q < count; ++q) {
+        const int s = q % kWgStages, u = q / kWgStages;
+        if (!(ok = tc::mbar_wait(&full[s], (uint32_t)u & 1u, kWaitNs))) break;
+        tc::fence_after_sync();
+        const uint32_t st = tc::smem_u32(ring + s * kWgStage);
+        const uint64_t ad = wg_desc_mn(st);
+        const uint64_t bd = job == 4 ? tc::smem_desc_sw128(st + 2 * kWgBox) : wg_desc_mn(st + 2 * kWgBox);
+        const uint32_t bstep = job == 4 ? 2u : 128u;  // 16 rows of the batch: 32 bytes K-major, 2048 MN-major
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) tc::mma_bf16(tmem, ad + 128u * kk, bd + bstep * kk, idesc, (q | kk) ? 1u : 0u);
+        tc::mma_commit(&empty[s]);
+      }
+      if (!ok) {  // before the epilogue can see the barrier
+        *reinterpret_cast<volatile int*>(&s_fail) = 1;
+        __threadfence_block();
+      }
+      tc::mma_commit(&acc_full);
+      if (!ok) tc::mbar_wait(&acc_full, 0u, kWaitNs);
+    }
+    __syncwarp();
+  } else {
+    // ---- the partial product into the gradient ----
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&acc_full, 0u, kWaitNs)) &&
+                    *reinterpret_cast<volatile int*>(&s_fail) == 0;
+    tc::fence_after_sync();
+    const uint32_t acc = tmem + ((uint32_t)(q * 32) << 16);
+    if (ok && job == 4) {
+      if (half == 0) {
+        float v[16];
+        tc::tmem_ld16(acc, v);
+#pragma unroll
+        for (int o = 0; o < kMlpOut; ++o) atomicAdd(a.grad + kOffW4 + o * kMlpHidden + m0 + q * 32 + lane, v[o]);
+      }
+    } else if (ok) {
+      // 32 x 32 boxes, staged where the operands were (every MMA has read them), added by the TMA engine
+      unsigned char* stg = ring + (warp - 2) * 4 * 4096;
+      const int boxes = n_cols / 64;  // per half
+      for (int k = 0; k < boxes; ++k) {
+        const int n0 = (half * boxes + k) * 32;
+        unsigned char* box = stg + k * 4096;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          float v[16];
+          tc::tmem_ld16(acc + (uint32_t)(n0 + 16 * c), v);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            *reinterpret_cast<float4*>(box + lane * 128 + (((4 * c + i) ^ (lane & 7)) << 4)) =
+                make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        }
+        tc::fence_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          tc::tma_reduce_add_2d(job == 3 ? &tmW3 : (job == 2 ? &tmW2 : &tmW1), box, n0, m0 + q * 32);
+          tc::bulk_commit();
+        }
+      }
+      if (lane == 0) tc::bulk_wait_all();
+      __syncwarp();
+    }
+    if (!ok && lane == 0) s_fail = 1;
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (s_fail && threadIdx.x == 0 && a.err) atomicCAS(a.err, 0, ERR_MMA_TIMEOUT);
+  __syncwarp();
+  if (warp == 0) tc::tmem_dealloc(tmem, 256);
+}
+
 cudaError_t launch_mlp_train(const TrainArgs& args, cudaStream_t stream, int n_sm) {
   TrainArgs a = args;
   if (!a.B) return cudaSuccess;
@@ -444,9 +675,39 @@ cudaError_t launch_mlp_train(const TrainArgs& args, cudaStream_t stream, int n_s
   while ((1ULL << (2 * a.h)) < a.n) ++a.h;
   const int smem = (int)sizeof(TrainSmem);
   cudaError_t e = cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
   if (e != cudaSuccess) return e;
+  // H and dZ [3][B][256], X [B][64], dY^T [16][ldY]; the FP32 gradients
+  CUtensorMap st_h, st_z, ld_h, ld_z, ld_x, ld_y, w[3];
+  constexpr auto kBf16 = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+  constexpr auto kSw = CU_TENSOR_MAP_SWIZZLE_128B;
+  const cuuint64_t hd[3] = {kMlpHidden, a.B, 3}, hs[2] = {kMlpHidden * 2, a.B * kMlpHidden * 2};
+  const cuuint64_t xd[2] = {kMlpIn, a.B}, xs[1] = {kMlpIn * 2}, yd[2] = {a.B, kMlpOut}, ys[1] = {a.ldY * 2};
+  const cuuint32_t st_box[3] = {64, 128, 1}, ld_box[3] = {64, 64, 1}, y_box[2] = {64, kMlpOut}, w_box[2] = {32, 32};
+  bool ok = encode_map(&st_h, kBf16, 3, a.H, hd, hs, st_box, kSw) && encode_map(&st_z, kBf16, 3, a.dZ, hd, hs, st_box, kSw) &&
+            encode_map(&ld_h, kBf16, 3, a.H, hd, hs, ld_box, kSw) && encode_map(&ld_z, kBf16, 3, a.dZ, hd, hs, ld_box, kSw) &&
+            encode_map(&ld_x, kBf16, 2, a.Xb, xd, xs, ld_box, kSw) && encode_map(&ld_y, kBf16, 2, a.dYt, yd, ys, y_box, kSw);
+  for (int l = 0; l < 3; ++l) {
+    const int K = l == 0 ? kMlpIn : kMlpHidden, off = l == 0 ? kOffW1 : (l == 1 ? kOffW2 : kOffW3);
+    const cuuint64_t wd[2] = {(cuuint64_t)K, kMlpHidden}, ws[1] = {(cuuint64_t)K * 4};
+    ok = ok && encode_map(&w[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, a.grad + off, wd, ws, w_box, kSw);
+  }
+  if (!ok) return cudaErrorInvalidValue;
   const uint64_t tiles = (a.B + 127) / 128, cap = (uint64_t)(n_sm > 1 ? n_sm / 2 : 1);
-  mlp_train_kernel<<<2u * (unsigned)(tiles < cap ? tiles : cap), kTrainThreads, smem, stream>>>(a);
+  mlp_train_kernel<<<2u * (unsigned)(tiles < cap ? tiles : cap), kTrainThreads, smem, stream>>>(a, st_h, st_z);
+  count_launch();
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  // One item per SM.  An item of dW2 or dW3 loads 48 KB per 64 rows and adds 128 KB, one of dW1 24 and 32 KB, one of
+  // dW4 18 and 8 KB: 28, 12 and 8 slices of 152 items make them about equal at 8192 rows.
+  const int stages = (int)((a.B + 63) / 64);
+  auto share = [&](int part) {
+    const int k = n_sm * part / 152;
+    return k < 1 ? 1 : (k < stages ? k : stages);
+  };
+  const WgradArgs g{a.B, share(28), share(12), share(8), a.grad, a.err};
+  mlp_wgrad_kernel<<<4 * g.k_hidden + 2 * g.k_first + 2 * g.k_last, kWgThreads, kWgSmem, stream>>>(
+      g, ld_h, ld_z, ld_x, ld_y, w[0], w[1], w[2]);
   count_launch();
   return cudaGetLastError();
 }

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -15,9 +16,7 @@ constexpr int kOffW1 = 0, kOffB1 = kOffW1 + 256 * 64, kOffW2 = kOffB1 + 256, kOf
               kOffW3 = kOffB2 + 256, kOffB3 = kOffW3 + 256 * 256, kOffW4 = kOffB3 + 256, kOffB4 = kOffW4 + 16 * 256,
               kMlpParams = kOffB4 + 16;
 
-// EPI_ATOMIC adds the product into C: the split-K partial products of the weight gradients, one per
-// CTA, go in by TMA tensor reduce-adds (row- or column-major C), else by atomics.
-enum EpilogueOp { EPI_STORE = 0, EPI_ATOMIC = 1, EPI_BIAS_GELU = 2, EPI_GELU_GRAD = 3 };
+enum EpilogueOp { EPI_STORE = 0, EPI_BIAS_GELU = 1 };
 
 // D[M x N] = sum_k A(m, k) B(n, k); A(m, k) = A[m * sam + k * sak], B(n, k) = B[n * sbn + k * sbk].
 struct GemmArgs {
@@ -27,20 +26,18 @@ struct GemmArgs {
   const __nv_bfloat16* B;
   long long sbn, sbk;
   int op;                 // EpilogueOp
-  const float* bias;      // [N] (EPI_STORE, EPI_BIAS_GELU) or null
-  float* C;               // FP32 output: D (+bias) / gelu'(pre-activation) (EPI_BIAS_GELU) / dZ, or null where optional
+  const float* bias;      // [N] or null
+  float* C;               // EPI_STORE: FP32 output, D (+ bias)
   long long scm, scn;
-  __nv_bfloat16* H;       // BF16 output: activation (EPI_BIAS_GELU) or dZ (EPI_GELU_GRAD)
+  __nv_bfloat16* H;       // EPI_BIAS_GELU: BF16 activation
   long long shm, shn;
-  __nv_bfloat16* Ht;      // optional second copy of H with its own strides (the transpose, for the backward)
-  long long shtm, shtn;
-  const float* Zin;       // EPI_GELU_GRAD: gelu' at the pre-activation, as the forward's EPI_BIAS_GELU wrote it
-  long long szm, szn;
-  float* colsum;          // EPI_GELU_GRAD: the column sums of the FP32 result are added here ([N]), or null
   int* err;               // device error word (MMA completion timeout)
 };
 
-cudaError_t launch_gemm(const GemmArgs& g, int k_split, cudaStream_t stream);
+// A tiled tensor map (false where the base or a stride does not allow one).
+bool encode_map(CUtensorMap* map, CUtensorMapDataType type, int rank, const void* base, const cuuint64_t* dims,
+                const cuuint64_t* strides, const cuuint32_t* box, CUtensorMapSwizzle swizzle);
+cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t stream);
 cudaError_t launch_mlp_features(const SceneDev& S, const BatchDev& B, int n, const PathRec* list, uint64_t first,
                                 uint64_t count, float inv_scale, __nv_bfloat16* X, float* G, cudaStream_t stream);
 // One Adam step, with the BF16 copies of the parameters (plain and as launch_mlp_tile_weights lays them out); with
@@ -61,10 +58,10 @@ constexpr uint32_t kMlpHalfTBytes = 8 * kMlpChunk + 128 * 16 * 2;
 // both from the BF16 parameter copy
 cudaError_t launch_mlp_tile_weights(const __nv_bfloat16* wb, __nv_bfloat16* wt, __nv_bfloat16* wtT,
                                     cudaStream_t stream);
-// Forward pass, loss and back-propagation of B rows.  Row i is sample perm(first + i) of n when n > 0 (perm = the
-// seeded permutation of [0, n) drawn by key), else sample i.  Written: the transposed features [64][B], hidden
-// activations [3][256][B] and gradients at the layers' outputs dZ [3][256][B], dY [16][B]; added: the bias
-// gradients (at their places in grad) and the mean loss.
+// Loss and gradient of B rows (two launches).  Row i is sample perm(first + i) of n when n > 0 (perm = the seeded
+// permutation of [0, n) drawn by key), else sample i.  grad and loss are added to.  Scratch: the rows' features
+// [B][64], hidden activations and gradients at the hidden layers' outputs [3][B][256], transposed gradient at the
+// outputs [16][ldY] (ldY >= B, a multiple of 8).
 struct TrainArgs {
   const __nv_bfloat16* X;
   const float* T;
@@ -72,7 +69,8 @@ struct TrainArgs {
   uint64_t B, n, first, key;
   const __nv_bfloat16 *wt, *wtT;
   const float* params;
-  __nv_bfloat16 *Xt, *Ht, *dZt, *dYt;
+  __nv_bfloat16 *Xb, *H, *dZ, *dYt;
+  uint64_t ldY;
   float *grad, *loss;
   int* err;
   int h, vec_x, vec_tg;  // set by the launch: half the permutation's bits, 16-byte alignment of X, of T and G
@@ -89,7 +87,5 @@ cudaError_t launch_mlp_infer(const SceneDev& S, const BatchDev& B, int n, const 
 // (device, optional) receives the wait's duration in nanoseconds of the global timer.
 cudaError_t launch_bounded_wait_check(uint32_t limit_ns, int arrive, int* err, unsigned long long* elapsed,
                                       cudaStream_t stream);
-cudaError_t launch_mlp_start(const SceneDev& S, const BatchDev& B, int n, const PathRec* list, uint64_t first,
-                             uint64_t count, const float* Y, float* T, cudaStream_t stream);
 
 }  // namespace fpt

@@ -11,7 +11,6 @@
 
 namespace fpt {
 
-
 constexpr uint32_t kWaitNs = 1000000000u;   // mbarrier waits give up after 1 s
 constexpr int ERR_MMA_TIMEOUT = 3;
 
@@ -33,17 +32,6 @@ constexpr float kGeluK01 = 0.0356774081363001f;  // K0 K1
 __device__ __forceinline__ float gelu(float z) {
   const float h = 0.5f * z;
   return fmaf(h, tanh_approx(z * fmaf(kGeluK01, z * z, kGeluK0)), h);
-}
-
-// gelu(z) and, in d, its derivative gelu'(z) = (1 + th) / 2 + (z / 2) (1 - th^2) K0 (1 + 3 K1 z^2), from one
-// tanh.  The training forward keeps gelu'(Z) for the backward (dZ = dH gelu'(Z)), so the backward's
-// epilogue multiplies instead of evaluating the derivative again.
-__device__ __forceinline__ float gelu_with_grad(float z, float& d) {
-  const float z2 = z * z;
-  const float th = tanh_approx(z * fmaf(kGeluK01, z2, kGeluK0));
-  const float h = 0.5f * z;
-  d = 0.5f * (1.f + th) + 0.5f * z * (1.f - th * th) * kGeluK0 * fmaf(3.f * kGeluK1, z2, 1.f);
-  return fmaf(h, th, h);
 }
 
 // Sum of x[i] over the warp's 32 lanes for each of the 16 columns i: a transposing butterfly (16 shuffles).

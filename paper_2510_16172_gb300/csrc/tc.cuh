@@ -125,19 +125,10 @@ __device__ __forceinline__ uint32_t map_rank(const void* p, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
   return a;
 }
-__device__ __forceinline__ void st_cluster(uint32_t addr, const uint4& v) {
-  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
-               : "memory");
-}
-// One arrival on CTA `rank`'s barrier at this shared-memory offset, releasing this thread's writes to the cluster
-// (the release waits for every earlier store of the thread: 400-850 cycles measured on a GB300).
-__device__ __forceinline__ void mbar_arrive_rank(uint64_t* bar, uint32_t rank) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(map_rank(bar, rank)) : "memory");
-}
-// The same without that wait: it orders this thread's earlier writes for its own CTA only.  Enough where the other CTA's
-// thread goes on to issue an MMA whose operands the writers' proxy fence has already made visible to the tensor core
-// that reads them, each CTA's own shared memory.
-// addr: the barrier's address from map_rank.
+// One arrival on another CTA's barrier (addr from map_rank), ordering this thread's earlier writes for its own CTA
+// only: enough where the other CTA's thread goes on to issue an MMA whose operands the writers' proxy fence has made
+// visible to the tensor core that reads them, each CTA's own shared memory.  (A release to the cluster waits for
+// every earlier store of the thread: 400-850 cycles measured.)
 __device__ __forceinline__ void mbar_arrive_remote_cta(uint32_t addr) {
   asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
@@ -180,12 +171,26 @@ __device__ __forceinline__ void tma_load_2d(void* dst_smem, const void* tmap, in
       : "memory");
 }
 
+// The same from a 3-D tensor map.
+__device__ __forceinline__ void tma_load_3d(void* dst_smem, const void* tmap, int x, int y, int z, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
+          "r"(smem_u32(dst_smem)),
+      "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
+      : "memory");
+}
+
 // Shared -> global tile stores by the TMA engine (bulk-group completion; the source box must not be
 // rewritten before cp.async.bulk.wait_group.read says the engine has read it).  The innermost
 // coordinate times the element size must be a multiple of 16 bytes, and no coordinate may be negative.
 __device__ __forceinline__ void tma_store_2d(const void* tmap, const void* src_smem, int x, int y) {
   asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(tmap), "r"(x),
                "r"(y), "r"(smem_u32(src_smem))
+               : "memory");
+}
+__device__ __forceinline__ void tma_store_3d(const void* tmap, const void* src_smem, int x, int y, int z) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(tmap), "r"(x),
+               "r"(y), "r"(z), "r"(smem_u32(src_smem))
                : "memory");
 }
 // The same box added element by element to global memory (the tensor map's element type; FP32 here) by the
@@ -214,11 +219,18 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, u
       : "memory");
 }
 
+// Shared memory of this CTA -> another CTA's of the cluster (addresses from map_rank), completing `bytes` transactions
+// on a barrier there.
+__device__ __forceinline__ void bulk_s2s(uint32_t dst, const void* src_smem, uint32_t bytes, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+      "r"(smem_u32(src_smem)), "r"(bytes), "r"(bar)
+      : "memory");
+}
+
 // ---- fences ----------------------------------------------------------------
 // generic-proxy writes to shared memory become visible to the tensor core
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-// the same for writes to the cluster's other CTAs too
-__device__ __forceinline__ void fence_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 __device__ __forceinline__ void fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
