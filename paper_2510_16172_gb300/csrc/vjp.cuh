@@ -19,7 +19,7 @@ __device__ __forceinline__ bool has_point_cotangent(const float* __restrict__ dX
   const float* p = dX + g * (uint64_t)n_max * 3;
   bool any = false;
 #pragma unroll
-  for (int k = 0; k < 3 * N; ++k) any = any || p[k] != 0.f;
+  for (int k = 0; k < 3 * N; ++k) any |= p[k] != 0.f;  // no early exit: the loads are independent
   return any;
 }
 
