@@ -470,7 +470,7 @@ def occlusion(ctx: Context, scene: Scene, batch: Batch, T, status=None, status_m
     _need_cuda(T, torch.float32, "T")
     _need_cuda(status, torch.uint8, "status")
     if out is None:
-        out = torch.zeros(batch.n_paths, dtype=torch.int16, device=T.device)
+        out = torch.empty(batch.n_paths, dtype=torch.int16, device=T.device)  # every path is written
     _need_cuda(out, torch.int16, "out")
     if out.numel() != batch.n_paths or T.numel() != batch.n_paths * batch.n_max * 2:
         raise FptError("T must be [N, n_max, 2] and out [N] for the batch")

@@ -96,3 +96,25 @@ def test_status_mask_and_arguments(ctx):
         fpt.occlusion(ctx, scene, batch, out["T"], tol=-1.0)
     with pytest.raises(fpt.FptError):
         fpt.occlusion(ctx, scene, batch, out["T"], out=torch.zeros(3, dtype=torch.int16, device="cuda"))
+
+
+@pytest.mark.parametrize("rx_grid,lo,shift", [(1, 1, 0), (3, 2, 0), (3, 3, 1), (2, 1, 1)])
+def test_listed_paths_match_every_path(ctx, rx_grid, lo, shift):
+    """The masks of the listed paths equal those of a call that tests every path, the others are zero: slices of one and
+    of several TX/RX pairs, with statuses and masks on 16-byte boundaries (read and cleared 16 at a time) and off them."""
+    import torch
+
+    sc = scenes.urban_canyon(2, rx_grid=rx_grid)
+    scene = fpt.Scene(ctx, sc.types, sc.verts, sc.tx, sc.rx)
+    batch = fpt.Batch.exhaustive(ctx, scene, lo, 3, sc.alphabet)
+    out = fpt.solve(ctx, scene, batch)
+    mask = fpt.ST_VALID | fpt.ST_SOLVED
+    buf = torch.zeros(batch.n_paths + shift, dtype=torch.uint8, device="cuda")
+    buf[shift:] = out["status"]
+    status = buf[shift:]
+    every = fpt.occlusion(ctx, scene, batch, out["T"])
+    listed = fpt.occlusion(ctx, scene, batch, out["T"], status, mask)
+    ctx.sync()
+    take = (status & mask) == mask
+    assert bool(take.any())
+    assert torch.equal(listed.int(), torch.where(take, every.int(), torch.zeros_like(every.int())))
