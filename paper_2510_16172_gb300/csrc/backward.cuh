@@ -22,47 +22,66 @@
 namespace fpt {
 
 // Paths with point cotangents are not listed beforehand: each CTA scans its share of the slice for the paths that
-// carry a cotangent (kScanRounds kThreads consecutive ones at a time, a lane per path) into a queue in shared memory, in index
-// order, and takes a full CTA of them at a time.  A loss on the valid paths of a canyon touches 7 % of them; one
+// carry a cotangent (kScanRounds kThreads consecutive ones at a time, a lane per path) into a queue in shared memory, in
+// index order, and takes a full CTA of them at a time.  A loss on the valid paths of a canyon touches 7 % of them; one
 // thread per path of the slice left nearly every warp running the whole adjoint for two lanes.
 // Measured on 2.16 M canyon paths of orders 1-3 with point and length cotangents on the valid ones:
-// 194 -> 126 us a call.
+// 194 -> 95 us a call (126 before the loads of four rounds went out together).
 // (One round at a time where the slice is too small to give every CTA of the launch four.)
 constexpr int kScanRounds = 4, kQueue = 1024;
 static_assert((kScanRounds + 2) * kThreads <= kQueue, "queue entries");
 
-// Appends the paths of [scan, scan + rounds kThreads) that carry a cotangent to the queue (its entries end at slot `end`); every
-// thread of the CTA calls it and gets their number.
+// Appends the paths of [scan, scan + rounds kThreads) that carry a cotangent to the queue (its entries end at slot
+// `end`); every thread of the CTA calls it and gets their number.
 template <int N>
 __device__ __forceinline__ unsigned backward_scan(const BatchDev& B, const BackwardCfg& cfg, uint64_t scan,
                                                   uint64_t n_local, const PathRec* __restrict__ list,
                                                   const uint8_t* __restrict__ status, const float* __restrict__ dX,
-                                                  const float* __restrict__ dLv, uint32_t* queue, unsigned end, int rounds) {
+                                                  const float* __restrict__ dLv, uint32_t* queue, unsigned end,
+                                                  int rounds) {
   __shared__ unsigned s_cnt[kScanRounds][kThreads / 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned votes[kScanRounds];
+  // the loads of one kind for all rounds together: the scan is bound by their latency
+  uint64_t g[kScanRounds];
+  unsigned st[kScanRounds];
+  float dl[kScanRounds];
 #pragma unroll
   for (int r = 0; r < kScanRounds; ++r) {
     const uint64_t j = scan + (uint64_t)(r * kThreads) + threadIdx.x;
-    bool take = false;
-    if (r < rounds && j < n_local) {
-      uint64_t g;
-      uint8_t st;
-      if (status) {  // the solver wrote the sequence's REPEAT / INVALID_INPUT bits into its status
-        g = slice_global(B, N, list, j);
-        st = status[g];
-      } else {
-        PathDesc d;
-        fetch_path_n<N>(B, list, j, d);
-        g = d.g;
-        st = d.flags;
-      }
-      if (!(st & (ST_REPEAT | ST_INVALID | ST_DEGENERATE | ST_NONFINITE))) {
-        const float dl = dLv ? dLv[g] : ((cfg.dl_mask && (st & cfg.dl_mask) == cfg.dl_mask) ? 1.f : 0.f);
-        take = dl != 0.f || has_point_cotangent<N>(dX, g, B.n_max);
-      }
+    const bool have = r < rounds && j < n_local;
+    g[r] = 0;
+    st[r] = ST_REPEAT;
+    if (have && status) {  // the solver wrote the sequence's REPEAT / INVALID_INPUT bits into its status
+      g[r] = slice_global(B, N, list, j);
+    } else if (have) {
+      PathDesc d;
+      fetch_path_n<N>(B, list, j, d);
+      g[r] = d.g;
+      st[r] = d.flags;
     }
-    votes[r] = __ballot_sync(0xffffffffu, take);
+  }
+  if (status) {
+#pragma unroll
+    for (int r = 0; r < kScanRounds; ++r)
+      if (r < rounds && scan + (uint64_t)(r * kThreads) + threadIdx.x < n_local) st[r] = status[g[r]];
+  }
+#pragma unroll
+  for (int r = 0; r < kScanRounds; ++r) {
+    const bool part = !(st[r] & (ST_REPEAT | ST_INVALID | ST_DEGENERATE | ST_NONFINITE));
+    dl[r] = !dLv && cfg.dl_mask && (st[r] & cfg.dl_mask) == cfg.dl_mask ? 1.f : 0.f;
+    if (part && dLv) dl[r] = dLv[g[r]];
+    st[r] = part ? 1u : 0u;
+  }
+  bool take[kScanRounds];
+#pragma unroll
+  for (int r = 0; r < kScanRounds; ++r) {
+    take[r] = st[r] && dl[r] != 0.f;
+    if (st[r] && !take[r]) take[r] = has_point_cotangent<N>(dX, g[r], B.n_max);
+  }
+  unsigned votes[kScanRounds];
+#pragma unroll
+  for (int r = 0; r < kScanRounds; ++r) {
+    votes[r] = __ballot_sync(0xffffffffu, take[r]);
     if (lane == 0) s_cnt[r][warp] = (unsigned)__popc(votes[r]);
   }
   __syncthreads();
@@ -82,8 +101,12 @@ __device__ __forceinline__ unsigned backward_scan(const BatchDev& B, const Backw
   return total;
 }
 
+// CTAs per SM the registers are bounded for, none with spills: what each order had before the scan was part of it.
 template <int N>
-__global__ void __launch_bounds__(kThreads) backward_kernel(SceneDev S, BatchDev B, BackwardCfg cfg,
+constexpr int kBackwardMinCtas = N == 1 ? 8 : (N == 2 ? 5 : (N == 3 ? 4 : (N == 4 ? 3 : (N == 5 ? 2 : 1))));
+
+template <int N>
+__global__ void __launch_bounds__(kThreads, kBackwardMinCtas<N>) backward_kernel(SceneDev S, BatchDev B, BackwardCfg cfg,
                                                             uint64_t n_local, const PathRec* __restrict__ list,
                                                             const float* __restrict__ T,
                                                             const uint8_t* __restrict__ status,
