@@ -407,14 +407,20 @@ cudaError_t launch_backward_rescue_n(const SceneDev& S, const BatchDev& B, const
   return cudaGetLastError();
 }
 
+// Slices up to this many paths per SM (four CTAs' worth of threads) are scanned by the adjoint's own CTAs also where
+// only length cotangents are given: the select pass, 16 paths per thread, has too few threads there and is one more link
+// of the order's chain.  Scanned against listed, whole solve with gradient: 5,000 paths per order (1-4) 110 / 121 us,
+// 50,000 168 / 180, 200,000 442 / 436, 1.6 M city paths per order 5281 / 5260, 33.5 M canyon paths 12,380 / 11,774.
+constexpr uint64_t kScanMaxPerSm = 4 * kThreads;
 template <int N>
 cudaError_t launch_backward_n(const SceneDev& S, const BatchDev& B, const BackwardCfg& cfg_in,
                                      uint64_t n_local, const PathRec* list, const float* T, const uint8_t* status,
                                      const float* dX, const float* dL, double* gacc, cudaStream_t stream, int n_sm,
                                      uint32_t* rescue_list, unsigned* rescue_count) {
   BackwardCfg cfg = cfg_in;
-  if (dX != nullptr || cfg.sel == nullptr || cfg.sel_count == nullptr) {
-    cfg.sel = nullptr;  // point cotangents, or no room for a list: the kernel scans for the paths with a cotangent
+  if (dX != nullptr || cfg.sel == nullptr || cfg.sel_count == nullptr ||
+      n_local <= (uint64_t)n_sm * kScanMaxPerSm) {
+    cfg.sel = nullptr;  // the kernel scans for the paths with a cotangent
     cfg.sel_count = nullptr;
   } else {
     const uint64_t want = (n_local + kSelChunk - 1) / kSelChunk;
