@@ -10,7 +10,7 @@
 // over twice the SMs.  An epilogue writes its half of the BF16 activations into its own shared memory; from there the
 // TMA engine copies it into the peer's, where the next layer reads all of it, and stores it to HBM for the weight
 // gradients, while the next layer's MMAs already run on the halves that are there.  (Threads storing to the peer and, two
-// bytes at a time, to transposed arrays in HBM took 39 us a batch of 8192; this takes 27.5.)  The derivatives stay in TMEM, in FP32, in place of
+// bytes at a time, to transposed arrays in HBM took 39 us a batch of 8192; this takes 25.4.)  The derivatives stay in TMEM, in FP32, in place of
 // the accumulators they came from: three 128-column regions for the hidden layers, one for the output layer and the
 // first back-propagated accumulator; each further one takes the region whose derivative was used last.  Bias gradients
 // are column sums kept per CTA until its last tile.
@@ -34,7 +34,7 @@
 
 namespace fpt {
 
-constexpr int kTrainEpiWarps = 16;   // four per 32-lane quarter of TMEM, 32 of the CTA's 128 columns each
+constexpr int kTrainEpiWarps = 16;   // four per 32-lane quarter of TMEM, 16 columns of each of the CTA's two chunks each
 constexpr int kTrainLoadWarps = 4;   // one thread per row
 constexpr int kTrainThreads = 32 * (kTrainEpiWarps + kTrainLoadWarps + 2);  // + MMAs, + activation copies
 constexpr uint32_t kW4tBytes = 128 * kMlpOut * 2;
@@ -51,7 +51,7 @@ struct TrainSmem {
   uint64_t fixed, full[2];              // weight copies
   uint64_t rows;                        // the tile's features are in act
   uint64_t half[2];                     // the CTA's own chunks of the activations are written,
-  uint64_t peer;                        // the peer's have arrived,
+  uint64_t peer[2];                     // the peer's have arrived,
   uint64_t stored;                      // and its own have been read by their copies to HBM
   uint64_t dy;                          // dY is written
   uint64_t tile;                        // the epilogues have read the tile's last accumulator
@@ -179,9 +179,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
     tc::mbar_init(&sm.full[0], 1);
     tc::mbar_init(&sm.full[1], 1);
     tc::mbar_init(&sm.rows, kTrainLoadWarps);
-    tc::mbar_init(&sm.half[0], kTrainEpiWarps / 2);
-    tc::mbar_init(&sm.half[1], kTrainEpiWarps / 2);
-    tc::mbar_init(&sm.peer, 1);
+    tc::mbar_init(&sm.half[0], kTrainEpiWarps);
+    tc::mbar_init(&sm.half[1], kTrainEpiWarps);
+    tc::mbar_init(&sm.peer[0], 1);
+    tc::mbar_init(&sm.peer[1], 1);
     tc::mbar_init(&sm.stored, 1);
     tc::mbar_init(&sm.dy, kTrainEpiWarps);
     tc::mbar_init(&sm.tile, kTrainEpiWarps);
@@ -208,6 +209,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
     tc::tmem_alloc(&sm.tmem, 512);
     tc::tmem_relinquish();
   }
+  // loader warps: a row's sample and features; the first tile's on the way while the CTA sets up
+  const int load_row = tid - 32 * kTrainEpiWarps;
+  uint4 f[kMlpIn / 8];
+  uint64_t src = 0;
+  auto load_rows = [&](uint64_t ti) {
+    const uint64_t b = (cluster + ti * n_clusters) * 128 + load_row;
+    src = 0;
+#pragma unroll
+    for (int k = 0; k < kMlpIn / 8; ++k) f[k] = make_uint4(0u, 0u, 0u, 0u);
+    if (b < a.B) {
+      src = a.n ? perm_index(a.first + b, a.n, a.h, a.key) : b;
+      load_features(a, src, f);
+    }
+  };
+  if (warp >= kTrainEpiWarps && warp < kTrainEpiWarps + kTrainLoadWarps && my_tiles > 0) load_rows(0);
   tc::fence_before_sync();
   __syncthreads();
   tc::cluster_sync();  // the peer's barriers are initialised before anything arrives on them
@@ -216,11 +232,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
 
   if (warp < kTrainEpiWarps) {
     // ---- epilogues ----
-    const int q = warp & 3, jc = warp >> 2;  // TMEM lane quarter; which 32 of the CTA's 128 columns
+    const int q = warp & 3, jc = warp >> 2;  // TMEM lane quarter; which 16 columns of a chunk
     const int row = q * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-    // this warp's 32 columns of the activations: its chunk (of the CTA's two) and the column within it
-    unsigned char* const act_own = sm.act + (2u * rank + (uint32_t)(jc >> 1)) * kMlpChunk;
+    unsigned char* const act_own = sm.act + 2u * rank * kMlpChunk;  // the CTA's two chunks of the activations
     uint32_t ph_layer = 0u, ph_stored = 0u;
     bool first_store = true;
     float loss = 0.f;
@@ -240,18 +255,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
       first_store = false;
       return ok;
     };
-    // 16 columns (step s) of the half-layer into the CTA's activations
+    // 16 columns of chunk s into the CTA's activations, and the chunk handed over: its copies start while the
+    // next one is worked on
     auto put_act = [&](int s, const uint32_t (&w)[8]) {
 #pragma unroll
       for (int h = 0; h < 2; ++h)
-        *reinterpret_cast<uint4*>(act_own + tc::sw128_offset(row, (jc & 1) * 32 + 16 * s + 8 * h)) =
+        *reinterpret_cast<uint4*>(act_own + s * kMlpChunk + tc::sw128_offset(row, jc * 16 + 8 * h)) =
             make_uint4(w[4 * h], w[4 * h + 1], w[4 * h + 2], w[4 * h + 3]);
-    };
-    auto act_done = [&]() {
       tc::fence_async_smem();
       tc::fence_before_sync();
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&sm.half[jc >> 1]);
+      if (lane == 0) tc::mbar_arrive(&sm.half[s]);
     };
     for (uint64_t ti = 0; ti < my_tiles && ok; ++ti) {
       const uint64_t b = (cluster + ti * n_clusters) * 128 + row;
@@ -259,21 +273,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
 #pragma unroll 1
       for (int l = 0; l < 3 && ok; ++l) {  // hidden layers: activation and derivative
         if (!layer_wait() || !stored_wait()) break;
-        const uint32_t acc = lane_addr + (uint32_t)(l * 128 + jc * 32);
+        const uint32_t acc = lane_addr + (uint32_t)(l * 128 + jc * 16);
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
           float z[16], d[16];
-          tc::tmem_ld16(acc + 16u * s, z);
-          const float* bias = sm.bias + l * 128 + jc * 32 + s * 16;
+          tc::tmem_ld16(acc + 64u * s, z);
+          const float* bias = sm.bias + l * 128 + s * 64 + jc * 16;
           uint32_t w[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             w[i] = gelu_grad_pair(z[2 * i], z[2 * i + 1], *reinterpret_cast<const uint64_t*>(bias + 2 * i), d[2 * i],
                                   d[2 * i + 1]);
-          tc::tmem_st16(acc + 16u * s, d);
+          tc::tmem_st16(acc + 64u * s, d);
           put_act(s, w);
         }
-        act_done();
       }
       if (!ok) break;
       // output layer: loss and dY, a thread per row (both CTAs compute them, the first keeps the sums)
@@ -314,21 +327,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
 #pragma unroll 1
       for (int l = 2; l >= 0 && ok; --l) {  // layer gradients: the accumulator times the derivative in TMEM
         if (!layer_wait() || (l < 2 && !stored_wait())) break;
-        const uint32_t acc = lane_addr + (uint32_t)((l + 1) * 128 + jc * 32);
+        const uint32_t acc = lane_addr + (uint32_t)((l + 1) * 128 + jc * 16);
+        // both chunks' values leave TMEM before the first chunk is handed over: the next MMAs write the region that
+        // held this layer's derivative
+        float x[2][16];
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
-          float x[16], d[16];
-          tc::tmem_ld16(acc + 16u * s, x);
-          tc::tmem_ld16(acc - 128u + 16u * s, d);
+          float d[16];
+          tc::tmem_ld16(acc + 64u * s, x[s]);
+          tc::tmem_ld16(acc - 128u + 64u * s, d);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) x[i] *= d[i];
-          uint32_t w[8];
-          pack_bf16(x, w);
-          put_act(s, w);
-          const float v = warp_colsum16(x, lane);
-          if (!(lane & 1)) atomicAdd(&sm.col[l * 128 + jc * 32 + s * 16 + warp_colsum16_column(lane)], v);
+          for (int i = 0; i < 16; ++i) x[s][i] *= d[i];
         }
-        act_done();
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          uint32_t w[8];
+          pack_bf16(x[s], w);
+          put_act(s, w);
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          const float v = warp_colsum16(x[s], lane);
+          if (!(lane & 1)) atomicAdd(&sm.col[l * 128 + s * 64 + jc * 16 + warp_colsum16_column(lane)], v);
+        }
         if (l == 0 && lane == 0) tc::mbar_arrive(&sm.tile);
       }
     }
@@ -337,18 +358,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
     if (!ok) sm.fail = 1;
   } else if (warp < kTrainEpiWarps + kTrainLoadWarps) {
     // ---- the tile's rows: sample numbers, features ----
-    const int row = tid - 32 * kTrainEpiWarps;
+    const int row = load_row;
     bool ok = true;
     for (uint64_t ti = 0; ti < my_tiles; ++ti) {
       const uint64_t b = (cluster + ti * n_clusters) * 128 + row;
-      uint4 f[kMlpIn / 8];
-      uint64_t src = 0;
-#pragma unroll
-      for (int k = 0; k < kMlpIn / 8; ++k) f[k] = make_uint4(0u, 0u, 0u, 0u);
-      if (b < a.B) {
-        src = a.n ? perm_index(a.first + b, a.n, a.h, a.key) : b;
-        load_features(a, src, f);
-      }
+      if (ti > 0) load_rows(ti);
       if (ti > 0 && !train_warp_wait(&sm.act_free, (uint32_t)(ti - 1) & 1u)) {
         ok = false;
         break;
@@ -372,7 +386,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
   } else if (warp == kTrainEpiWarps + kTrainLoadWarps + 1) {
     if (lane == 0) {
       // ---- copies of the CTA's half of the activations: to the peer for the next layer, to HBM ----
-      const uint32_t peer_act = tc::map_rank(sm.act, rank ^ 1u), peer_bar = tc::map_rank(&sm.peer, rank ^ 1u);
+      const uint32_t peer_act = tc::map_rank(sm.act, rank ^ 1u), peer_bar = tc::map_rank(sm.peer, rank ^ 1u);
       uint32_t ph = 0u;
       bool ok = true;
       for (uint64_t ti = 0; ti < my_tiles && ok; ++ti) {
@@ -381,7 +395,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
           for (uint32_t c = 0; c < 2; ++c) {
             if (!(ok = tc::mbar_wait(&sm.half[c], ph, kWaitNs))) break;
             const uint32_t at = 2u * rank + c;
-            if (e < 5) tc::bulk_s2s(peer_act + at * kMlpChunk, sm.act + at * kMlpChunk, kMlpChunk, peer_bar);
+            if (e < 5) tc::bulk_s2s(peer_act + at * kMlpChunk, sm.act + at * kMlpChunk, kMlpChunk, peer_bar + 8u * c);
             tc::tma_store_3d(e < 3 ? &tmH : &tmZ, sm.act + at * kMlpChunk, (int)at * 64, row0, e < 3 ? e : 5 - e);
           }
           ph ^= 1u;
@@ -412,10 +426,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
       // a layer from the activations and weights of 64-column chunks of w_stride bytes.  Columns in ascending order in
       // both CTAs: the first CTA starts with its own half, the second waits for the first one's.
       auto layer = [&](uint32_t d, uint32_t w, uint32_t w_stride, uint32_t idesc) {
-        tc::mbar_expect_tx(&sm.peer, 2 * kMlpChunk);
+        for (int c = 0; c < 2; ++c) tc::mbar_expect_tx(&sm.peer[c], kMlpChunk);
         for (uint32_t c = 0; c < 4 && ok; ++c) {
           ok = c / 2 == rank ? tc::mbar_wait(&sm.half[c & 1], ph_half, kWaitNs)
-                             : ((c & 1) || tc::mbar_wait_cluster(&sm.peer, ph_peer, kWaitNs));
+                             : tc::mbar_wait_cluster(&sm.peer[c & 1], ph_peer, kWaitNs);
           if (!ok) return;
           tc::fence_after_sync();
           chunk(d, act + c * kMlpChunk, w + c * w_stride, idesc, c == 0);
