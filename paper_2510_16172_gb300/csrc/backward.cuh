@@ -181,23 +181,11 @@ __global__ void __launch_bounds__(kThreads, kBackwardMinCtas<N>) backward_kernel
       // geometry (FP32, hi/lo differences of b) and parameters
       float bh[N + 2][3], bl[N + 2][3], a[N][2][3];
       bool edge[N];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        bh[0][c] = __ldg(S.tx32 + kEnd32 * d.tx + c);
-        bl[0][c] = __ldg(S.tx32 + kEnd32 * d.tx + 3 + c);
-        bh[N + 1][c] = __ldg(S.rx32 + kEnd32 * d.rx + c);
-        bl[N + 1][c] = __ldg(S.rx32 + kEnd32 * d.rx + 3 + c);
-      }
+      load_pair3(S.tx32 + kEnd32 * d.tx, bh[0], bl[0]);
+      load_pair3(S.rx32 + kEnd32 * d.rx, bh[N + 1], bl[N + 1]);
 #pragma unroll
       for (int i = 0; i < N; ++i) {
-        const float* r = s_rec + kRec32 * d.ids[i];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          bh[i + 1][c] = r[c];
-          bl[i + 1][c] = r[3 + c];
-          a[i][0][c] = r[6 + c];
-          a[i][1][c] = r[9 + c];
-        }
+        load_rec32(s_rec + kRec32 * d.ids[i], bh[i + 1], bl[i + 1], a[i][0], a[i][1]);
         edge[i] = s_aux[kAux * d.ids[i] + 2] != 0.f;
       }
       const float2* Ti = reinterpret_cast<const float2*>(T) + g * (uint64_t)n_max;

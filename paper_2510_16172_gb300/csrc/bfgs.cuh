@@ -139,25 +139,12 @@ __device__ __forceinline__ void fetch_path_q(const BatchDev& B, const Tables& tb
 template <int N, unsigned Q>
 __device__ __forceinline__ void load_geo(const PathDesc& d, const Tables& tb, Geo<N>& G) {
   float bh[N + 2][3], bl[N + 2][3];
-  const float* tx = tb.tx + kEnd32 * d.tx;
-  const float* rx = tb.rx + kEnd32 * d.rx;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    bh[0][c] = tx[c];
-    bl[0][c] = tx[3 + c];
-    bh[N + 1][c] = rx[c];
-    bl[N + 1][c] = rx[3 + c];
-  }
+  load_pair3(tb.tx + kEnd32 * d.tx, bh[0], bl[0]);
+  load_pair3(tb.rx + kEnd32 * d.rx, bh[N + 1], bl[N + 1]);
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    const float* r = tb.rec + kRec32 * d.ids[i];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      bh[i + 1][c] = r[c];
-      bl[i + 1][c] = r[3 + c];
-      G.a[i][0][c] = r[6 + c];
-      G.a[i][1][c] = Pat<N, Q>::quad(i) ? r[9 + c] : 0.f;
-    }
+    load_rec32(tb.rec + kRec32 * d.ids[i], bh[i + 1], bl[i + 1], G.a[i][0], G.a[i][1]);
+    if (!Pat<N, Q>::quad(i)) G.a[i][1][0] = G.a[i][1][1] = G.a[i][1][2] = 0.f;
   }
 #pragma unroll
   for (int j = 0; j <= N; ++j)

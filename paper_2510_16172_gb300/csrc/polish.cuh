@@ -282,36 +282,15 @@ __global__ void __launch_bounds__(kThreads, kPolishMinBlocks<N>) polish_ff_kerne
       // geometry: b as hi + lo, A as hi + lo
       GeoFF<N> G;
       bool edge[N];
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-        const float* r = rec32 + kRec32 * d.ids[i];
-        const float* rl = reclo + kRecLo * d.ids[i];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          G.ah[i][0][c] = r[6 + c];
-          G.ah[i][1][c] = r[9 + c];
-          G.al[i][0][c] = rl[c];
-          G.al[i][1][c] = rl[3 + c];
-        }
-        edge[i] = aux[kAux * d.ids[i] + 2] != 0.f;
-      }
       {
         float bh[N + 2][3], bl[N + 2][3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          bh[0][c] = __ldg(S.tx32 + kEnd32 * d.tx + c);
-          bl[0][c] = __ldg(S.tx32 + kEnd32 * d.tx + 3 + c);
-          bh[N + 1][c] = __ldg(S.rx32 + kEnd32 * d.rx + c);
-          bl[N + 1][c] = __ldg(S.rx32 + kEnd32 * d.rx + 3 + c);
-        }
+        load_pair3(S.tx32 + kEnd32 * d.tx, bh[0], bl[0]);
+        load_pair3(S.rx32 + kEnd32 * d.rx, bh[N + 1], bl[N + 1]);
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-          const float* r = rec32 + kRec32 * d.ids[i];
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            bh[i + 1][c] = r[c];
-            bl[i + 1][c] = r[3 + c];
-          }
+          load_rec32(rec32 + kRec32 * d.ids[i], bh[i + 1], bl[i + 1], G.ah[i][0], G.ah[i][1]);
+          load_pair3(reclo + kRecLo * d.ids[i], G.al[i][0], G.al[i][1]);
+          edge[i] = aux[kAux * d.ids[i] + 2] != 0.f;
         }
 #pragma unroll
         for (int jj = 0; jj <= N; ++jj)
