@@ -15,7 +15,7 @@
 // only the last chunk's four MMAs are exposed.  The next features go into the first activation chunk as
 // soon as the output layer has read it.
 //
-// Measured on 4 M city paths of orders 1-5: 2580 -> 1430 us (0.36 ns per path; the same bits).  What bounds it now
+// Measured on 4 M city paths of orders 1-5: 2580 -> 1366 us (0.34 ns per path; the same bits).  What bounds it now
 // is the epilogues: 768 tanh per path at 16 a clock and SM are 6144 cycles per 128 paths (the MMAs 4900), and three
 // times per tile the last chunk's MMAs and two hand-overs between warps (about 1000 cycles) are exposed: 12,700
 // cycles in all.  The rest of the GELU runs in packed FP32 pairs, five instructions for two values.

@@ -73,10 +73,13 @@ __device__ __forceinline__ int warp_colsum16_column(int lane) {
 __device__ __forceinline__ void path_features(const SceneDev& S, const PathDesc& d, float inv_scale,
                                               __nv_bfloat16* f, float* G) {
   float tx[3], rx[3], o[3];
+  float txl[3], rxl[3];
+  load_pair3(S.tx32 + kEnd32 * d.tx, tx, txl);
+  load_pair3(S.rx32 + kEnd32 * d.rx, rx, rxl);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    tx[c] = S.tx32[kEnd32 * d.tx + c] + S.tx32[kEnd32 * d.tx + 3 + c];
-    rx[c] = S.rx32[kEnd32 * d.rx + c] + S.rx32[kEnd32 * d.rx + 3 + c];
+    tx[c] += txl[c];
+    rx[c] += rxl[c];
     o[c] = 0.5f * (tx[c] + rx[c]);
   }
   float v[kMlpIn], gram[12];
@@ -93,15 +96,11 @@ __device__ __forceinline__ void path_features(const SceneDev& S, const PathDesc&
 #pragma unroll
   for (int s = 0; s < 4; ++s) {
     if (s < d.n && valid) {
-      const float* r = S.rec32 + kRec32 * d.ids[s];
       const bool edge = S.aux[kAux * d.ids[s] + 2] != 0.f;
-      float b[3], a1[3], a2[3];
+      float b[3], bl[3], a1[3], a2[3];
+      load_rec32(S.rec32 + kRec32 * d.ids[s], b, bl, a1, a2);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        b[c] = r[c] + r[3 + c];
-        a1[c] = r[6 + c];
-        a2[c] = r[9 + c];
-      }
+      for (int c = 0; c < 3; ++c) b[c] += bl[c];
       const float g11 = a1[0] * a1[0] + a1[1] * a1[1] + a1[2] * a1[2];
       const float g12 = a1[0] * a2[0] + a1[1] * a2[1] + a1[2] * a2[2];
       const float g22 = a2[0] * a2[0] + a2[1] * a2[1] + a2[2] * a2[2];
