@@ -642,14 +642,17 @@ __global__ void adam_kernel(float* __restrict__ w, float* __restrict__ m, float*
                             __nv_bfloat16* __restrict__ wt, __nv_bfloat16* __restrict__ wtT,
                             const float* __restrict__ loss, float* hist, float hist_w) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool have = i < kMlpParams;
+  const float m0 = have ? m[i] : 0.f, v0 = have ? v[i] : 0.f, w0 = have ? w[i] : 0.f;
+  tc::wait_previous();  // the gradient and the loss
   if (i == 0 && hist) *hist += hist_w * *loss;
-  if (i >= kMlpParams) return;
+  if (!have) return;
   const float gi = g[i];
-  const float mi = 0.9f * m[i] + 0.1f * gi;
-  const float vi = 0.999f * v[i] + 0.001f * gi * gi;
+  const float mi = 0.9f * m0 + 0.1f * gi;
+  const float vi = 0.999f * v0 + 0.001f * gi * gi;
   m[i] = mi;
   v[i] = vi;
-  const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+  const float wi = w0 - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
   w[i] = wi;
   const __nv_bfloat16 b = __float2bfloat16(wi);
   wb[i] = b;
@@ -683,9 +686,10 @@ cudaError_t launch_mlp_features(const SceneDev& S, const BatchDev& B, int n, con
 cudaError_t launch_adam(float* w, float* m, float* v, const float* g, float lr, float c1, float c2, __nv_bfloat16* wb,
                         __nv_bfloat16* wt, __nv_bfloat16* wtT, const float* loss, float* hist, float hist_w,
                         cudaStream_t stream) {
-  adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, stream>>>(w, m, v, g, lr, c1, c2, wb, wt, wtT, loss, hist, hist_w);
+  const cudaError_t e = launch_overlapped(adam_kernel, (kMlpParams + 255) / 256, 256, 0, stream, w, m, v, g, lr, c1, c2, wb,
+                                          wt, wtT, loss, hist, hist_w);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_mlp_tile_weights(const __nv_bfloat16* wb, __nv_bfloat16* wt, __nv_bfloat16* wtT,
