@@ -127,11 +127,13 @@ __global__ void __launch_bounds__(kThreads, kBackwardMinCtas<N>) backward_kernel
   __syncthreads();
   const int n_max = B.n_max;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  wait_previous();  // the scene's tables are older than the chain of kernels this one is part of
   // listed launch: the paths the select pass found with a cotangent; else the CTA's queue
   __shared__ uint32_t s_queue[kQueue];
   const uint64_t n_iter = cfg.sel ? (uint64_t)*cfg.sel_count : 0;
   const int rounds = n_local > (uint64_t)gridDim.x * (kScanRounds * kThreads) ? kScanRounds : 1;
   uint64_t scan = (uint64_t)blockIdx.x * (unsigned)(rounds * kThreads);
+  if (kChained<N> && (cfg.sel ? n_iter : n_local) <= stride) launch_dependents();  // one round: the FP64 pass sets up beside it
   unsigned head = 0, fill = 0;
   int tiles = 0;
   for (uint64_t j0 = (uint64_t)blockIdx.x * blockDim.x;; j0 += stride) {
@@ -265,6 +267,7 @@ __global__ void __launch_bounds__(kSelThreads) backward_select_kernel(BatchDev B
                                                                       const PathRec* list,
                                                                       const uint8_t* __restrict__ status,
                                                                       const float* __restrict__ dLv) {
+  wait_previous();
   for (uint64_t c0 = (uint64_t)blockIdx.x * kSelChunk; c0 < n_local; c0 += (uint64_t)gridDim.x * kSelChunk) {
     const uint64_t j0 = c0 + (uint64_t)threadIdx.x * kSelPer;
     unsigned bits = 0;
@@ -320,6 +323,7 @@ __global__ void __launch_bounds__(kThreads, kLongOrderMinBlocks<N>)
         const float* __restrict__ T, const uint8_t* __restrict__ status, const float* __restrict__ dX,
         const float* __restrict__ dLv, double* gacc, const uint32_t* __restrict__ rescue_list,
         const unsigned* __restrict__ rescue_count) {
+  wait_previous();
   const uint64_t n = *rescue_count;
   const int n_max = B.n_max;
   for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (uint64_t)gridDim.x * blockDim.x) {
@@ -389,10 +393,10 @@ cudaError_t launch_backward_rescue_n(const SceneDev& S, const BatchDev& B, const
                                             const unsigned* rescue_count) {
   const unsigned rgrid = rescue_grid(n_local, n_sm);
   if (rgrid == 0) return cudaSuccess;
-  backward_rescue_kernel<N><<<rgrid, kRescueThreads, 0, stream>>>(S, B, cfg, list, T, status, dX, dL, gacc, rescue_list,
-                                                             rescue_count);
+  const cudaError_t e = launch_path(true, backward_rescue_kernel<N>, rgrid, kRescueThreads, 0, stream, S, B, cfg, list, T,
+                                    status, dX, dL, gacc, rescue_list, rescue_count);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 // Slices up to this many paths per SM (four CTAs' worth of threads) are scanned by the adjoint's own CTAs also where
@@ -406,6 +410,7 @@ cudaError_t launch_backward_n(const SceneDev& S, const BatchDev& B, const Backwa
                                      const float* dX, const float* dL, double* gacc, cudaStream_t stream, int n_sm,
                                      uint32_t* rescue_list, unsigned* rescue_count) {
   BackwardCfg cfg = cfg_in;
+  bool chained = cfg.chained;  // the previous launch on the stream is the order's polish
   if (dX != nullptr || cfg.sel == nullptr || cfg.sel_count == nullptr ||
       n_local <= (uint64_t)n_sm * kScanMaxPerSm) {
     cfg.sel = nullptr;  // the kernel scans for the paths with a cotangent
@@ -414,10 +419,11 @@ cudaError_t launch_backward_n(const SceneDev& S, const BatchDev& B, const Backwa
     const uint64_t want = (n_local + kSelChunk - 1) / kSelChunk;
     const unsigned g = (unsigned)(want < (uint64_t)n_sm * 8 ? want : (uint64_t)n_sm * 8);
     if (g == 0) return cudaSuccess;
-    backward_select_kernel<N><<<g, kSelThreads, 0, stream>>>(B, cfg, n_local, list, status, dL);
+    const cudaError_t e =
+        launch_path(chained, backward_select_kernel<N>, g, kSelThreads, 0, stream, B, cfg, n_local, list, status, dL);
     count_launch();
-    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    chained = true;
   }
   const size_t base = (size_t)S.n_obj * (kRec32 + kAux) * sizeof(float);
   const size_t accb = (size_t)(S.n_obj * 9 + 3 * (S.n_tx + S.n_rx)) * sizeof(float);
@@ -434,10 +440,9 @@ cudaError_t launch_backward_n(const SceneDev& S, const BatchDev& B, const Backwa
   unsigned grid = 0;
   cudaError_t e = strided_grid(backward_kernel<N>, kThreads, smem, n_local, n_sm, grid);
   if (e != cudaSuccess || grid == 0) return e;
-  backward_kernel<N><<<grid, kThreads, smem, stream>>>(S, B, cfg, n_local, list, T, status, dX, dL, gacc, rescue_list,
-                                                        rescue_count);
+  e = launch_path(chained, backward_kernel<N>, grid, kThreads, smem, stream, S, B, cfg, n_local, list, T, status, dX, dL, gacc,
+                  rescue_list, rescue_count);
   count_launch();
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_backward_rescue_n<N>(S, B, cfg, n_local, list, T, status, dX, dL, gacc, stream, n_sm, rescue_list,
                                      rescue_count);

@@ -1134,7 +1134,10 @@ static fpt_status solve_impl(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* 
                                       r.stream, ctx->n_sm, r.lists, &r.ctl->polish64, grad ? &gc : nullptr, step_list,
                                       &r.ctl->stepped, r.step));
     }
-    return after ? backward_order(ctx, S, b, r, after->cfg, T, status, after->dX, after->dL) : FPT_OK;
+    if (!after) return FPT_OK;
+    BackwardCfg cfg = after->cfg;
+    cfg.chained = !ctx->prof;  // (kernel timing records events in between)
+    return backward_order(ctx, S, b, r, cfg, T, status, after->dX, after->dL);
   });
 }
 

@@ -458,6 +458,12 @@ __device__ __forceinline__ void load_pair3(const float* p, float (&h)[3], float 
   l[2] = c.y;
 }
 
+// Programmatic dependent launch: let the stream's next kernel start its set-up once every CTA of this one has come here;
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// and, in that kernel (launched with launch_overlapped), wait until the one before has completed and its writes are visible.
+// Returns at once after an ordinary launch.
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Stage `count` elements of T from global to shared memory (whole CTA).
 template <typename T>
 __device__ __forceinline__ void stage(T* dst, const T* src, int count) {

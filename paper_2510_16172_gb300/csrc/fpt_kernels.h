@@ -44,6 +44,39 @@ inline cudaError_t strided_grid(Kernel fn, int threads, size_t smem, uint64_t n,
   grid = (unsigned)(want < cap ? want : cap);
   return cudaSuccess;
 }
+// A launch whose kernel may set up while the stream's previous kernel runs (it calls wait_previous before it touches
+// anything that one writes).
+template <typename... P, typename... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream,
+                              A&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+// Orders whose kernels let the next link of their chain (two polish passes, FP64 polish, select, adjoint, FP64 adjoint)
+// set up while they run, where one round of CTAs takes their whole slice: the chain of a small batch is launches and
+// set-up for a good part.  33,800 canyon paths of orders 1-3 132 -> 116 us, 200,000 tiny-scene paths 166 -> 158, 541,000
+// canyon paths 440 -> 430.  Not the longer sequences: their waiting CTAs (255 registers) take the place of the
+// other orders' solvers (100,000 paths of orders 6-8 961 -> 981).
+template <int N>
+constexpr bool kChained = N <= kMaxBfgsOrder;
+// A link of an order's chain of kernels: overlapped when the previous launch on the stream is the link before it.
+template <typename... P, typename... A>
+cudaError_t launch_path(bool chained, void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem,
+                        cudaStream_t stream, A&&... args) {
+  if (chained) return launch_overlapped(kernel, grid, threads, smem, stream, args...);
+  kernel<<<grid, threads, smem, stream>>>(P(args)...);
+  return cudaGetLastError();
+}
 constexpr size_t kMaxSmemBytes = 200 * 1024;  // dynamic shared memory a path kernel may request
 
 // Kernels launched by the calling thread; the API's profiler reads the
@@ -89,6 +122,7 @@ struct BackwardCfg {
   unsigned* sel_count = nullptr;
   // counter of the paths whose Hessian also fails the FP64 pivot test (left out of the sums; nullptr: not counted)
   unsigned* dropped = nullptr;
+  bool chained = false;  // the previous launch on the stream is the polish of the same paths
 };
 
 // Per-order launches (n = 1..kMaxOrder).  `list` = nullptr for exhaustive batches.  The counters that a launch

@@ -644,7 +644,7 @@ __global__ void adam_kernel(float* __restrict__ w, float* __restrict__ m, float*
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const bool have = i < kMlpParams;
   const float m0 = have ? m[i] : 0.f, v0 = have ? v[i] : 0.f, w0 = have ? w[i] : 0.f;
-  tc::wait_previous();  // the gradient and the loss
+  wait_previous();  // the gradient and the loss
   if (i == 0 && hist) *hist += hist_w * *loss;
   if (!have) return;
   const float gi = g[i];

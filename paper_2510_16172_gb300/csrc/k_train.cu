@@ -224,7 +224,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
     }
   };
   if (warp >= kTrainEpiWarps && warp < kTrainEpiWarps + kTrainLoadWarps && my_tiles > 0) load_rows(0);
-  tc::launch_dependents();  // the weight gradients' CTAs set up on SMs this launch leaves idle or has left
+  launch_dependents();  // the weight gradients' CTAs set up on SMs this launch leaves idle or has left
   tc::fence_before_sync();
   __syncthreads();
   tc::cluster_sync();  // the peer's barriers are initialised before anything arrives on them
@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
   const int total = (int)((a.B + 63) / 64), per = (total + slices - 1) / slices;
   const int first = slice * per, last = first + per < total ? first + per : total;
   if (first >= last) return;  // (the whole CTA)
-  tc::launch_dependents();  // Adam's CTAs fit beside this launch's and load the weights and moments meanwhile
+  launch_dependents();  // Adam's CTAs fit beside this launch's and load the weights and moments meanwhile
   const int count = last - first;
   const int n_cols = job == 4 ? kMlpOut : (job == 1 ? kMlpIn : kMlpHidden);
   if (threadIdx.x == 0) {
@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = s_tmem;
-  tc::wait_previous();
+  wait_previous();
   if (warp == 0) {
     if (lane == 0) {
       // ---- loads ----

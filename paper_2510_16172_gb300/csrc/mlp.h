@@ -6,7 +6,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
-#include "fpt_device.cuh"
+#include "fpt_kernels.h"
 
 namespace fpt {
 
@@ -33,24 +33,6 @@ struct GemmArgs {
   long long shm, shn;
   int* err;               // device error word (MMA completion timeout)
 };
-
-// A launch whose kernel may set up while the stream's previous kernel runs (it calls tc::wait_previous before it touches
-// anything that one writes).
-template <typename... P, typename... A>
-cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream,
-                              A&&... args) {
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
-}
 
 // A tiled tensor map (false where the base or a stride does not allow one).
 bool encode_map(CUtensorMap* map, CUtensorMapDataType type, int rank, const void* base, const cuuint64_t* dims,

@@ -253,8 +253,10 @@ __global__ void __launch_bounds__(kThreads, kPolishMinBlocks<N>) polish_ff_kerne
   __syncthreads();
   const int n_max = B.n_max;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  wait_previous();  // the scene's tables are older than the chain of kernels this one is part of
   // second pass: only the paths the first pass listed for a Newton step
   const uint64_t n_iter = in_list ? (uint64_t)*in_count : n_local;
+  if (kChained<N> && n_iter <= stride) launch_dependents();  // one round: the chain's next kernel sets up beside it
   int tiles = 0;
   for (uint64_t k0 = (uint64_t)blockIdx.x * blockDim.x; k0 < n_iter; k0 += stride) {
     const uint64_t k = k0 + threadIdx.x;
@@ -531,8 +533,10 @@ __global__ void __launch_bounds__(kThreads, kLongOrderMinBlocks<N>)
   }
   const int n_max = B.n_max;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  wait_previous();
   // rescue mode: only the paths the double-float pass listed
   const uint64_t n_iter = rescue_list ? (uint64_t)*rescue_count : n_local;
+  if (kChained<N> && n_iter <= stride) launch_dependents();
   for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n_iter; k += stride) {
     const uint64_t j = rescue_list ? (uint64_t)rescue_list[k] : k;
     PathDesc d;
@@ -723,28 +727,26 @@ cudaError_t launch_polish_n(const SceneDev& S, const BatchDev& B, const PolishCf
     if (grad) {
       e = grid_of((const void*)polish_ff_kernel<N, true>, sff, n_grid, grid);
       if (e != cudaSuccess || grid == 0) return e;
-      polish_ff_kernel<N, true><<<grid, kThreads, sff, stream>>>(S, B, cfg, n_local, list, T, X, L, status, rho,
-                                                                 mask, bdist, use_smem, rescue_list, rescue_count, gc,
-                                                                 in_l, in_c, out_l, out_c, step_delta);
+      e = launch_path(pass == 1, polish_ff_kernel<N, true>, grid, kThreads, sff, stream, S, B, cfg, n_local, list, T, X, L,
+                      status, rho, mask, bdist, use_smem, rescue_list, rescue_count, gc, in_l, in_c, out_l, out_c,
+                      step_delta);
     } else {
       e = grid_of((const void*)polish_ff_kernel<N, false>, sff, n_grid, grid);
       if (e != cudaSuccess || grid == 0) return e;
-      polish_ff_kernel<N, false><<<grid, kThreads, sff, stream>>>(S, B, cfg, n_local, list, T, X, L, status, rho,
-                                                                  mask, bdist, use_smem, rescue_list, rescue_count,
-                                                                  gc, in_l, in_c, out_l, out_c, step_delta);
+      e = launch_path(pass == 1, polish_ff_kernel<N, false>, grid, kThreads, sff, stream, S, B, cfg, n_local, list, T, X,
+                      L, status, rho, mask, bdist, use_smem, rescue_list, rescue_count, gc, in_l, in_c, out_l, out_c,
+                      step_delta);
     }
     count_launch();
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   // FP64 pass over the listed paths, in CTAs of one warp (kRescueThreads) that read the records where they
   // stand: a listed path needs a few of them, so staging the scene's tables would cost more than it saves
   const unsigned rgrid = rescue_grid(n_local, n_sm);
   if (rgrid == 0) return cudaSuccess;
-  polish64_kernel<N><<<rgrid, kRescueThreads, 0, stream>>>(S, B, cfg, n_local, list, T, X, L, status, rho, mask, bdist,
-                                                            0, rescue_list, rescue_count);
+  e = launch_path(true, polish64_kernel<N>, rgrid, kRescueThreads, 0, stream, S, B, cfg, n_local, list, T, X, L, status, rho,
+                  mask, bdist, 0, rescue_list, rescue_count);
   count_launch();
-  e = cudaGetLastError();
   if (e != cudaSuccess || !grad) return e;
   // FP64 adjoint for the paths the fused kernel listed (final T and status are in place)
   BackwardCfg bc{gc.cond_adj, gc.deg_tol, 0, 0, gc.dL ? (uint8_t)0 : gc.dl_mask};

@@ -154,12 +154,6 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
   return false;
 }
 
-// ---- programmatic dependent launch ---------------------------------------------
-// Let the stream's next kernel start its set-up once every CTA of this one has come here;
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// and, in that kernel (launched with launch_overlapped), wait until the one before has completed and its writes are visible.
-__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // ---- TMA bulk copy ------------------------------------------------------------
 // Arm the barrier for `bytes` of incoming transactions (one arrival).
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
