@@ -40,7 +40,7 @@ struct fpt_ctx {
   unsigned long long* d_count = nullptr;   // counters for reductions
   unsigned char* d_ctl = nullptr;          // launch counters of the orders (OrderCtl), cleared once per call
   static constexpr int kSide = FPT_SIDE_STREAMS;  // streams for the independent pattern launches of one order
-  cudaStream_t side[kSide] = {};
+  cudaStream_t side[kSide] = {};           // created by the first call that needs them (side_streams)
   cudaEvent_t fork_ev = nullptr;
   cudaEvent_t join_ev[kSide] = {};
   // orders of one call that run side by side: the first on `stream`, the others dealt over these
@@ -251,10 +251,8 @@ fpt_status fpt_create(fpt_ctx** out, int device, void* cuda_stream) {
   static_assert(kPatternKeys <= 128, "pattern counters");
   if (e == cudaSuccess) e = cudaMalloc(&ctx->d_count, 128 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMalloc(&ctx->d_ctl, kCtlBytes);
-  for (int k = 0; k < fpt_ctx::kSide && e == cudaSuccess; ++k) {
-    e = cudaStreamCreateWithFlags(&ctx->side[k], cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->join_ev[k], cudaEventDisableTiming);
-  }
+  for (int k = 0; k < fpt_ctx::kSide && e == cudaSuccess; ++k)
+    e = cudaEventCreateWithFlags(&ctx->join_ev[k], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming);
   for (int k = 0; k < fpt_ctx::kOrderStreams && e == cudaSuccess; ++k) {
     e = cudaStreamCreateWithFlags(&ctx->ostream[k], cudaStreamNonBlocking);
@@ -1010,8 +1008,31 @@ static fpt_status backward_order(fpt_ctx* ctx, const SceneDev& S, const fpt_batc
   return FPT_OK;
 }
 
+// Streams for the pattern launches of one order.  With one order at a time the order streams are idle and serve; orders
+// side by side get streams of their own, created here once (a context whose batches never need them does not pay for
+// them), or, where that is not possible (a stream capture, an error), the order streams too: that only
+// adds dependencies.
+static const cudaStream_t* side_streams(fpt_ctx* ctx, bool overlap) {
+  static_assert(fpt_ctx::kSide <= fpt_ctx::kOrderStreams, "order streams in place of side streams");
+  if (!overlap) return ctx->ostream;
+  if (!ctx->side[fpt_ctx::kSide - 1]) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      return ctx->ostream;
+    }
+    for (cudaStream_t& s : ctx->side)
+      if (!s && cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) {
+        s = nullptr;
+        cudaGetLastError();
+        return ctx->ostream;
+      }
+  }
+  return ctx->side;
+}
+
 // BFGS of one order's paths.
-static fpt_status bfgs_order(fpt_ctx* ctx, const SceneDev& S, const fpt_batch* b, const OrderRun& r,
+static fpt_status bfgs_order(fpt_ctx* ctx, const SceneDev& S, const fpt_batch* b, const OrderRun& r, bool overlap,
                              const SolveCfg& sc, int specialize, float* T, uint8_t* status, uint8_t* iters) {
   ProfScope ps(ctx, FPT_K_BFGS);
   const int n = r.n;
@@ -1049,17 +1070,18 @@ static fpt_status bfgs_order(fpt_ctx* ctx, const SceneDev& S, const fpt_batch* b
   // the pattern launches of one order are independent: spread them over the side streams so that
   // each launch's tail overlaps the next one; each concurrent launch has its own work counter
   const int used = count < 2 ? 0 : (count < fpt_ctx::kSide ? count : fpt_ctx::kSide);
+  const cudaStream_t* side = used ? side_streams(ctx, overlap) : nullptr;
   if (used) {
     CUDA_OR_FAIL(ctx, cudaEventRecord(ctx->fork_ev, r.stream));
-    for (int k = 0; k < used; ++k) CUDA_OR_FAIL(ctx, cudaStreamWaitEvent(ctx->side[k], ctx->fork_ev, 0));
+    for (int k = 0; k < used; ++k) CUDA_OR_FAIL(ctx, cudaStreamWaitEvent(side[k], ctx->fork_ev, 0));
   }
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < count && e == cudaSuccess; ++i)
     e = launch_bfgs(n, todo[i].pattern, S, b->dev, sc, todo[i].cnt, todo[i].list, T, status, iters,
-                    used ? ctx->side[i % used] : r.stream, ctx->n_sm, todo[i].work);
+                    used ? side[i % used] : r.stream, ctx->n_sm, todo[i].work);
   // join every side stream that waited on the fork, also after an error (a stream capture must end joined)
   for (int k = 0; k < used; ++k) {
-    const cudaError_t f = cudaEventRecord(ctx->join_ev[k], ctx->side[k]);
+    const cudaError_t f = cudaEventRecord(ctx->join_ev[k], side[k]);
     const cudaError_t w = f == cudaSuccess ? cudaStreamWaitEvent(r.stream, ctx->join_ev[k], 0) : f;
     if (e == cudaSuccess) e = w;
   }
@@ -1119,7 +1141,7 @@ static fpt_status solve_impl(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* 
       CUDA_OR_FAIL(ctx, launch_mlp_infer(S, b->dev, r.n, r.list, r.cnt, 1.f / m->scale, m->d_wt, m->d_w, T, 0, ctx->d_err,
                                          r.stream, ctx->n_sm));
     }
-    fpt_status rs = bfgs_order(ctx, S, b, r, sc, p.specialize, T, status, iters);
+    fpt_status rs = bfgs_order(ctx, S, b, r, plan.overlap, sc, p.specialize, T, status, iters);
     if (rs != FPT_OK) return rs;
     {
       ProfScope ps(ctx, FPT_K_POLISH);
