@@ -17,7 +17,7 @@
 //
 // Measured on 4 M city paths of orders 1-5: 2580 -> 1366 us (0.34 ns per path; the same bits).  What bounds it now
 // is the epilogues: 768 tanh per path at 16 a clock and SM are 6144 cycles per 128 paths (the MMAs 4900), and three
-// times per tile the last chunk's MMAs and two hand-overs between warps (about 1000 cycles) are exposed: 12,700
+// times per tile the last chunk's MMAs and two hand-overs between warps (about 1000 cycles) are exposed: 12,100
 // cycles in all.  The rest of the GELU runs in packed FP32 pairs, five instructions for two values.
 //
 // Every wait is bounded; a role that runs out of time marks its CTA failed and leaves its loop, the others

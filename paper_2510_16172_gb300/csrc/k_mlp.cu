@@ -7,7 +7,7 @@
 //
 // GEMMs D[M x N] = sum_k A(m, k) B(n, k), N <= 256, K in chunks of 64, for the unfused forward pass.  Operands whose
 // rows are contiguous and 16-byte aligned go to gemm_ws_kernel: persistent, one CTA per SM over 128-row tiles, the
-// chunks loaded by TMA into a three- or two-stage ring (128-byte swizzled K-major tiles), one thread issuing the MMAs
+// chunks loaded by TMA into a three-stage ring (128-byte swizzled K-major tiles), one thread issuing the MMAs
 // into two TMEM accumulators, twelve epilogue warps staging the outputs in shared memory for TMA tensor stores.
 // Other strides take gemm_kernel, one tile per CTA with the operands gathered element by element.  Epilogues: plain
 // store (+ bias); bias + GELU with a BF16 activation.  Inference is fused in k_infer.cu, training in k_train.cu.
