@@ -1526,14 +1526,16 @@ static fpt_status mlp_forward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16
   return FPT_OK;
 }
 
-// Loss and gradient (d_loss, d_g) of a batch.  n > 0: row i is sample perm(first + i) of n (fpt_mlp_train).
+// Loss and gradient (d_loss, d_g) of a batch.  n > 0: row i is sample perm(first + i) of n (fpt_mlp_train).  chained: the
+// previous launch on the stream is this network's mlp_adam with `clear`, which left both at zero.
 static fpt_status mlp_backward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16* X, const float* T, const float* G,
-                                    uint64_t B, uint64_t n, uint64_t first, uint64_t key) {
+                                    uint64_t B, uint64_t n, uint64_t first, uint64_t key, bool chained) {
   fpt_status st = mlp_ensure_ws(ctx, m, B, true);
   if (st == FPT_OK) st = mlp_tiled_weights(ctx, m);
   if (st != FPT_OK) return st;
-  CUDA_OR_FAIL(ctx, cudaMemsetAsync(m->d_g, 0, (kMlpParams + 1) * sizeof(float), ctx->stream));
+  if (!chained) CUDA_OR_FAIL(ctx, cudaMemsetAsync(m->d_g, 0, (kMlpParams + 1) * sizeof(float), ctx->stream));
   TrainArgs a{};
+  a.chained = chained;
   a.X = X;
   a.T = T;
   a.G = G;
@@ -1556,12 +1558,12 @@ static fpt_status mlp_backward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat1
   return FPT_OK;
 }
 
-// Adam step on d_g; with hist, also *hist += hist_w * the batch's loss.
-static fpt_status mlp_adam(fpt_ctx* ctx, fpt_mlp* m, float lr, float* hist, float hist_w) {
+// Adam step on d_g; with hist, also *hist += hist_w * the batch's loss; with clear, d_g and d_loss are zero afterwards.
+static fpt_status mlp_adam(fpt_ctx* ctx, fpt_mlp* m, float lr, float* hist, float hist_w, bool clear) {
   m->step += 1;
   const float c1 = 1.f - std::pow(0.9f, (float)m->step), c2 = 1.f - std::pow(0.999f, (float)m->step);
   CUDA_OR_FAIL(ctx, launch_adam(m->d_w, m->d_m, m->d_v, m->d_g, lr, c1, c2, m->d_wb, m->d_wt, m->d_wtT, m->d_loss, hist,
-                                hist_w, ctx->stream));
+                                hist_w, clear, ctx->stream));
   return FPT_OK;
 }
 
@@ -1737,7 +1739,7 @@ fpt_status fpt_mlp_loss_grad(fpt_ctx* ctx, fpt_mlp* m, const void* X, const floa
   if (!ctx || !m || !X || !T || !G) return fail(ctx, FPT_EINVAL, "null argument");
   if (B < 1 || B > (1ull << 30)) return fail(ctx, FPT_EINVAL, "bad batch size");
   CUDA_OR_FAIL(ctx, cudaSetDevice(ctx->device));
-  fpt_status st = mlp_backward_impl(ctx, m, static_cast<const __nv_bfloat16*>(X), T, G, B, 0, 0, 0);
+  fpt_status st = mlp_backward_impl(ctx, m, static_cast<const __nv_bfloat16*>(X), T, G, B, 0, 0, 0, false);
   if (st != FPT_OK) return st;
   if (grad_out)
     CUDA_OR_FAIL(ctx, cudaMemcpyAsync(grad_out, m->d_g, kMlpParams * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
@@ -1752,7 +1754,7 @@ fpt_status fpt_mlp_train_step(fpt_ctx* ctx, fpt_mlp* m, const void* X, const flo
                               float lr, float* loss) {
   if (!(lr > 0.f)) return fail(ctx, FPT_EINVAL, "learning rate must be positive");
   fpt_status st = fpt_mlp_loss_grad(ctx, m, X, T, G, B, nullptr, nullptr);
-  if (st == FPT_OK) st = mlp_adam(ctx, m, lr, nullptr, 0.f);
+  if (st == FPT_OK) st = mlp_adam(ctx, m, lr, nullptr, 0.f, false);
   if (st != FPT_OK) return st;
   if (loss) {
     CUDA_OR_FAIL(ctx, cudaMemcpyAsync(loss, m->d_loss, sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1790,8 +1792,9 @@ fpt_status fpt_mlp_train(fpt_ctx* ctx, fpt_mlp* m, const void* X, const float* T
     uint64_t s0 = p.seed + 0x9E3779B97F4A7C15ULL * (uint64_t)(ep + 1);
     const uint64_t key = sm64_next(s0);
     for (uint64_t k = 0; k < steps; ++k) {
-      fpt_status st = mlp_backward_impl(ctx, m, Xs, T, G, B, n, k * B, key);
-      if (st == FPT_OK) st = mlp_adam(ctx, m, lr, m->d_hist + ep, 1.f / (float)steps);
+      // the steps of one call are a chain: each starts from the gradient that the one before cleared
+      fpt_status st = mlp_backward_impl(ctx, m, Xs, T, G, B, n, k * B, key, ep > 0 || k > 0);
+      if (st == FPT_OK) st = mlp_adam(ctx, m, lr, m->d_hist + ep, 1.f / (float)steps, true);
       if (st != FPT_OK) return st;
     }
     lr *= p.lr_decay;

@@ -638,16 +638,19 @@ __global__ void mlp_features_kernel(SceneDev S, BatchDev B, int n, const PathRec
 // One Adam step; the updated weights' BF16 copies go straight into every layout that reads them, and one thread
 // adds the batch's loss to its epoch's mean.
 __global__ void adam_kernel(float* __restrict__ w, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ g, float lr, float c1, float c2, __nv_bfloat16* __restrict__ wb,
-                            __nv_bfloat16* __restrict__ wt, __nv_bfloat16* __restrict__ wtT,
-                            const float* __restrict__ loss, float* hist, float hist_w) {
+                            float* __restrict__ g, float lr, float c1, float c2, __nv_bfloat16* __restrict__ wb,
+                            __nv_bfloat16* __restrict__ wt, __nv_bfloat16* __restrict__ wtT, float* __restrict__ loss,
+                            float* hist, float hist_w, int clear) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const bool have = i < kMlpParams;
   const float m0 = have ? m[i] : 0.f, v0 = have ? v[i] : 0.f, w0 = have ? w[i] : 0.f;
-  wait_previous();  // the gradient and the loss
+  wait_previous();      // the gradient and the loss
+  launch_dependents();  // the next step's CTAs set up and gather their rows
   if (i == 0 && hist) *hist += hist_w * *loss;
+  if (i == 0 && clear) *loss = 0.f;
   if (!have) return;
   const float gi = g[i];
+  if (clear) g[i] = 0.f;
   const float mi = 0.9f * m0 + 0.1f * gi;
   const float vi = 0.999f * v0 + 0.001f * gi * gi;
   m[i] = mi;
@@ -683,11 +686,11 @@ cudaError_t launch_mlp_features(const SceneDev& S, const BatchDev& B, int n, con
   return cudaGetLastError();
 }
 
-cudaError_t launch_adam(float* w, float* m, float* v, const float* g, float lr, float c1, float c2, __nv_bfloat16* wb,
-                        __nv_bfloat16* wt, __nv_bfloat16* wtT, const float* loss, float* hist, float hist_w,
+cudaError_t launch_adam(float* w, float* m, float* v, float* g, float lr, float c1, float c2, __nv_bfloat16* wb,
+                        __nv_bfloat16* wt, __nv_bfloat16* wtT, float* loss, float* hist, float hist_w, int clear,
                         cudaStream_t stream) {
   const cudaError_t e = launch_overlapped(adam_kernel, (kMlpParams + 255) / 256, 256, 0, stream, w, m, v, g, lr, c1, c2, wb,
-                                          wt, wtT, loss, hist, hist_w);
+                                          wt, wtT, loss, hist, hist_w, clear);
   count_launch();
   return e;
 }

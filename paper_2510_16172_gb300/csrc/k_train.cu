@@ -191,18 +191,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
     tc::mbar_init(&sm.drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     sm.fail = 0;
-    tc::mbar_expect_tx(&sm.fixed, kMlpChunk + 4 * kMlpW4Chunk + kW4tBytes);
-    tc::bulk_g2s(sm.w1, wf, kMlpChunk, &sm.fixed);
-    tc::bulk_g2s(sm.w4, wf + kMlpTileW4, 4 * kMlpW4Chunk, &sm.fixed);
-    tc::bulk_g2s(sm.w4t, wb + kMlpTileW4t, kW4tBytes, &sm.fixed);
-    fill(0, false);
-    fill(1, false);
   }
-  for (int i = tid; i < 3 * 128; i += blockDim.x) {
-    const int off = i < 128 ? kOffB1 : (i < 256 ? kOffB2 : kOffB3);
-    sm.bias[i] = a.params[off + (int)rank * 128 + (i & 127)];
-  }
-  if (tid < kMlpOut) sm.bias[384 + tid] = a.params[kOffB4 + tid];
   for (int i = tid; i < 3 * 128 + kMlpOut; i += blockDim.x) sm.col[i] = 0.f;
   __syncwarp();
   if (warp == 0) {
@@ -224,7 +213,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
     }
   };
   if (warp >= kTrainEpiWarps && warp < kTrainEpiWarps + kTrainLoadWarps && my_tiles > 0) load_rows(0);
-  launch_dependents();  // the weight gradients' CTAs set up on SMs this launch leaves idle or has left
+  wait_previous();  // what the last step's Adam wrote, and what its weight gradients read
+  // The weight gradients' CTAs set up on SMs this launch leaves idle or has left.  Only after the wait: they let the next
+  // Adam's CTAs load the weights and moments, which the last one must have written by then.
+  launch_dependents();
+  if (tid == 0) {
+    tc::mbar_expect_tx(&sm.fixed, kMlpChunk + 4 * kMlpW4Chunk + kW4tBytes);
+    tc::bulk_g2s(sm.w1, wf, kMlpChunk, &sm.fixed);
+    tc::bulk_g2s(sm.w4, wf + kMlpTileW4, 4 * kMlpW4Chunk, &sm.fixed);
+    tc::bulk_g2s(sm.w4t, wb + kMlpTileW4t, kW4tBytes, &sm.fixed);
+    fill(0, false);
+    fill(1, false);
+  }
+  for (int i = tid; i < 3 * 128; i += blockDim.x) {
+    const int off = i < 128 ? kOffB1 : (i < 256 ? kOffB2 : kOffB3);
+    sm.bias[i] = a.params[off + (int)rank * 128 + (i & 127)];
+  }
+  if (tid < kMlpOut) sm.bias[384 + tid] = a.params[kOffB4 + tid];
   tc::fence_before_sync();
   __syncthreads();
   tc::cluster_sync();  // the peer's barriers are initialised before anything arrives on them
@@ -711,9 +716,9 @@ cudaError_t launch_mlp_train(const TrainArgs& args, cudaStream_t stream, int n_s
   }
   if (!ok) return cudaErrorInvalidValue;
   const uint64_t tiles = (a.B + 127) / 128, cap = (uint64_t)(n_sm > 1 ? n_sm / 2 : 1);
-  mlp_train_kernel<<<2u * (unsigned)(tiles < cap ? tiles : cap), kTrainThreads, smem, stream>>>(a, st_h, st_z);
+  e = launch_path(a.chained != 0, mlp_train_kernel, 2u * (unsigned)(tiles < cap ? tiles : cap), kTrainThreads, smem, stream, a,
+                  st_h, st_z);
   count_launch();
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // One item per SM.  An item of dW2 or dW3 loads 48 KB per 64 rows and adds 128 KB, one of dW1 24 and 32 KB, one of
   // dW4 18 and 8 KB: 28, 12 and 8 slices of 152 items make them about equal at 8192 rows.

@@ -41,9 +41,9 @@ cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t stream);
 cudaError_t launch_mlp_features(const SceneDev& S, const BatchDev& B, int n, const PathRec* list, uint64_t first,
                                 uint64_t count, float inv_scale, __nv_bfloat16* X, float* G, cudaStream_t stream);
 // One Adam step, with the BF16 copies of the parameters (plain and as launch_mlp_tile_weights lays them out); with
-// hist, also *hist += hist_w * *loss.
-cudaError_t launch_adam(float* w, float* m, float* v, const float* g, float lr, float c1, float c2, __nv_bfloat16* wb,
-                        __nv_bfloat16* wt, __nv_bfloat16* wtT, const float* loss, float* hist, float hist_w,
+// hist, also *hist += hist_w * *loss; with clear, g and *loss are zero afterwards.
+cudaError_t launch_adam(float* w, float* m, float* v, float* g, float lr, float c1, float c2, __nv_bfloat16* wb,
+                        __nv_bfloat16* wt, __nv_bfloat16* wtT, float* loss, float* hist, float hist_w, int clear,
                         cudaStream_t stream);
 cudaError_t launch_to_bf16(const float* src, __nv_bfloat16* dst, int n, cudaStream_t stream);
 // The weights as the fused kernels' CTA pairs read them (k_infer.cu, k_train.cu): CTA r of a pair holds outputs
@@ -73,6 +73,7 @@ struct TrainArgs {
   uint64_t ldY;
   float *grad, *loss;
   int* err;
+  int chained;           // the previous launch on the stream is the last step's Adam, which left grad and loss at zero
   int h, vec_x, vec_tg;  // set by the launch: half the permutation's bits, 16-byte alignment of X, of T and G
 };
 cudaError_t launch_mlp_train(const TrainArgs& a, cudaStream_t stream, int n_sm);
