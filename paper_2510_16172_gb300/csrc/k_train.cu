@@ -334,8 +334,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
       for (int l = 2; l >= 0 && ok; --l) {  // layer gradients: the accumulator times the derivative in TMEM
         if (!layer_wait() || (l < 2 && !stored_wait())) break;
         const uint32_t acc = lane_addr + (uint32_t)((l + 1) * 128 + jc * 16);
-        // both chunks' values leave TMEM before the first chunk is handed over: the next MMAs write the region that
-        // held this layer's derivative
+        // both chunks' values leave TMEM before the first chunk is handed over: the next MMAs, which wait for it in either
+        // CTA, write the region that held this layer's derivative
         float x[2][16];
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
@@ -430,10 +430,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
         for (int kk = 0; kk < 4; ++kk) tc::mma_bf16(d, ad + 2u * kk, bd + 2u * kk, idesc, fresh && kk == 0 ? 0u : 1u);
       };
       // a layer from the activations and weights of 64-column chunks of w_stride bytes.  Columns in ascending order in
-      // both CTAs: the first CTA starts with its own half, the second waits for the first one's.
+      // both CTAs: the first CTA starts with its own half, the second waits for the first one's.  The second CTA too
+      // waits for its own first chunk before its first MMA: in the back-propagation that MMA overwrites the derivatives
+      // which this CTA's epilogue has read by the time it hands that chunk over, and the peer's chunk says nothing
+      // about them.  (The chunk is there well before the peer's copy.)
       auto layer = [&](uint32_t d, uint32_t w, uint32_t w_stride, uint32_t idesc) {
         for (int c = 0; c < 2; ++c) tc::mbar_expect_tx(&sm.peer[c], kMlpChunk);
-        for (uint32_t c = 0; c < 4 && ok; ++c) {
+        if (!(ok = tc::mbar_wait(&sm.half[0], ph_half, kWaitNs))) return;
+        for (uint32_t c = 0; c < 4; ++c) {
           ok = c / 2 == rank ? tc::mbar_wait(&sm.half[c & 1], ph_half, kWaitNs)
                              : tc::mbar_wait_cluster(&sm.peer[c & 1], ph_peer, kWaitNs);
           if (!ok) return;

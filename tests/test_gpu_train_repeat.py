@@ -1,0 +1,61 @@
+"""The training pass repeated on one batch while another stream keeps the memory busy: the same gradient every time.
+
+A CTA pair's MMAs overwrite, layer by layer, the tensor-memory regions whose derivatives its epilogues read; an MMA that
+does not wait for both CTAs' epilogues gives wrong layer gradients whenever one of them falls behind.  The
+repeats differ only in the order of the FP32 additions: at most 76 partial sums per entry (one per pair for the biases,
+28 batch slices for the weights), so by no more than 76 eps sum|partials|, eps = 2^-24; the partials are sums of independent
+rows, so sum|partials| is about sqrt(76) times the entry's own scale: 4e-5 of a layer's largest entry, and 1e-4 is
+allowed.  One warp's rows (32 of 8192) with wrong derivatives move an entry by about sqrt(32 / 8192) = 6 % of its scale.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from oracle import mlp_oracle as mo
+from paper_2510_16172_gb300 import fpt
+from test_gpu_mlp import SCALE, numpy_params
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_2510_16172_gb300 import build
+
+    build.build()
+    oracle.build()
+    return fpt.Context(0)
+
+
+@pytest.mark.parametrize("n", [256, 8192, 30_001])
+def test_repeated_gradients_agree(ctx, n):
+    import torch
+
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    X = (2.0 * torch.rand((n, 64), generator=gen, device="cuda") - 1.0).to(torch.bfloat16)
+    T = 2.0 * torch.rand((n, 8), generator=gen, device="cuda") - 0.5
+    G = torch.randn((n, 12), generator=gen, device="cuda") ** 2
+    net = fpt.Mlp(ctx, 0, SCALE)
+    net.set_params(numpy_params(8))
+    quiet_loss, quiet = net.loss_grad(X, T, G)
+    quiet = quiet.clone()
+    busy = torch.cuda.Stream()
+    a = torch.zeros(1 << 27, device="cuda")
+    b = torch.empty_like(a)
+    torch.cuda.synchronize()
+    runs = []
+    for _ in range(24):
+        with torch.cuda.stream(busy):
+            b.copy_(a)
+        loss, g = net.loss_grad(X, T, G)
+        assert abs(loss - quiet_loss) <= 1e-4 * abs(quiet_loss)
+        runs.append(g.clone())
+    torch.cuda.synchronize()
+    at = 0
+    for name, shape in mo.SIZES:
+        layer = slice(at, at + int(np.prod(shape)))
+        at = layer.stop
+        bound = 1e-4 * float(quiet[layer].abs().max())
+        for g in runs:
+            assert float((g[layer] - quiet[layer]).abs().max()) <= bound, name
+    net.close()
