@@ -30,6 +30,9 @@ namespace fpt {
 // (One round at a time where the slice is too small to give every CTA of the launch four.)
 constexpr int kScanRounds = 4, kQueue = 1024;
 static_assert((kScanRounds + 2) * kThreads <= kQueue, "queue entries");
+// The queue and the scan's counts are the kernel's static shared memory.  With its dynamic memory they may take 48 KB
+// without the opt-in (cudaFuncAttributeMaxDynamicSharedMemorySize): 449 objects with a TX and an RX.
+constexpr size_t kBackwardStaticSmem = kQueue * sizeof(uint32_t) + kScanRounds * (kThreads / 32) * sizeof(unsigned);
 
 // Appends the paths of [scan, scan + rounds kThreads) that carry a cotangent to the queue (its entries end at slot
 // `end`); every thread of the CTA calls it and gets their number.
@@ -433,7 +436,7 @@ cudaError_t launch_backward_n(const SceneDev& S, const BatchDev& B, const Backwa
     smem = base;
   }
   if (smem > 160 * 1024) return cudaErrorInvalidValue;  // scene too large for this kernel
-  if (smem > 48 * 1024) {
+  if (smem + kBackwardStaticSmem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(backward_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
