@@ -119,7 +119,14 @@ void fpt_default_params(fpt_solve_params* p);
 
 /* Create a context on CUDA device `device`, launching on `cuda_stream`
  * (a cudaStream_t; NULL = legacy default stream).  The context owns its
- * device workspace.  Returns FPT_ECUDA if the device cannot be used. */
+ * device workspace and keeps it until it is destroyed: per path of the
+ * largest call, 12 bytes and, for solves, 8 per interaction (a call of several
+ * orders holds all of them while that is at most 4 GiB and 2^27 paths, and the
+ * largest order's otherwise or where the memory is not there), and
+ * fpt_backward_unrolled's tape (at most 16 GiB).  A call that is captured
+ * into a graph takes the workspace as it stands; a later call that needs more
+ * leaves what the graph uses in place.  Returns FPT_ECUDA if the device cannot
+ * be used. */
 fpt_status fpt_create(fpt_ctx** out, int device, void* cuda_stream);
 void fpt_destroy(fpt_ctx* ctx);
 /* Switch the context's stream.  No synchronisation (legal inside a stream

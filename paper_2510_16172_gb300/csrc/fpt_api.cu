@@ -28,6 +28,13 @@ using namespace fpt;
 #define FPT_SIDE_STREAMS 4
 #endif
 
+// Device scratch of a context, grown when a call needs more (reserve).
+struct Scratch {
+  void* p = nullptr;
+  size_t cap = 0;         // bytes
+  bool captured = false;  // a stream capture has recorded launches that use it
+};
+
 struct fpt_ctx {
   int device = 0;
   int n_sm = 0;
@@ -35,8 +42,7 @@ struct fpt_ctx {
   int* d_err = nullptr;                    // device error word
   double* d_gacc = nullptr;                // backward accumulators (FP64)
   size_t gacc_cap = 0;
-  float* d_tape = nullptr;                 // per-step state of fpt_backward_unrolled
-  size_t tape_cap = 0;                     // floats
+  Scratch tape;                            // per-step state of fpt_backward_unrolled
   unsigned long long* d_count = nullptr;   // counters for reductions
   unsigned char* d_ctl = nullptr;          // launch counters of the orders (OrderCtl), cleared once per call
   static constexpr int kSide = FPT_SIDE_STREAMS;  // streams for the independent pattern launches of one order
@@ -48,10 +54,9 @@ struct fpt_ctx {
   cudaStream_t ostream[kOrderStreams] = {};
   cudaEvent_t ofork_ev = nullptr;
   cudaEvent_t ojoin_ev[kOrderStreams] = {};
-  uint32_t* d_rescue = nullptr;            // path lists: FP64 polish, FP64 adjoint, second polish pass
-  float* d_step = nullptr;                 // first Newton steps of the second polish pass's paths
-  size_t rescue_cap = 0;                   // entries of each of d_rescue's three lists
-  size_t step_cap = 0;                     // floats of d_step
+  Scratch rescue;                          // path lists: FP64 polish, FP64 adjoint, second polish pass
+  Scratch step;                            // first Newton steps of the second polish pass's paths
+  std::vector<void*> kept;                 // outgrown scratch that captured graphs use
   unsigned* d_dropped = nullptr;           // paths the last backward left out (fpt_backward_dropped)
   fpt_mlp* init_mlp = nullptr;             // network for init_mode = 1
   int acc_flush_tiles = 64;                // backward sums: CTA tiles between flushes of the FP32 partial sums
@@ -293,10 +298,9 @@ void fpt_destroy(fpt_ctx* ctx) {
     if (ctx->ojoin_ev[k]) cudaEventDestroy(ctx->ojoin_ev[k]);
   }
   if (ctx->ofork_ev) cudaEventDestroy(ctx->ofork_ev);
-  cudaFree(ctx->d_rescue);
-  cudaFree(ctx->d_step);
   cudaFree(ctx->d_dropped);
-  cudaFree(ctx->d_tape);
+  for (const Scratch* s : {&ctx->rescue, &ctx->step, &ctx->tape}) cudaFree(s->p);
+  for (void* p : ctx->kept) cudaFree(p);
   delete ctx;
 }
 
@@ -853,26 +857,46 @@ static uint64_t order_slice(const fpt_batch* b, int n, const PathRec** list) {
   return c;
 }
 
-// Path scratch for `entries` paths (three uint32 lists of them) and `step` floats of first Newton steps.
-static cudaError_t ensure_rescue(fpt_ctx* ctx, uint64_t entries, size_t step) {
-  cudaError_t e = cudaSuccess;
-  if (entries > ctx->rescue_cap) {
-    cudaFree(ctx->d_rescue);
-    ctx->d_rescue = nullptr;
-    ctx->rescue_cap = 0;
-    e = cudaMalloc(&ctx->d_rescue, 3 * entries * sizeof(uint32_t));
-    if (e != cudaSuccess) return e;
-    ctx->rescue_cap = entries;
+// Whether the context's stream is being captured.
+static bool capturing(const fpt_ctx* ctx) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return false;
+}
+
+// At least `bytes` of scratch for a call that may be part of a capture.  Scratch that a captured graph uses stays until the
+// context is destroyed; other outgrown scratch is freed.  With must = false a shortage leaves the scratch as it was, and
+// nothing is allocated inside a capture (most capture modes refuse that, and end).
+static cudaError_t reserve(fpt_ctx* ctx, Scratch& s, size_t bytes, bool in_capture, bool must) {
+  if (bytes > s.cap) {
+    if (in_capture && !must) return cudaErrorMemoryAllocation;
+    void* p = nullptr;
+    cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation && must && !s.captured) {  // no room beside the old block
+      cudaGetLastError();
+      cudaFree(s.p);
+      s = Scratch{};
+      e = cudaMalloc(&p, bytes);
+    }
+    if (e != cudaSuccess) {
+      if (!must) cudaGetLastError();
+      return e;
+    }
+    if (s.captured)
+      ctx->kept.push_back(s.p);
+    else
+      cudaFree(s.p);
+    s = Scratch{p, bytes, false};
   }
-  if (step > ctx->step_cap) {
-    cudaFree(ctx->d_step);
-    ctx->d_step = nullptr;
-    ctx->step_cap = 0;
-    e = cudaMalloc(&ctx->d_step, step * sizeof(float));
-    if (e != cudaSuccess) return e;
-    ctx->step_cap = step;
-  }
+  s.captured = s.captured || in_capture;
   return cudaSuccess;
+}
+
+// Path scratch for `entries` paths (three uint32 lists of them) and `steps` floats of first Newton steps.
+static cudaError_t reserve_paths(fpt_ctx* ctx, uint64_t entries, size_t steps, bool in_capture, bool must) {
+  const cudaError_t e = reserve(ctx, ctx->rescue, 3 * entries * sizeof(uint32_t), in_capture, must);
+  return e != cudaSuccess ? e : reserve(ctx, ctx->step, steps * sizeof(float), in_capture, must);
 }
 
 // One order's share of a call: its paths, the stream its kernels go to and its scratch.
@@ -892,9 +916,10 @@ struct OrderRun {
 // after the other against side by side: 200,000 tiny-scene paths of orders 1-4 353 -> 174 us, 541,000 canyon
 // paths of orders 1-3 651 -> 456 us, city batches of orders 1-5 with 8 M paths 5.70 -> 5.21 ms, 24 M 15.6 -> 14.8 ms,
 // 48 M 29.0 -> 27.9 ms.  The gain shrinks as single kernels fill the GPU, while overlapped orders need
-// their scratch side by side (12 + 8 n bytes per path of order n instead of the largest order's alone): the
-// line keeps that to a few GB.
+// their scratch side by side (12 + 8 n bytes per path of order n instead of the largest order's alone), which the
+// context keeps: hence the second line, on those bytes (100 M city paths of orders 1-5: 3.6 GB, in turn 1.0).
 constexpr uint64_t kOverlapMaxPaths = 1ull << 27;
+constexpr size_t kOverlapMaxScratch = size_t(4) << 30;
 
 // The orders of a call.  With overlap, the longest sequences come first (the longest chain) on the context's
 // stream and the others on the order streams, each with its own scratch; else all on the context's stream
@@ -927,13 +952,13 @@ static fpt_status plan_orders(fpt_ctx* ctx, const fpt_batch* b, bool scratch, bo
     step_most = st > step_most ? st : step_most;
   }
   // kernel timing brackets the launches of one class on the context's stream: one order after the other
-  plan.overlap = plan.count > 1 && sum <= kOverlapMaxPaths && !ctx->prof;
+  plan.overlap = plan.count > 1 && sum <= kOverlapMaxPaths && !ctx->prof &&
+                 (!scratch || 3 * sum * sizeof(uint32_t) + step_sum * sizeof(float) <= kOverlapMaxScratch);
   if (scratch && plan.count) {
-    if (plan.overlap && ensure_rescue(ctx, sum, step_sum) != cudaSuccess) {
-      cudaGetLastError();  // no room side by side: one order after the other, as for large batches
-      plan.overlap = false;
-    }
-    if (!plan.overlap) CUDA_OR_FAIL(ctx, ensure_rescue(ctx, most, step_most));
+    const bool in_capture = capturing(ctx);
+    // no room side by side, or no scratch for it before a capture: one order after the other, as for large batches
+    if (plan.overlap) plan.overlap = reserve_paths(ctx, sum, step_sum, in_capture, false) == cudaSuccess;
+    if (!plan.overlap) CUDA_OR_FAIL(ctx, reserve_paths(ctx, most, step_most, in_capture, true));
   }
   if (plan.overlap)
     for (int i = 0, j = plan.count - 1; i < j; ++i, --j) std::swap(plan.runs[i], plan.runs[j]);
@@ -942,8 +967,8 @@ static fpt_status plan_orders(fpt_ctx* ctx, const fpt_batch* b, bool scratch, bo
   for (int i = 0; i < plan.count; ++i) {
     OrderRun& r = plan.runs[i];
     if (scratch) {
-      r.lists = ctx->d_rescue + 3 * at;
-      r.step = steps ? ctx->d_step + step_at : nullptr;
+      r.lists = static_cast<uint32_t*>(ctx->rescue.p) + 3 * at;
+      r.step = steps ? static_cast<float*>(ctx->step.p) + step_at : nullptr;
     }
     if (plan.overlap) {
       if (i > 0) r.stream = ctx->ostream[(i - 1) % fpt_ctx::kOrderStreams];
@@ -1016,11 +1041,7 @@ static const cudaStream_t* side_streams(fpt_ctx* ctx, bool overlap) {
   static_assert(fpt_ctx::kSide <= fpt_ctx::kOrderStreams, "order streams in place of side streams");
   if (!overlap) return ctx->ostream;
   if (!ctx->side[fpt_ctx::kSide - 1]) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-      cudaGetLastError();
-      return ctx->ostream;
-    }
+    if (capturing(ctx)) return ctx->ostream;
     for (cudaStream_t& s : ctx->side)
       if (!s && cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) {
         s = nullptr;
@@ -1321,27 +1342,16 @@ fpt_status fpt_backward_unrolled(fpt_ctx* ctx, const fpt_scene* s, const fpt_bat
     most = need > most ? need : most;
   }
   if (sum * sizeof(float) > kUnrolledMaxTape) plan.run_in_turn(ctx->stream);
-  for (size_t cap = plan.overlap ? sum : most; cap > ctx->tape_cap;) {
-    cudaFree(ctx->d_tape);
-    ctx->d_tape = nullptr;
-    ctx->tape_cap = 0;
-    const cudaError_t e = cudaMalloc(&ctx->d_tape, cap * sizeof(float));
-    if (e == cudaSuccess) {
-      ctx->tape_cap = cap;
-    } else if (plan.overlap) {  // no room side by side
-      cudaGetLastError();
-      plan.run_in_turn(ctx->stream);
-      cap = most;
-    } else {
-      CUDA_OR_FAIL(ctx, e);
-    }
-  }
+  const bool in_capture = capturing(ctx);
+  if (plan.overlap && reserve(ctx, ctx->tape, sum * sizeof(float), in_capture, false) != cudaSuccess)
+    plan.run_in_turn(ctx->stream);  // no room side by side
+  if (!plan.overlap) CUDA_OR_FAIL(ctx, reserve(ctx, ctx->tape, most * sizeof(float), in_capture, true));
   size_t at = 0;
   st = run_orders(ctx, plan, [&](const OrderRun& r) -> fpt_status {
     ProfScope ps(ctx, FPT_K_BACKWARD);
     const size_t need = tape_floats(r);
     CUDA_OR_FAIL(ctx, launch_unrolled(r.n, S, b->dev, steps, fp_iters, r.cnt, r.list, dX, dL, ctx->d_gacc,
-                                      ctx->d_tape + at, need, T_out, status_out, r.stream, ctx->n_sm));
+                                      static_cast<float*>(ctx->tape.p) + at, need, T_out, status_out, r.stream, ctx->n_sm));
     if (plan.overlap) at += need;
     return FPT_OK;
   });
