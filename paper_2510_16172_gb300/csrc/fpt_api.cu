@@ -1798,6 +1798,8 @@ fpt_status fpt_mlp_train(fpt_ctx* ctx, fpt_mlp* m, const void* X, const float* T
   const __nv_bfloat16* Xs = static_cast<const __nv_bfloat16*>(X);
   float lr = p.lr;
   for (int ep = 0; ep < p.epochs; ++ep) {
+    // (lr_decay can take it to zero)
+    if (!(lr > 0.f)) return fail(ctx, FPT_EINVAL, "fpt_mlp_train: learning rate not positive in epoch %d", ep);
     // a new seeded order of the samples every epoch (splitmix64 of seed and epoch)
     uint64_t s0 = p.seed + 0x9E3779B97F4A7C15ULL * (uint64_t)(ep + 1);
     const uint64_t key = sm64_next(s0);

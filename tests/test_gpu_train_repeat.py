@@ -59,3 +59,18 @@ def test_repeated_gradients_agree(ctx, n):
         for g in runs:
             assert float((g[layer] - quiet[layer]).abs().max()) <= bound, name
     net.close()
+
+
+def test_train_refuses_a_learning_rate_decayed_to_zero(ctx):
+    """As fpt_mlp_train_step refuses it: 1e-3, 1e-23, 1e-43 (subnormal), then zero in FP32."""
+    import torch
+
+    net = fpt.Mlp(ctx, 5, SCALE)
+    X = torch.zeros((128, 64), dtype=torch.bfloat16, device="cuda")
+    T, G = torch.zeros((128, 8), device="cuda"), torch.zeros((128, 12), device="cuda")
+    assert len(net.train(X, T, G, epochs=3, batch=128, lr=1e-3, lr_decay=1e-20)) == 3
+    with pytest.raises(fpt.FptError, match="learning rate"):
+        net.train(X, T, G, epochs=4, batch=128, lr=1e-3, lr_decay=1e-20)
+    with pytest.raises(fpt.FptError, match="learning rate"):
+        net.train_step(X, T, G, 0.0)
+    net.close()
