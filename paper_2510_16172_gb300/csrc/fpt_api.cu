@@ -186,8 +186,7 @@ struct fpt_mlp {
   float* d_g = nullptr;          // gradient
   __nv_bfloat16* d_wb = nullptr;  // BF16 copy used by the tensor cores
   __nv_bfloat16* d_wt = nullptr;   // the weights as the fused kernels read them (mlp.h),
-  __nv_bfloat16* d_wtT = nullptr;  // and their transposes; both brought up to date when stale
-  bool wt_stale = true;
+  __nv_bfloat16* d_wtT = nullptr;  // and their transposes
   float* d_loss = nullptr;       // the batch's loss, behind the gradient (cleared with it)
   float* d_hist = nullptr;       // fpt_mlp_train: per-epoch mean losses
   size_t hist_cap = 0;
@@ -198,8 +197,6 @@ struct fpt_mlp {
   uint64_t train_cap = 0;
   __nv_bfloat16 *d_H = nullptr, *d_dZ = nullptr, *d_dYt = nullptr, *d_X = nullptr;
 };
-
-static fpt_status mlp_tiled_weights(fpt_ctx* ctx, fpt_mlp* m);
 
 static SceneDev scene_dev(const fpt_scene* s) {
   SceneDev d{};
@@ -1153,7 +1150,6 @@ static fpt_status solve_impl(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* 
     if (X) CUDA_OR_FAIL(ctx, cudaMemsetAsync(X, 0, b->dev.n_paths * (uint64_t)b->dev.n_max * 3 * sizeof(float), ctx->stream));
   }
   fpt_mlp* m = p.init_mode == 1 ? ctx->init_mlp : nullptr;
-  if (m && plan.count && (st = mlp_tiled_weights(ctx, m)) != FPT_OK) return st;
   CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_ctl, 0, kCtlBytes, ctx->stream));
   return run_orders(ctx, plan, [&](const OrderRun& r) -> fpt_status {
     if (m) {
@@ -1485,13 +1481,6 @@ static fpt_status mlp_ensure_ws(fpt_ctx* ctx, fpt_mlp* m, uint64_t B, bool train
   return FPT_OK;
 }
 
-static fpt_status mlp_tiled_weights(fpt_ctx* ctx, fpt_mlp* m) {
-  if (!m->wt_stale) return FPT_OK;
-  CUDA_OR_FAIL(ctx, launch_mlp_tile_weights(m->d_wb, m->d_wt, m->d_wtT, ctx->stream));
-  m->wt_stale = false;
-  return FPT_OK;
-}
-
 static GemmArgs gemm_args(int M, int N, int K, const __nv_bfloat16* A, long long sam, long long sak,
                           const __nv_bfloat16* Bm, long long sbn, long long sbk, int op, int* err) {
   GemmArgs g{};
@@ -1541,7 +1530,6 @@ static fpt_status mlp_forward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16
 static fpt_status mlp_backward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16* X, const float* T, const float* G,
                                     uint64_t B, uint64_t n, uint64_t first, uint64_t key, bool chained) {
   fpt_status st = mlp_ensure_ws(ctx, m, B, true);
-  if (st == FPT_OK) st = mlp_tiled_weights(ctx, m);
   if (st != FPT_OK) return st;
   if (!chained) CUDA_OR_FAIL(ctx, cudaMemsetAsync(m->d_g, 0, (kMlpParams + 1) * sizeof(float), ctx->stream));
   TrainArgs a{};
@@ -1659,10 +1647,12 @@ fpt_status fpt_mlp_set_params(fpt_mlp* m, const float* host) {
   CUDA_OR_FAIL(ctx, cudaMemcpy(m->d_w, host, kMlpParams * sizeof(float), cudaMemcpyHostToDevice));
   CUDA_OR_FAIL(ctx, cudaMemset(m->d_m, 0, kMlpParams * sizeof(float)));
   CUDA_OR_FAIL(ctx, cudaMemset(m->d_v, 0, kMlpParams * sizeof(float)));
+  // every layout that a kernel reads is written here and by each Adam step, so that no call (one recorded in a graph
+  // among them) depends on what ran before it
   CUDA_OR_FAIL(ctx, launch_to_bf16(m->d_w, m->d_wb, kMlpParams, ctx->stream));
+  CUDA_OR_FAIL(ctx, launch_mlp_tile_weights(m->d_wb, m->d_wt, m->d_wtT, ctx->stream));
   CUDA_OR_FAIL(ctx, cudaStreamSynchronize(ctx->stream));
   m->step = 0;
-  m->wt_stale = true;
   return FPT_OK;
 }
 
@@ -1831,8 +1821,6 @@ fpt_status fpt_mlp_infer(fpt_ctx* ctx, fpt_mlp* m, const fpt_scene* s, const fpt
   if (st != FPT_OK) return st;
   const SceneDev S = scene_dev(s);
   if (b->dev.n_paths == 0) return FPT_OK;
-  st = mlp_tiled_weights(ctx, m);
-  if (st != FPT_OK) return st;
   // Records carry their order, and a batch's lists follow the orders: one launch takes all orders whose records
   // hold the ids, one the longer sequences.  The kernel also clears the slots past a path's order.
   const PathRec* first = nullptr;
