@@ -190,10 +190,10 @@ struct fpt_mlp {
   float* d_loss = nullptr;       // the batch's loss, behind the gradient (cleared with it)
   float* d_hist = nullptr;       // fpt_mlp_train: per-epoch mean losses
   size_t hist_cap = 0;
-  // forward activations and outputs for up to cap rows
+  // forward activations for up to cap rows, where those of a training batch do not serve
   uint64_t cap = 0;
   __nv_bfloat16 *d_H1 = nullptr, *d_H2 = nullptr;
-  // operands of the weight gradients dW = dZ^T act for up to train_cap rows
+  // operands of the weight gradients dW = dZ^T act for up to train_cap rows (d_H: the activations of three layers)
   uint64_t train_cap = 0;
   __nv_bfloat16 *d_H = nullptr, *d_dZ = nullptr, *d_dYt = nullptr, *d_X = nullptr;
 };
@@ -1454,7 +1454,7 @@ static void mlp_free_ws(fpt_mlp* m) {
 // Buffers for B rows of a forward pass, or of a training batch.
 static fpt_status mlp_ensure_ws(fpt_ctx* ctx, fpt_mlp* m, uint64_t B, bool train) {
   const uint64_t want = B < 128 ? 128 : B;
-  if (want <= (train ? m->train_cap : m->cap)) return FPT_OK;
+  if (want <= m->train_cap || (!train && want <= m->cap)) return FPT_OK;
   cudaError_t e = cudaSuccess;
   auto bf = [&](__nv_bfloat16** p, size_t n) {
     cudaFree(*p);
@@ -1504,7 +1504,9 @@ static fpt_status mlp_forward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16
   const __nv_bfloat16* W = m->d_wb;
   const float* P = m->d_w;
   const __nv_bfloat16* in = X;
-  __nv_bfloat16* H[3] = {m->d_H1, m->d_H2, m->d_H1};
+  const bool own = B <= m->cap;  // else the training batch's, which mlp_ensure_ws has found large enough
+  __nv_bfloat16 *const H1 = own ? m->d_H1 : m->d_H, *const H2 = own ? m->d_H2 : m->d_H + m->train_cap * kMlpHidden;
+  __nv_bfloat16* H[3] = {H1, H2, H1};
   const int offW[3] = {kOffW1, kOffW2, kOffW3}, offB[3] = {kOffB1, kOffB2, kOffB3};
   for (int l = 0; l < 3; ++l) {
     const int K = l == 0 ? kMlpIn : kMlpHidden;

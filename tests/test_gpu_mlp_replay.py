@@ -1,4 +1,5 @@
-"""Captured calls of the network replayed after its parameters were set anew: they use the new ones throughout."""
+"""Captured calls of the network: replayed after its parameters were set anew they use the new ones throughout, and a
+forward pass no larger than a training batch before it needs no memory of its own (a capture cannot allocate)."""
 import pytest
 
 from paper_2510_16172_gb300 import fpt, scenes
@@ -70,5 +71,25 @@ def test_replayed_training_step_uses_the_parameters_set_last(ctx):
     b.train_step(X, T, G, lr)
     diff = abs(a.get_params() - b.get_params())
     assert (diff > 1e-3 * lr).mean() <= 0.01, (diff > 1e-3 * lr).mean()
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("n", [1, 100, 1000])
+def test_captured_forward_after_training_allocates_nothing(ctx, n):
+    import torch
+
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    X = (2.0 * torch.rand((1000, 64), generator=gen, device="cuda") - 1.0).to(torch.bfloat16)
+    T, G = torch.rand((1000, 8), generator=gen, device="cuda"), torch.rand((1000, 12), generator=gen, device="cuda")
+    a, b = fpt.Mlp(ctx, 0, SCALE), fpt.Mlp(ctx, 0, SCALE)
+    for net in (a, b):
+        net.set_params(numpy_params(3))
+    a.loss_grad(X, T, G)
+    rows = X[:n].clone()
+    g, Y = capture(ctx, lambda: a.forward(rows))
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(Y, b.forward(rows))
     a.close()
     b.close()
