@@ -642,14 +642,16 @@ __global__ void adam_kernel(float* __restrict__ w, float* __restrict__ m, float*
                             __nv_bfloat16* __restrict__ wt, __nv_bfloat16* __restrict__ wtT, float* __restrict__ loss,
                             float* hist, float hist_w, int clear) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool have = i < kMlpParams;
-  const float m0 = have ? m[i] : 0.f, v0 = have ? v[i] : 0.f, w0 = have ? w[i] : 0.f;
-  wait_previous();      // the gradient and the loss
+  // Not only the gradient and the loss, the weights and moments too are loaded after the wait.  The last step's Adam has
+  // completed by the time this one is launched, but that its writes are visible here is promised only by this grid's own
+  // wait.  (Loaded before it, while the weight gradients ran, they slowed those down: one epoch of 524,288
+  // samples 2.30 ms, 2.22 so.)
+  wait_previous();
   launch_dependents();  // the next step's CTAs set up and gather their rows
   if (i == 0 && hist) *hist += hist_w * *loss;
   if (i == 0 && clear) *loss = 0.f;
-  if (!have) return;
-  const float gi = g[i];
+  if (i >= kMlpParams) return;
+  const float gi = g[i], m0 = m[i], v0 = v[i], w0 = w[i];
   if (clear) g[i] = 0.f;
   const float mi = 0.9f * m0 + 0.1f * gi;
   const float vi = 0.999f * v0 + 0.001f * gi * gi;

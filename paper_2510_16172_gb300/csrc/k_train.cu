@@ -214,8 +214,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTrainThreads, 1)
   };
   if (warp >= kTrainEpiWarps && warp < kTrainEpiWarps + kTrainLoadWarps && my_tiles > 0) load_rows(0);
   wait_previous();  // what the last step's Adam wrote, and what its weight gradients read
-  // The weight gradients' CTAs set up on SMs this launch leaves idle or has left.  Only after the wait: they let the next
-  // Adam's CTAs load the weights and moments, which the last one must have written by then.
+  // The weight gradients' CTAs set up on SMs this launch leaves idle or has left.  Only after the wait, so that no
+  // later link of the chain starts before the last step is complete.
   launch_dependents();
   if (tid == 0) {
     tc::mbar_expect_tx(&sm.fixed, kMlpChunk + 4 * kMlpW4Chunk + kW4tBytes);
@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
   const int total = (int)((a.B + 63) / 64), per = (total + slices - 1) / slices;
   const int first = slice * per, last = first + per < total ? first + per : total;
   if (first >= last) return;  // (the whole CTA)
-  launch_dependents();  // Adam's CTAs fit beside this launch's and load the weights and moments meanwhile
+  launch_dependents();  // Adam's CTAs fit beside this launch's and wait there
   const int count = last - first;
   const int n_cols = job == 4 ? kMlpOut : (job == 1 ? kMlpIn : kMlpHidden);
   if (threadIdx.x == 0) {
