@@ -138,6 +138,8 @@ __global__ void __launch_bounds__(kThreads, kBackwardMinCtas<N>) backward_kernel
   uint64_t scan = (uint64_t)blockIdx.x * (unsigned)(rounds * kThreads);
   if (kChained<N> && (cfg.sel ? n_iter : n_local) <= stride) launch_dependents();  // one round: the FP64 pass sets up beside it
   unsigned head = 0, fill = 0;
+  // Tiles whose terms are in the FP32 partial sums.  A queue launch counts the tiles it has scanned, so that a flush comes
+  // after as many paths of the slice as where every path has its thread, however few of them carry a cotangent.
   int tiles = 0;
   for (uint64_t j0 = (uint64_t)blockIdx.x * blockDim.x;; j0 += stride) {
     bool have;
@@ -147,8 +149,10 @@ __global__ void __launch_bounds__(kThreads, kBackwardMinCtas<N>) backward_kernel
       have = j0 + threadIdx.x < n_iter;
       if (have) j = (uint64_t)cfg.sel[j0 + threadIdx.x];
     } else {
-      for (; fill < kThreads && scan < n_local; scan += stride * (unsigned)rounds)
+      for (; fill < kThreads && scan < n_local; scan += stride * (unsigned)rounds) {
         fill += backward_scan<N>(B, cfg, scan, n_local, list, status, dX, dLv, s_queue, head + fill, rounds);
+        tiles += rounds;
+      }
       if (fill == 0) break;
       have = threadIdx.x < fill;
       if (have) j = (uint64_t)s_queue[(head + threadIdx.x) & (kQueue - 1)];
@@ -236,7 +240,8 @@ __global__ void __launch_bounds__(kThreads, kBackwardMinCtas<N>) backward_kernel
     }
     warp_accumulate<3>(s_acc, have ? acc_tx + 3 * d.tx : -1, gtx, sm, gacc, acc_tx + 3 * d.tx);
     warp_accumulate<3>(s_acc, have ? acc_rx + 3 * d.rx : -1, grx, sm, gacc, acc_rx + 3 * d.rx);
-    if (sm && ++tiles >= cfg.flush_tiles) {
+    if (cfg.sel) ++tiles;
+    if (sm && tiles >= cfg.flush_tiles) {
       tiles = 0;
       __syncthreads();
       for (int k = threadIdx.x; k < n_acc; k += blockDim.x) {
