@@ -15,9 +15,16 @@
 // only the last chunk's four MMAs are exposed.  The next features go into the first activation chunk as
 // soon as the output layer has read it.
 //
-// Measured on 4 M city paths of orders 1-5: 2580 -> 1366 us (0.34 ns per path; the same bits).  What bounds it now
+// Hand-overs to the first CTA, whose thread issues the MMAs: the warps of each CTA arrive on its own barriers, and a thread
+// of the second CTA, which has seen their arrivals, passes them on by a 16-byte bulk copy that completes on the first CTA's
+// barrier.  That completion releases at cluster scope and holds no thread up.  (4 M city paths: the writers' own
+// arrivals on the remote barrier with a cluster-scope release 2135 us, one thread that passes them on with such
+// arrivals 1740, a thread per barrier 1685, the copies 1418.  Remote arrivals that release to the writers' own CTA
+// only, 1364, are not ordered for the other CTA's thread by the memory model.)
+//
+// Measured on 4 M city paths of orders 1-5: 2580 -> 1418 us (0.35 ns per path; the same bits).  What bounds it now
 // is the epilogues: 768 tanh per path at 16 a clock and SM are 6144 cycles per 128 paths (the MMAs 4900), and three
-// times per tile the last chunk's MMAs and two hand-overs between warps (about 1000 cycles) are exposed: 12,100
+// times per tile the last chunk's MMAs and the hand-overs (about 1200 cycles) are exposed: 12,600
 // cycles in all.  The rest of the GELU runs in packed FP32 pairs, five instructions for two values.
 //
 // Every wait is bounded; a role that runs out of time marks its CTA failed and leaves its loop, the others
@@ -42,15 +49,17 @@ struct InferSmem {
   float half_bias[3 * 256];   // of the hidden layers
   float bias4[16];
   uint64_t weights;           // this CTA's weights have arrived
-  uint64_t weights_pair;      // first CTA: both CTAs' have
-  uint64_t chunk[4];          // first CTA: activation chunk c is written in both CTAs
-  uint64_t feat;              // first CTA: the features are written in both CTAs
+  uint64_t weights_pair;      // first CTA: the second's have
+  // activation chunk c is written, the features are: by this CTA's warps; in the first CTA, by the second's too
+  uint64_t chunk[4];
+  uint64_t feat;
   uint64_t out_read;          // first CTA: the output layer's accumulator has been read in both CTAs
   uint64_t layer, out;        // MMAs of a hidden layer / of the output layer are done
   uint64_t chunk0;            // the output layer has read activation chunk 0
   uint64_t drain;
   uint32_t tmem;
   int fail;
+  uint4 word[5];              // of the hand-overs (chunks, features); never read
 };
 static_assert(sizeof(InferSmem) <= 227 * 1024, "one CTA per SM");
 
@@ -92,10 +101,10 @@ __device__ __forceinline__ uint32_t gelu_pair(uint32_t v0, uint32_t v1, uint64_t
   return *reinterpret_cast<const uint32_t*>(&p);
 }
 
-// A bounded wait of a whole warp: true only if every lane saw the phase complete (the lanes stay together for
-// the warp-wide instructions that follow).
+// A bounded wait of a whole warp for a commit of the pair's MMAs: true only if every lane saw the phase complete (the lanes
+// stay together for the warp-wide instructions that follow).
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity) {
-  return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, kWaitNs));
+  return __all_sync(0xffffffffu, tc::mbar_wait_cluster(bar, parity, kWaitNs));
 }
 
 template <int kSrc>
@@ -112,9 +121,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kInferThreads, 1)
   const uint64_t my_tiles = pair < n_tiles ? (n_tiles - pair + n_pairs - 1) / n_pairs : 0;
   if (tid == 0) {
     tc::mbar_init(&sm.weights, 1);
-    tc::mbar_init(&sm.weights_pair, 2);
-    for (int c = 0; c < 4; ++c) tc::mbar_init(&sm.chunk[c], 2 * kInferEpiWarps);
-    tc::mbar_init(&sm.feat, 2 * kInferFeatWarps);
+    tc::mbar_init(&sm.weights_pair, 1);
+    const uint32_t other = rank == 0 ? 1u : 0u;  // the second CTA's hand-over
+    for (int c = 0; c < 4; ++c) tc::mbar_init(&sm.chunk[c], kInferEpiWarps + other);
+    tc::mbar_init(&sm.feat, kInferFeatWarps + other);
     tc::mbar_init(&sm.out_read, 2 * kInferFeatWarps);
     tc::mbar_init(&sm.layer, 1);
     tc::mbar_init(&sm.out, 1);
@@ -152,12 +162,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kInferThreads, 1)
     const uint32_t lane_addr = tmem + ((rg * 32u) << 16) + part * 16u;
     uint4* const dst0 = reinterpret_cast<uint4*>(sm.act + tc::sw128_offset(row, part * 16u));
     uint4* const dst1 = reinterpret_cast<uint4*>(sm.act + tc::sw128_offset(row, part * 16u + 8u));
-    const uint32_t chunk_first = tc::map_rank(sm.chunk, 0);  // the first CTA's barriers
     auto hand_over = [&](int c) {
       tc::fence_async_smem();
       tc::fence_before_sync();
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive_remote_cta(chunk_first + 8u * c);
+      if (lane == 0) tc::mbar_arrive(&sm.chunk[c]);
     };
     uint32_t ph_layer = 0u;
     bool ok = true;
@@ -224,7 +233,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kInferThreads, 1)
           *reinterpret_cast<uint4*>(sm.act + tc::sw128_offset(row, k * 8)) = f[k];
         tc::fence_async_smem();
         __syncwarp();
-        if (lane == 0) tc::mbar_arrive_remote_cta(tc::map_rank(&sm.feat, 0));
+        if (lane == 0) tc::mbar_arrive(&sm.feat);
       }
       if (ti > 0) {
         if (!(ok = warp_wait(&sm.out, (uint32_t)(ti - 1) & 1u))) break;
@@ -233,7 +242,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kInferThreads, 1)
         tc::tmem_ld16(out_addr, v);
         tc::fence_before_sync();
         __syncwarp();
-        if (lane == 0) tc::mbar_arrive_remote_cta(tc::map_rank(&sm.out_read, 0));
+        if (lane == 0) tc::mbar_arrive_remote_relaxed(tc::map_rank(&sm.out_read, 0));
         if (info & 0xFFu) {
           float y[8];
 #pragma unroll
@@ -251,14 +260,36 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kInferThreads, 1)
   } else {
     if (lane == 0) {
       bool ok = tc::mbar_wait(&sm.weights, 0u, kWaitNs);
-      if (ok) tc::mbar_arrive_remote_cta(tc::map_rank(&sm.weights_pair, 0));
-      if (rank == 0) {
+      if (rank == 1) {
+        // ---- the second CTA's hand-overs, passed on in the order in which they come (the next tile's features follow the
+        // output layer's first chunk).  The first CTA waits for each of them before it leaves. ----
+        if (ok) tc::mbar_arrive_remote(tc::map_rank(&sm.weights_pair, 0));
+        const uint32_t words = tc::map_rank(sm.word, 0), chunks = tc::map_rank(sm.chunk, 0);
+        const uint32_t feat = tc::map_rank(&sm.feat, 0);
+        uint32_t ph_chunk = 0u;
+        auto pass_features = [&](uint64_t ti) {
+          ok = ok && tc::mbar_wait(&sm.feat, (uint32_t)ti & 1u, kWaitNs);
+          if (ok) tc::signal_remote(words + 4u * sizeof(uint4), sm.word + 4, feat);
+        };
+        if (my_tiles > 0) pass_features(0);
+        for (uint64_t ti = 0; ti < my_tiles && ok; ++ti) {
+          for (int l = 1; l < 4; ++l) {
+            for (int c = 0; c < 4 && ok; ++c) {
+              ok = tc::mbar_wait(&sm.chunk[c], ph_chunk, kWaitNs);
+              if (ok) tc::signal_remote(words + c * (uint32_t)sizeof(uint4), sm.word + c, chunks + 8u * c);
+            }
+            ph_chunk ^= 1u;
+          }
+          if (ti + 1 < my_tiles) pass_features(ti + 1);
+        }
+      } else {
         // ---- the pair's MMAs ----
         ok = ok && tc::mbar_wait_cluster(&sm.weights_pair, 0u, kWaitNs);
         const uint32_t w = tc::smem_u32(sm.w), act = tc::smem_u32(sm.act);
         constexpr uint32_t id256 = tc::idesc_bf16(256, 256), id32 = tc::idesc_bf16(256, 32);
         uint32_t ph_chunk = 0u, ph_feat = 0u;
         for (uint64_t ti = 0; ti < my_tiles && ok; ++ti) {
+          tc::mbar_expect_tx(&sm.feat, tc::kSignalBytes);
           if (!(ok = tc::mbar_wait_cluster(&sm.feat, ph_feat, kWaitNs))) break;
           ph_feat ^= 1u;
           tc::fence_after_sync();
@@ -270,6 +301,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kInferThreads, 1)
             const uint32_t acc = tmem + (l & 1 ? 256u : 0u);
             const uint32_t wl = w + (l == 1 ? kMlpTileW2 : (l == 2 ? kMlpTileW3 : kMlpTileW4));
             const uint32_t wc = l < 3 ? kMlpChunk : kMlpW4Chunk;
+            for (int c = 0; c < 4; ++c) tc::mbar_expect_tx(&sm.chunk[c], tc::kSignalBytes);
             for (int c = 0; c < 4; ++c) {
               if (!(ok = tc::mbar_wait_cluster(&sm.chunk[c], ph_chunk, kWaitNs))) break;
               tc::fence_after_sync();

@@ -125,12 +125,14 @@ __device__ __forceinline__ uint32_t map_rank(const void* p, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
   return a;
 }
-// One arrival on another CTA's barrier (addr from map_rank), ordering this thread's earlier writes for its own CTA
-// only: enough where the other CTA's thread goes on to issue an MMA whose operands the writers' proxy fence has made
-// visible to the tensor core that reads them, each CTA's own shared memory.  (A release to the cluster waits for
-// every earlier store of the thread: 400-850 cycles measured.)
-__device__ __forceinline__ void mbar_arrive_remote_cta(uint32_t addr) {
-  asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+// One arrival on another CTA's barrier (addr from map_rank), releasing this thread's earlier writes, and those it has
+// seen, to the cluster.  The release waits for them: 400-850 cycles measured (signal_remote does not hold the thread up).
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+// The same without ordering memory: enough between tcgen05 operations, which their own thread-sync fences order.
+__device__ __forceinline__ void mbar_arrive_remote_relaxed(uint32_t addr) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
@@ -226,6 +228,13 @@ __device__ __forceinline__ void bulk_s2s(uint32_t dst, const void* src_smem, uin
       "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
       "r"(smem_u32(src_smem)), "r"(bytes), "r"(bar)
       : "memory");
+}
+// A hand-over to another CTA: a copy of one 16-byte word whose completion there is kSignalBytes transactions on the barrier,
+// a release at cluster scope of what this thread has seen to be written (after the writers' proxy fence and an acquire of
+// their arrivals, as before any bulk copy of their data).  The thread goes on at once.
+constexpr uint32_t kSignalBytes = 16;
+__device__ __forceinline__ void signal_remote(uint32_t dst_word, const uint4* src_word, uint32_t bar) {
+  bulk_s2s(dst_word, src_word, kSignalBytes, bar);
 }
 
 // ---- fences ----------------------------------------------------------------
