@@ -1721,8 +1721,8 @@ fpt_status fpt_mlp_features(fpt_ctx* ctx, const fpt_mlp* m, const fpt_scene* s, 
   if (!m || !X) return fail(ctx, FPT_EINVAL, "null argument");
   CUDA_OR_FAIL(ctx, cudaSetDevice(ctx->device));
   ProfScope ps(ctx, FPT_K_OTHER);
-  CUDA_OR_FAIL(ctx, launch_mlp_features(scene_dev(s), b->dev, 0, nullptr, 0, b->dev.n_paths, 1.f / m->scale,
-                                        static_cast<__nv_bfloat16*>(X), G, ctx->stream));
+  CUDA_OR_FAIL(ctx, launch_mlp_features(scene_dev(s), b->dev, 1.f / m->scale, static_cast<__nv_bfloat16*>(X), G,
+                                        ctx->stream));
   return FPT_OK;
 }
 

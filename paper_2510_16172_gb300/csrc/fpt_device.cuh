@@ -401,18 +401,6 @@ __device__ __forceinline__ uint64_t slice_global(const BatchDev& B, int n, const
   return pair * B.per_pair + B.offset[n] + (j - pair * kn);
 }
 
-// Path source for one per-order launch: exhaustive batches need no list; other
-// batches pass their bucket of decoded path records.
-__device__ __forceinline__ void fetch_path(const BatchDev& B, int n, const PathRec* list, uint64_t j,
-                                           PathDesc& d) {
-  if (list == nullptr) {
-    decode_exhaustive_order(B, n, j, d);
-  } else {
-    load_rec(list, j, d);
-    if (n > kMaxBfgsOrder) decode_global(B, d.g, d);
-  }
-}
-
 // Path source of a kernel compiled for order N: the bucket of records, else the
 // exhaustive enumeration of order N (both keep the descriptor in registers).
 template <int N>

@@ -270,10 +270,6 @@ constexpr int kWsStageBytes = kWsTileA + 256 * 128;       // + B, up to 256 rows
 // the ring, two 2 KB output staging buffers per epilogue warp, slack to align the ring to 1024 bytes
 constexpr int kWsSmem = kWsStages * kWsStageBytes + kWsEpiWarps * 2 * 2048 + 1024;
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
-}
-
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
 // Which accesses may take 16 bytes (unit stride along n, row strides and bases aligned).
@@ -520,7 +516,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
         ws_epilogue<EPI_BIAS_GELU>(g, ev, tacc, m, mrow0, j0, n_groups, &tmOut, tma_out != 0, stg, gi);
       tc::fence_before_sync();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[b]);
+      if (lane == 0) tc::mbar_arrive(&acc_empty[b]);
     }
     // every TMA store of this warp has completed before its staging buffers go away
     if (lane == 0) tc::bulk_wait_all();
@@ -622,15 +618,11 @@ cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t stream) {
 // features, Adam, learned start
 // ---------------------------------------------------------------------------
 
-// all paths of a batch (global index order) or one order slice (local index order)
-__global__ void mlp_features_kernel(SceneDev S, BatchDev B, int n, const PathRec* list, uint64_t first,
-                                    uint64_t count, float inv_scale, __nv_bfloat16* X, float* G) {
-  for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count; k += (uint64_t)gridDim.x * blockDim.x) {
+__global__ void mlp_features_kernel(SceneDev S, BatchDev B, float inv_scale, __nv_bfloat16* X, float* G) {
+  for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < B.n_paths;
+       k += (uint64_t)gridDim.x * blockDim.x) {
     PathDesc d;
-    if (n > 0)
-      fetch_path(B, n, list, first + k, d);
-    else
-      decode_global(B, first + k, d);
+    decode_global(B, k, d);
     path_features(S, d, inv_scale, X + k * kMlpIn, G ? G + k * 12 : nullptr);
   }
 }
@@ -680,10 +672,10 @@ static unsigned grid_1d(uint64_t n, int threads, int cap) {
   return (unsigned)(g < (uint64_t)cap ? (g ? g : 1) : (uint64_t)cap);
 }
 
-cudaError_t launch_mlp_features(const SceneDev& S, const BatchDev& B, int n, const PathRec* list, uint64_t first,
-                                uint64_t count, float inv_scale, __nv_bfloat16* X, float* G, cudaStream_t stream) {
-  if (!count) return cudaSuccess;
-  mlp_features_kernel<<<grid_1d(count, 128, 4096), 128, 0, stream>>>(S, B, n, list, first, count, inv_scale, X, G);
+cudaError_t launch_mlp_features(const SceneDev& S, const BatchDev& B, float inv_scale, __nv_bfloat16* X, float* G,
+                                cudaStream_t stream) {
+  if (!B.n_paths) return cudaSuccess;
+  mlp_features_kernel<<<grid_1d(B.n_paths, 128, 4096), 128, 0, stream>>>(S, B, inv_scale, X, G);
   count_launch();
   return cudaGetLastError();
 }

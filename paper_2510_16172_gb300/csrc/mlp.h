@@ -38,8 +38,9 @@ struct GemmArgs {
 bool encode_map(CUtensorMap* map, CUtensorMapDataType type, int rank, const void* base, const cuuint64_t* dims,
                 const cuuint64_t* strides, const cuuint32_t* box, CUtensorMapSwizzle swizzle);
 cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t stream);
-cudaError_t launch_mlp_features(const SceneDev& S, const BatchDev& B, int n, const PathRec* list, uint64_t first,
-                                uint64_t count, float inv_scale, __nv_bfloat16* X, float* G, cudaStream_t stream);
+// Features (and Gram entries, if G) of every path of a batch, by global index.
+cudaError_t launch_mlp_features(const SceneDev& S, const BatchDev& B, float inv_scale, __nv_bfloat16* X, float* G,
+                                cudaStream_t stream);
 // One Adam step, with the BF16 copies of the parameters (plain and as launch_mlp_tile_weights lays them out); with
 // hist, also *hist += hist_w * *loss; with clear, g and *loss are zero afterwards.
 cudaError_t launch_adam(float* w, float* m, float* v, float* g, float lr, float c1, float c2, __nv_bfloat16* wb,
@@ -48,7 +49,9 @@ cudaError_t launch_adam(float* w, float* m, float* v, float* g, float lr, float 
 cudaError_t launch_to_bf16(const float* src, __nv_bfloat16* dst, int n, cudaStream_t stream);
 // The weights as the fused kernels' CTA pairs read them (k_infer.cu, k_train.cu): CTA r of a pair holds outputs
 // 128 r .. 128 r + 127 of the hidden layers in chunks of 64 inputs, and the whole output layer; transposed, for the
-// back-propagation, inputs 128 r .. 128 r + 127.  Every piece is K-major in core matrices (tc.cuh).
+// back-propagation, inputs 128 r .. 128 r + 127.  Chunks of 64 columns are K-major in the 128-byte swizzled layout
+// (tc.cuh, sw128_offset, read through smem_desc_sw128); only the transposed output layer, 16 columns, is in core
+// matrices (kmajor_offset, smem_desc).
 constexpr uint32_t kMlpChunk = 128 * 64 * 2;   // 128 rows x 64 columns
 constexpr uint32_t kMlpW4Chunk = 16 * 64 * 2;  // the output layer's 16 rows
 constexpr uint32_t kMlpTileW2 = kMlpChunk, kMlpTileW3 = 5 * kMlpChunk, kMlpTileW4 = 9 * kMlpChunk;

@@ -1,12 +1,16 @@
 // tc.cuh -- 5th-generation tensor core (tcgen05) building blocks for sm_103a.
 //
-// Operands live in shared memory in the canonical K-major layout without
-// swizzle: the tile is cut into "core matrices" of 8 rows x 16 bytes (8 bf16);
-// a core matrix is 128 contiguous bytes (row r at +16 r).  Core matrix (rg, kg)
-// of an R x K tile sits at byte ((rg * (K / 8)) + kg) * 128, so neighbours
-// along K are 128 B apart (leading byte offset) and neighbours along the rows
-// are K * 16 B apart (stride byte offset).  One MMA consumes K = 16 (two core
-// matrices along K); step kk starts at tile + kk * 256 B.
+// Operands live in shared memory in one of three layouts.
+// K-major, 128-byte swizzled (smem_desc_sw128, sw128_offset; what TMA loads write with that swizzle): 64 columns a
+// tile, a row of 128 bytes, its 16-byte unit u at unit u ^ (row mod 8), tiles on 1024-byte boundaries.  One MMA consumes
+// K = 16: step kk starts 32 bytes further.  The network's activations, weights and GEMM operands.
+// The same boxes read MN-major (the descriptors of k_train.cu): 64 columns of M or N by 64 rows of K, for operands used
+// transposed; 16 rows of K are 2048 bytes.
+// K-major without swizzle (smem_desc, kmajor_offset): the tile is cut into "core matrices" of 8 rows x 16 bytes (8
+// bf16); a core matrix is 128 contiguous bytes (row r at +16 r).  Core matrix (rg, kg) of an R x K tile sits
+// at byte ((rg * (K / 8)) + kg) * 128, so neighbours along K are 128 B apart (leading byte offset) and neighbours
+// along the rows are K * 16 B apart (stride byte offset); step kk of an MMA starts at tile + kk * 256 B.  gemm_kernel's
+// gathered operands, and the training kernel's 16-column dY and W4^T.
 //
 // The accumulator lives in tensor memory (TMEM): lane = output row, column =
 // output column, 32-bit FP32 values.  One thread issues the MMAs; completion is
@@ -23,7 +27,7 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// byte offset of element (r, k) in an R x K bf16 tile in the layout above
+// byte offset of element (r, k) in an R x K bf16 tile in core matrices
 __host__ __device__ __forceinline__ uint32_t kmajor_offset(uint32_t r, uint32_t k, uint32_t K) {
   return ((r >> 3) * (K >> 3) + (k >> 3)) * 128u + (r & 7u) * 16u + (k & 7u) * 2u;
 }
