@@ -40,8 +40,7 @@ struct fpt_ctx {
   int n_sm = 0;
   cudaStream_t stream = nullptr;
   int* d_err = nullptr;                    // device error word
-  double* d_gacc = nullptr;                // backward accumulators (FP64)
-  size_t gacc_cap = 0;
+  Scratch gacc;                            // backward accumulators (FP64)
   Scratch tape;                            // per-step state of fpt_backward_unrolled
   unsigned long long* d_count = nullptr;   // counters for reductions
   unsigned char* d_ctl = nullptr;          // launch counters of the orders (OrderCtl), cleared once per call
@@ -282,7 +281,6 @@ void fpt_destroy(fpt_ctx* ctx) {
   }
   for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
   cudaFree(ctx->d_err);
-  cudaFree(ctx->d_gacc);
   cudaFree(ctx->d_count);
   cudaFree(ctx->d_ctl);
   for (int k = 0; k < fpt_ctx::kSide; ++k) {
@@ -296,7 +294,7 @@ void fpt_destroy(fpt_ctx* ctx) {
   }
   if (ctx->ofork_ev) cudaEventDestroy(ctx->ofork_ev);
   cudaFree(ctx->d_dropped);
-  for (const Scratch* s : {&ctx->rescue, &ctx->step, &ctx->tape}) cudaFree(s->p);
+  for (const Scratch* s : {&ctx->gacc, &ctx->rescue, &ctx->step, &ctx->tape}) cudaFree(s->p);
   for (void* p : ctx->kept) cudaFree(p);
   delete ctx;
 }
@@ -890,6 +888,9 @@ static cudaError_t reserve(fpt_ctx* ctx, Scratch& s, size_t bytes, bool in_captu
   return cudaSuccess;
 }
 
+// The backward accumulators (ensure_gacc).
+static double* gacc(const fpt_ctx* ctx) { return static_cast<double*>(ctx->gacc.p); }
+
 // Path scratch for `entries` paths (three uint32 lists of them) and `steps` floats of first Newton steps.
 static cudaError_t reserve_paths(fpt_ctx* ctx, uint64_t entries, size_t steps, bool in_capture, bool must) {
   const cudaError_t e = reserve(ctx, ctx->rescue, 3 * entries * sizeof(uint32_t), in_capture, must);
@@ -1025,7 +1026,7 @@ static fpt_status backward_order(fpt_ctx* ctx, const SceneDev& S, const fpt_batc
   BackwardCfg cfg_n = cfg;
   cfg_n.sel = r.lists + 2 * r.cnt;  // the third list of the scratch (the polish's, free here)
   cfg_n.sel_count = &r.ctl->selected;
-  CUDA_OR_FAIL(ctx, launch_backward(r.n, S, b->dev, cfg_n, r.cnt, r.list, T, status, dX, dL, ctx->d_gacc, r.stream,
+  CUDA_OR_FAIL(ctx, launch_backward(r.n, S, b->dev, cfg_n, r.cnt, r.list, T, status, dX, dL, gacc(ctx), r.stream,
                                     ctx->n_sm, r.lists, &r.ctl->backward64));
   return FPT_OK;
 }
@@ -1187,15 +1188,9 @@ fpt_status fpt_solve(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* bc, cons
 
 // Context-owned FP64 gradient accumulators, sized for the scene and cleared.
 static fpt_status ensure_gacc(fpt_ctx* ctx, const fpt_scene* s) {
-  const size_t need = (size_t)(9 * s->n_obj + 3 * (s->n_tx + s->n_rx));
-  if (need > ctx->gacc_cap) {
-    cudaFree(ctx->d_gacc);
-    ctx->d_gacc = nullptr;
-    ctx->gacc_cap = 0;
-    CUDA_OR_FAIL(ctx, cudaMalloc(&ctx->d_gacc, need * sizeof(double)));
-    ctx->gacc_cap = need;
-  }
-  CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->d_gacc, 0, need * sizeof(double), ctx->stream));
+  const size_t bytes = (size_t)(9 * s->n_obj + 3 * (s->n_tx + s->n_rx)) * sizeof(double);
+  CUDA_OR_FAIL(ctx, reserve(ctx, ctx->gacc, bytes, capturing(ctx), true));
+  CUDA_OR_FAIL(ctx, cudaMemsetAsync(ctx->gacc.p, 0, bytes, ctx->stream));
   return FPT_OK;
 }
 
@@ -1234,7 +1229,7 @@ fpt_status fpt_solve_grad(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* bc,
     gc.dl_mask = dL ? (uint8_t)0 : dL_status_mask;
     gc.cond_adj = p.cond_fp64;
     gc.deg_tol = prm->deg_tol;
-    gc.gacc = ctx->d_gacc;
+    gc.gacc = gacc(ctx);
     gc.flush_tiles = ctx->acc_flush_tiles;
     gc.acc_in_smem = ctx->acc_smem;
     gc.dropped = ctx->d_dropped;
@@ -1243,7 +1238,7 @@ fpt_status fpt_solve_grad(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* bc,
   if (st != FPT_OK) return st;
   const SceneDev S = scene_dev(s);
   ProfScope ps(ctx, FPT_K_OTHER);
-  CUDA_OR_FAIL(ctx, launch_backward_finalize(S, nullptr, ctx->d_gacc, g_tx, g_rx, g_vertices, ctx->stream));
+  CUDA_OR_FAIL(ctx, launch_backward_finalize(S, nullptr, gacc(ctx), g_tx, g_rx, g_vertices, ctx->stream));
   return FPT_OK;
 }
 
@@ -1297,7 +1292,7 @@ fpt_status fpt_backward(fpt_ctx* ctx, const fpt_scene* s, const fpt_batch* bc, c
   if (st != FPT_OK) return st;
   {
     ProfScope ps(ctx, FPT_K_OTHER);
-    CUDA_OR_FAIL(ctx, launch_backward_finalize(S, nullptr, ctx->d_gacc, g_tx, g_rx, g_vertices, ctx->stream));
+    CUDA_OR_FAIL(ctx, launch_backward_finalize(S, nullptr, gacc(ctx), g_tx, g_rx, g_vertices, ctx->stream));
   }
   return FPT_OK;
 }
@@ -1346,7 +1341,7 @@ fpt_status fpt_backward_unrolled(fpt_ctx* ctx, const fpt_scene* s, const fpt_bat
   st = run_orders(ctx, plan, [&](const OrderRun& r) -> fpt_status {
     ProfScope ps(ctx, FPT_K_BACKWARD);
     const size_t need = tape_floats(r);
-    CUDA_OR_FAIL(ctx, launch_unrolled(r.n, S, b->dev, steps, fp_iters, r.cnt, r.list, dX, dL, ctx->d_gacc,
+    CUDA_OR_FAIL(ctx, launch_unrolled(r.n, S, b->dev, steps, fp_iters, r.cnt, r.list, dX, dL, gacc(ctx),
                                       static_cast<float*>(ctx->tape.p) + at, need, T_out, status_out, r.stream, ctx->n_sm));
     if (plan.overlap) at += need;
     return FPT_OK;
@@ -1354,7 +1349,7 @@ fpt_status fpt_backward_unrolled(fpt_ctx* ctx, const fpt_scene* s, const fpt_bat
   if (st != FPT_OK) return st;
   {
     ProfScope ps(ctx, FPT_K_OTHER);
-    CUDA_OR_FAIL(ctx, launch_backward_finalize(S, nullptr, ctx->d_gacc, g_tx, g_rx, g_vertices, ctx->stream));
+    CUDA_OR_FAIL(ctx, launch_backward_finalize(S, nullptr, gacc(ctx), g_tx, g_rx, g_vertices, ctx->stream));
   }
   return FPT_OK;
 }

@@ -96,3 +96,18 @@ def test_graph_outlives_its_scratch(ctx):
     again = everything(ctx, *large)
     torch.cuda.synchronize()
     agree(again, direct)
+
+
+def test_graph_outlives_its_accumulators(ctx):
+    """The gradient sums are sized for the scene: a later call on a larger one."""
+    scene, batch = batch_of(ctx, 3000)
+    want = everything(ctx, scene, batch)
+    ctx.sync()
+    g, out = captured(ctx, scene, batch)
+    sc = scenes.city(1, n_obj=400, n_rx=2)
+    other = fpt.Scene(ctx, sc.types, sc.verts, sc.tx, sc.rx)
+    small = fpt.Batch.seeded(ctx, other, 17, 1000, 1, 4)
+    direct = everything(ctx, other, small)
+    ctx.sync()
+    agree(replayed(g, out), want)
+    agree(everything(ctx, other, small), direct)
