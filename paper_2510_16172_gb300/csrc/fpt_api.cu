@@ -189,12 +189,17 @@ struct fpt_mlp {
   float* d_loss = nullptr;       // the batch's loss, behind the gradient (cleared with it)
   float* d_hist = nullptr;       // fpt_mlp_train: per-epoch mean losses
   size_t hist_cap = 0;
-  // forward activations for up to cap rows, where those of a training batch do not serve
+  // activations of two layers for a forward pass of up to cap rows, where those of a training batch do not serve
+  Scratch fwd;
   uint64_t cap = 0;
-  __nv_bfloat16 *d_H1 = nullptr, *d_H2 = nullptr;
-  // operands of the weight gradients dW = dZ^T act for up to train_cap rows (d_H: the activations of three layers)
+  // operands of the weight gradients dW = dZ^T act for a training batch of up to train_cap rows: activations and
+  // gradients of the three hidden layers, features, transposed gradient at the outputs
+  Scratch train;
   uint64_t train_cap = 0;
-  __nv_bfloat16 *d_H = nullptr, *d_dZ = nullptr, *d_dYt = nullptr, *d_X = nullptr;
+  __nv_bfloat16* H() const { return static_cast<__nv_bfloat16*>(train.p); }
+  __nv_bfloat16* dZ() const { return H() + 3 * train_cap * kMlpHidden; }
+  __nv_bfloat16* Xb() const { return dZ() + 3 * train_cap * kMlpHidden; }
+  __nv_bfloat16* dYt() const { return Xb() + train_cap * kMlpIn; }
 };
 
 static SceneDev scene_dev(const fpt_scene* s) {
@@ -1438,41 +1443,20 @@ fpt_status fpt_count_status(fpt_ctx* ctx, const uint8_t* status, uint64_t n, uin
 // ---------------------------------------------------------------------------
 // learned warm start
 // ---------------------------------------------------------------------------
-static void mlp_free_ws(fpt_mlp* m) {
-  for (__nv_bfloat16** p : {&m->d_H1, &m->d_H2, &m->d_H, &m->d_dZ, &m->d_dYt, &m->d_X}) {
-    cudaFree(*p);
-    *p = nullptr;
-  }
-  m->cap = m->train_cap = 0;
-}
-
-// Buffers for B rows of a forward pass, or of a training batch.
+// Scratch for B rows of a forward pass, or of a training batch.
 static fpt_status mlp_ensure_ws(fpt_ctx* ctx, fpt_mlp* m, uint64_t B, bool train) {
-  const uint64_t want = B < 128 ? 128 : B;
-  if (want <= m->train_cap || (!train && want <= m->cap)) return FPT_OK;
-  cudaError_t e = cudaSuccess;
-  auto bf = [&](__nv_bfloat16** p, size_t n) {
-    cudaFree(*p);
-    *p = nullptr;
-    if (e == cudaSuccess) e = cudaMalloc(p, n * sizeof(__nv_bfloat16));
-  };
-  const size_t H = want * kMlpHidden;
-  if (train) {
-    m->train_cap = 0;
-    bf(&m->d_H, 3 * H);
-    bf(&m->d_dZ, 3 * H);
-    bf(&m->d_dYt, (want + 7) / 8 * 8 * kMlpOut);
-    bf(&m->d_X, want * kMlpIn);
-  } else {
-    m->cap = 0;
-    bf(&m->d_H1, H);
-    bf(&m->d_H2, H);
-  }
+  const uint64_t rows = B < 128 ? 128 : B;
+  const bool shared = !train && rows > m->cap && rows <= m->train_cap;  // a forward pass in the training batch's
+  uint64_t& cap = train || shared ? m->train_cap : m->cap;
+  const uint64_t want = rows > cap ? rows : cap;
+  const size_t elems = train || shared ? want * (6 * kMlpHidden + kMlpIn) + (want + 7) / 8 * 8 * kMlpOut
+                                       : want * 2 * kMlpHidden;
+  const cudaError_t e = reserve(ctx, train || shared ? m->train : m->fwd, elems * sizeof(__nv_bfloat16), capturing(ctx), true);
   if (e != cudaSuccess) {
-    mlp_free_ws(m);
+    cap = 0;
     return fail(ctx, FPT_ENOMEM, "MLP workspace for %llu rows: %s", (unsigned long long)want, cudaGetErrorString(e));
   }
-  (train ? m->train_cap : m->cap) = want;
+  cap = want;
   return FPT_OK;
 }
 
@@ -1500,7 +1484,8 @@ static fpt_status mlp_forward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat16
   const float* P = m->d_w;
   const __nv_bfloat16* in = X;
   const bool own = B <= m->cap;  // else the training batch's, which mlp_ensure_ws has found large enough
-  __nv_bfloat16 *const H1 = own ? m->d_H1 : m->d_H, *const H2 = own ? m->d_H2 : m->d_H + m->train_cap * kMlpHidden;
+  __nv_bfloat16* const H1 = own ? static_cast<__nv_bfloat16*>(m->fwd.p) : m->H();
+  __nv_bfloat16* const H2 = H1 + (own ? m->cap : m->train_cap) * kMlpHidden;
   __nv_bfloat16* H[3] = {H1, H2, H1};
   const int offW[3] = {kOffW1, kOffW2, kOffW3}, offB[3] = {kOffB1, kOffB2, kOffB3};
   for (int l = 0; l < 3; ++l) {
@@ -1541,10 +1526,10 @@ static fpt_status mlp_backward_impl(fpt_ctx* ctx, fpt_mlp* m, const __nv_bfloat1
   a.wt = m->d_wt;
   a.wtT = m->d_wtT;
   a.params = m->d_w;
-  a.Xb = m->d_X;
-  a.H = m->d_H;
-  a.dZ = m->d_dZ;
-  a.dYt = m->d_dYt;
+  a.Xb = m->Xb();
+  a.H = m->H();
+  a.dZ = m->dZ();
+  a.dYt = m->dYt();
   a.ldY = (B + 7) / 8 * 8;
   a.grad = m->d_g;
   a.loss = m->d_loss;
@@ -1618,7 +1603,8 @@ fpt_status fpt_mlp_create(fpt_ctx* ctx, uint64_t seed, float length_scale, fpt_m
 void fpt_mlp_free(fpt_mlp* m) {
   if (!m) return;
   if (m->ctx && m->ctx->init_mlp == m) m->ctx->init_mlp = nullptr;
-  mlp_free_ws(m);
+  cudaFree(m->fwd.p);
+  cudaFree(m->train.p);
   for (void* p : {(void*)m->d_w, (void*)m->d_m, (void*)m->d_v, (void*)m->d_g, (void*)m->d_wb, (void*)m->d_wt,
                   (void*)m->d_wtT, (void*)m->d_hist})
     cudaFree(p);

@@ -93,3 +93,35 @@ def test_captured_forward_after_training_allocates_nothing(ctx, n):
     assert torch.equal(Y, b.forward(rows))
     a.close()
     b.close()
+
+
+def test_graphs_outlive_their_workspace(ctx):
+    """A captured forward pass and a captured training step, replayed after larger ones of the same network; the step against
+    one of a second network from the same parameters (see above)."""
+    import torch
+
+    gen = torch.Generator(device="cuda").manual_seed(8)
+    X = (2.0 * torch.rand((20_000, 64), generator=gen, device="cuda") - 1.0).to(torch.bfloat16)
+    T = 2.0 * torch.rand((20_000, 8), generator=gen, device="cuda") - 0.5
+    G = torch.randn((20_000, 12), generator=gen, device="cuda") ** 2
+    lr = 1e-3
+    few = [t[:700].clone() for t in (X, T, G)]
+    a, b = fpt.Mlp(ctx, 0, SCALE), fpt.Mlp(ctx, 0, SCALE)
+    for net in (a, b):
+        net.set_params(numpy_params(5))
+    want = b.forward(few[0])
+    a.loss_grad(*few)
+    forward, Y = capture(ctx, lambda: a.forward(few[0]))
+    step, _ = capture(ctx, lambda: a.train_step(*few, lr, want_loss=False))
+    a.loss_grad(X, T, G)
+    a.set_params(numpy_params(5))
+    Y.zero_()
+    forward.replay()
+    step.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(Y, want)
+    b.train_step(*few, lr)
+    diff = abs(a.get_params() - b.get_params())
+    assert (diff > 1e-3 * lr).mean() <= 0.01, (diff > 1e-3 * lr).mean()
+    a.close()
+    b.close()
