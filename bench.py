@@ -167,7 +167,7 @@ NCU_TRAFFIC = {
     ("f6467978743f", "bfgs"): 568.6e6,
     ("886638d3c5ec", "bfgs"): 568.8e6,
     ("e1979203e5c7", "bfgs"): 567.1e6,
-    ("825f0b7fe12d", "bfgs"): 564.5e6,
+    ("aae16943659c", "bfgs"): 564.7e6,
 }
 
 

@@ -125,8 +125,8 @@ void fpt_default_params(fpt_solve_params* p);
  * largest order's otherwise or where the memory is not there), and
  * fpt_backward_unrolled's tape (at most 16 GiB).  A call that is captured
  * into a graph takes the workspace as it stands; a later call that needs more
- * leaves what the graph uses in place.  Returns FPT_ECUDA if the device cannot
- * be used. */
+ * leaves what the graph uses in place, in a network's workspace too.  Returns
+ * FPT_ECUDA if the device cannot be used. */
 fpt_status fpt_create(fpt_ctx** out, int device, void* cuda_stream);
 void fpt_destroy(fpt_ctx* ctx);
 /* Switch the context's stream.  No synchronisation (legal inside a stream

@@ -25,8 +25,9 @@ namespace fpt {
 // carry a cotangent (kScanRounds kThreads consecutive ones at a time, a lane per path) into a queue in shared memory, in
 // index order, and takes a full CTA of them at a time.  A loss on the valid paths of a canyon touches 7 % of them; one
 // thread per path of the slice left nearly every warp running the whole adjoint for two lanes.
-// Measured on 2.16 M canyon paths of orders 1-3 with point and length cotangents on the valid ones:
-// 194 -> 95 us a call (126 before the loads of four rounds went out together).
+// Measured on 2.16 M canyon paths of orders 1-3 with point and length cotangents on the valid ones, as the step was made:
+// 194 -> 95 us a call (126 before the loads of four rounds went out together); with the rest of the path's changes
+// 226 -> 97 to 106 from GPU to GPU, a first pass on new cotangents 282 -> 162.
 // (One round at a time where the slice is too small to give every CTA of the launch four.)
 constexpr int kScanRounds = 4, kQueue = 1024;
 static_assert((kScanRounds + 2) * kThreads <= kQueue, "queue entries");
