@@ -10,7 +10,6 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
-#include <functional>
 #include <new>
 #include <utility>
 #include <vector>
@@ -883,10 +882,16 @@ static cudaError_t reserve(fpt_ctx* ctx, Scratch& s, size_t bytes, bool in_captu
       if (!must) cudaGetLastError();
       return e;
     }
-    if (s.captured)
-      ctx->kept.push_back(s.p);
-    else
+    if (s.captured) {
+      try {
+        ctx->kept.push_back(s.p);
+      } catch (...) {  // (no exception leaves a C entry)
+        cudaFree(p);
+        return cudaErrorMemoryAllocation;
+      }
+    } else {
       cudaFree(s.p);
+    }
     s = Scratch{p, bytes, false};
   }
   s.captured = s.captured || in_capture;
@@ -982,8 +987,10 @@ static fpt_status plan_orders(fpt_ctx* ctx, const fpt_batch* b, bool scratch, bo
   return FPT_OK;
 }
 
-static fpt_status run_orders(fpt_ctx* ctx, const OrderPlan& plan,
-                             const std::function<fpt_status(const OrderRun&)>& body) {
+// (body as it is: a std::function of it would allocate, and could throw across the C entries)
+extern "C++" {
+template <class Body>
+static fpt_status run_orders(fpt_ctx* ctx, const OrderPlan& plan, const Body& body) {
   const int used = !plan.overlap ? 0 : (plan.count - 1 < fpt_ctx::kOrderStreams ? plan.count - 1 : fpt_ctx::kOrderStreams);
   if (used) {
     CUDA_OR_FAIL(ctx, cudaEventRecord(ctx->ofork_ev, ctx->stream));
@@ -992,13 +999,16 @@ static fpt_status run_orders(fpt_ctx* ctx, const OrderPlan& plan,
   fpt_status st = FPT_OK;
   for (int i = 0; i < plan.count && st == FPT_OK; ++i) st = body(plan.runs[i]);
   // joined also after an error: later calls reuse the scratch, and a stream capture must end joined
+  cudaError_t joined = cudaSuccess;
   for (int k = 0; k < used; ++k) {
-    const cudaError_t e = cudaEventRecord(ctx->ojoin_ev[k], ctx->ostream[k]);
-    const cudaError_t w = e == cudaSuccess ? cudaStreamWaitEvent(ctx->stream, ctx->ojoin_ev[k], 0) : e;
-    if (st == FPT_OK) CUDA_OR_FAIL(ctx, w);
+    cudaError_t e = cudaEventRecord(ctx->ojoin_ev[k], ctx->ostream[k]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, ctx->ojoin_ev[k], 0);
+    if (joined == cudaSuccess) joined = e;
   }
+  if (st == FPT_OK) CUDA_OR_FAIL(ctx, joined);
   return st;
 }
+}  // extern "C++"
 
 // Paths of order n and interaction-type pattern q: count and list (nullptr for exhaustive batches).
 static uint64_t pattern_slice(const fpt_batch* b, int n, unsigned q, const PathRec** list) {
